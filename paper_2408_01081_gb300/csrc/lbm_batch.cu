@@ -655,9 +655,7 @@ lbm_status lbm_batch_init(lbm_batch* b, int32_t index, const double* U0, const d
             dev[q] = stage + q * 5 * n;
         }
     }
-    dim3 grid, block;
-    node_grid_for((long long)n, grid, block);
-    cudaError_t e = b->ops->init(lattice_node_args(b, index), dev[0], dev[1], dev[2], nullptr, nullptr, grid, block, b->s);
+    cudaError_t e = b->ops->init(lattice_node_args(b, index), dev[0], dev[1], dev[2], nullptr, nullptr, b->s);
     if (stage) cudaFreeAsync(stage, b->s);
     if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch init: ") + cudaGetErrorString(e));
     if (!on_device) B_CUDA(b, cudaStreamSynchronize(b->s));

@@ -805,14 +805,12 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
     if ((st = stage_in(ctx, dU0dy, 5 * n, on_device, &dUy, &o3)) != LBM_OK) return st;
     if ((st = stage_in(ctx, B0, 2 * n, on_device, &dB0, &o4)) != LBM_OK) return st;
     if ((st = stage_in(ctx, ctx->w ? u0 : nullptr, 2 * n, on_device, &du0, &o5)) != LBM_OK) return st;
-    dim3 grid, block;
-    node_grid(ctx, grid, block);
     st = choose_neq_scale(ctx, [&](const lbmk::NodeArgs& M) {
-        return ctx->ops->init(M, dU0, dUx, dUy, dB0, du0, grid, block, ctx->s);
+        return ctx->ops->init(M, dU0, dUx, dUy, dB0, du0, ctx->s);
     });
     if (st != LBM_OK) return st;
     lbmk::NodeArgs A = node_args(ctx, -1);
-    cudaError_t e = ctx->ops->init(A, dU0, dUx, dUy, dB0, du0, grid, block, ctx->s);
+    cudaError_t e = ctx->ops->init(A, dU0, dUx, dUy, dB0, du0, ctx->s);
     for (double* o : {o1, o2, o3, o4, o5})
         if (o) cudaFreeAsync(o, ctx->s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "init kernel");

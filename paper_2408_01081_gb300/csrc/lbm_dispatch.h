@@ -57,7 +57,7 @@ struct KindOps {
     int state_bytes_per_node;      // bytes of one node in one state buffer
     cudaError_t (*step)(const lbmk::StepArgs&, int variant, dim3 grid, dim3 block, cudaStream_t s);
     cudaError_t (*init)(const lbmk::NodeArgs&, const double* U0, const double* Ux, const double* Uy,
-                        const double* B0, const double* u0, dim3 grid, dim3 block, cudaStream_t s);
+                        const double* B0, const double* u0, cudaStream_t s);
     cudaError_t (*moments)(const lbmk::NodeArgs&, double* out, dim3 grid, dim3 block, cudaStream_t s);
     cudaError_t (*get_pop)(const lbmk::NodeArgs&, double* f, double* ustar, dim3 grid, dim3 block, cudaStream_t s);
     cudaError_t (*set_pop)(const lbmk::NodeArgs&, const double* f, const double* ustar, dim3 grid, dim3 block,

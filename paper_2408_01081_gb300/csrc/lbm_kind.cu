@@ -3,6 +3,8 @@
 // or block-floating-point deviations).
 #include "lbm_dispatch.h"
 
+#include <algorithm>
+
 #ifndef LBM_KIND
 #error "LBM_KIND must be defined"
 #endif
@@ -146,8 +148,12 @@ cudaError_t step(const lbmk::StepArgs& a, int variant, dim3 g, dim3 b, cudaStrea
 }
 
 cudaError_t init(const lbmk::NodeArgs& a, const double* U0, const double* Ux, const double* Uy,
-                 const double* B0, const double* u0, dim3 g, dim3 b, cudaStream_t s)
+                 const double* B0, const double* u0, cudaStream_t s)
 {
+    // enough blocks for several per SM, then more rows per block: a thread's constants cost
+    // about as many FP64 operations as a tenth of a node
+    const int nbx = (a.nx + 127) / 128;
+    const dim3 b(128), g(nbx, std::min(a.ny, std::max(1, 152 * 48 / nbx)));
     if (B0) lbmk::init_kernel<K, true><<<g, b, 0, s>>>(a, U0, Ux, Uy, B0, u0);
     else lbmk::init_kernel<K, false><<<g, b, 0, s>>>(a, U0, Ux, Uy, B0, u0);
     return cudaGetLastError();
