@@ -762,6 +762,76 @@ __device__ __forceinline__ void uncollide_node(const double (&S)[4][5], double b
     }
 }
 
+// scaled fluxes phi_x(v) = Phi_x(v)/c, phi_y(v) = Phi_y(v)/c (Eq. system)
+__device__ __forceinline__ void phix(const double (&v)[5], double a, double b, double (&o)[5])
+{
+    o[0] = a * v[2] + b * v[3];
+    o[1] = b * v[4];
+    o[2] = a * v[0];
+    o[3] = b * v[0];
+    o[4] = b * v[1];
+}
+__device__ __forceinline__ void phiy(const double (&v)[5], double a, double b, double (&o)[5])
+{
+    o[0] = b * v[4];
+    o[1] = a * v[2] - b * v[3];
+    o[2] = a * v[1];
+    o[3] = -b * v[1];
+    o[4] = b * v[0];
+}
+
+// Eq. ic_second evaluated in the order it is written (scaled fluxes Phi/c), then the first
+// collision: S = f*, U its moments.  HASB: a body load is given.
+template <bool HASB>
+__device__ __forceinline__ void init_node_sequence(const NodeArgs& A, const double (&u)[5], const double (&ux)[5],
+                                                   const double (&uy)[5], const double (&bv)[5], double (&S)[4][5],
+                                                   double (&U)[5])
+{
+    const double a = A.a, b = A.b, c = A.c;
+    // Phi/c is linear, so px(px u_x) + px(py u_y) = px(px u_x + py u_y), likewise py
+    double pxu[5], pyu[5], pxb[5], pyb[5], pxx[5], pyy[5], sxy[5], pxs[5], pys[5];
+    phix(u, a, b, pxu);
+    phiy(u, a, b, pyu);
+    if (HASB) {
+        phix(bv, a, b, pxb);
+        phiy(bv, a, b, pyb);
+    }
+    phix(ux, a, b, pxx);
+    phiy(uy, a, b, pyy);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) sxy[k] = pxx[k] + pyy[k];
+    phix(sxy, a, b, pxs);
+    phiy(sxy, a, b, pys);
+    // per velocity (i, j), with the zero and unit factors of i, j written out:
+    //   f = 1/4 (u + 2 (i px u + j py u)) - dt/8 [ b + 2 (i px b + j py b)
+    //       + c (i u_x + (2 i^2 - 1) px u_x - 2 (i px + j py) px u_x)
+    //       + c (j u_y + (2 j^2 - 1) py u_y - 2 (i px + j py) py u_y) ]
+    // so for (+-1, 0): 1/4 u +- 1/2 px u - dt/8 [ b +- 2 px b + c (px u_x - py u_y)
+    //                  +- c (u_x - 2 px (px u_x + py u_y)) ], and (0, +-1) with x, y exchanged
+    double f[4][5];
+    const double h = 0.125 * A.dt;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const double qu = 0.25 * u[k];
+        const double sx = c * (pxx[k] - pyy[k]);                     // the y rows carry -sx
+        const double ex = 0.5 * pxu[k], ey = 0.5 * pyu[k];
+        const double dxp = c * fma(-2.0, pxs[k], ux[k]);
+        const double dyp = c * fma(-2.0, pys[k], uy[k]);
+        double gxp = sx + dxp, gxm = sx - dxp, gyp = dyp - sx, gym = -sx - dyp;
+        if (HASB) {
+            gxp += bv[k] + 2.0 * pxb[k];
+            gxm += bv[k] - 2.0 * pxb[k];
+            gyp += bv[k] + 2.0 * pyb[k];
+            gym += bv[k] - 2.0 * pyb[k];
+        }
+        f[0][k] = fma(-h, gxp, qu + ex);
+        f[2][k] = fma(-h, gxm, qu - ex);
+        f[1][k] = fma(-h, gyp, qu + ey);
+        f[3][k] = fma(-h, gym, qu - ey);
+    }
+    collide_node(f, bv[0], bv[1], A.dt, A.omega, a, b, S, U);
+}
+
 // Eq. ic_second (written with phi = Phi/c), then the first collision.  Inputs are dense
 // [5][ny][nx] (U0, dU0dx, dU0dy), [2][ny][nx] (B0, u0; may be null).  HASB: B0 is given.
 //
@@ -778,7 +848,75 @@ __device__ __forceinline__ void uncollide_node(const double (&S)[4][5], double b
 // memory: 22.4 ms before, 9.5 ms now, 2.8 ms of HBM traffic in FP64).  Other
 // omega build f (s = -1) and collide it.  Every operation is written as one rounding, so the
 // two instantiations agree bit for bit where b = 0.
-// Grid: blocks of columns x rows (strided), no division per node.
+template <bool HASB>
+__device__ __forceinline__ void init_node_fused(const NodeArgs& A, const double (&u)[5], const double (&ux)[5],
+                                                const double (&uy)[5], const double (&bv)[5], double (&f)[4][5])
+{
+    const double a = A.a, b = A.b;
+    const double s = (A.omega == 2.0) ? 1.0 : -1.0;
+    const double h = s * (0.125 * A.dt), e = h * A.c;
+    const double e4 = 4.0 * e, h4 = 4.0 * h, ha = 0.5 * a, hb = 0.5 * b;
+    // S and D: Phi_x = [cK js + cmu jd, cmu jxy, cK vx, cmu vx, cmu vy],
+    // Phi_y = [cmu jxy, cK js - cmu jd, cK vy, -cmu vy, cmu vx]
+    const double gx = fma(a, ux[2], __dmul_rn(b, ux[3])), gy = fma(a, uy[2], -__dmul_rn(b, uy[3]));
+    const double p = __dadd_rn(ux[0], uy[1]), m = __dadd_rn(ux[0], -uy[1]);
+    const double q = __dadd_rn(ux[1], uy[0]), r = __dadd_rn(ux[1], -uy[0]);
+    const double S[5] = {fma(b, uy[4], gx), fma(b, ux[4], gy), __dmul_rn(a, p), __dmul_rn(b, m), __dmul_rn(b, q)};
+    const double D[5] = {fma(-b, uy[4], gx), fma(b, ux[4], -gy), __dmul_rn(a, m), __dmul_rn(b, p),
+                         __dmul_rn(b, r)};
+    double w[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) w[k] = fma(-e4, S[k], u[k]);
+    if (HASB) {
+        w[0] = fma(h4, bv[0], w[0]);
+        w[1] = fma(h4, bv[1], w[1]);
+    }
+    const double a2 = __dmul_rn(ha, w[2]), b4 = __dmul_rn(hb, w[4]), b0 = __dmul_rn(hb, w[0]);
+    const double b1 = __dmul_rn(hb, w[1]);
+    const double px[5] = {fma(hb, w[3], a2), b4, __dmul_rn(ha, w[0]), b0, b1};
+    const double py[5] = {b4, fma(-hb, w[3], a2), __dmul_rn(ha, w[1]), -b1, b0};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        double qu = __dmul_rn(0.25, u[k]);
+        if (HASB && k < 2) qu = fma(h, bv[k], qu);
+        const double cx = fma(e, D[k], qu), cy = fma(-e, D[k], qu);
+        const double tx = fma(e, ux[k], px[k]), ty = fma(e, uy[k], py[k]);
+        f[0][k] = __dadd_rn(cx, tx);
+        f[2][k] = __dadd_rn(cx, -tx);
+        f[1][k] = __dadd_rn(cy, ty);
+        f[3][k] = __dadd_rn(cy, -ty);
+    }
+}
+
+// Whether the values of a node, as init_node_fused gives them, might round to another FP32 than
+// init_node_sequence's: the two differ by some units of 2^-52 of the node's largest value (the sums
+// and differences of each axis keep every intermediate within a few times that), so only a value
+// that close to the middle between two FP32 can.  64 of those units are allowed for.  Values below
+// FP32's normal range, or 2^20 times smaller than the largest, count as close.
+__device__ __forceinline__ bool init_rounding_open(const double (&f)[4][5])
+{
+    unsigned mx = 0;
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) mx = max(mx, (unsigned)__double2hiint(f[d][k]) & 0x7FFFFFFFu);
+    const unsigned emax = mx >> 20;
+    bool open = false;
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const unsigned e = ((unsigned)__double2hiint(f[d][k]) >> 20) & 0x7FFu;
+            const unsigned below = min(emax - e, 21u);
+            const unsigned tol = 64u << below;                       // below 2^28
+            const unsigned t = ((unsigned)__double2loint(f[d][k]) & 0x1FFFFFFFu) - 0x10000000u;
+            open |= t + tol <= 2u * tol || below > 20u || e < 897u;
+        }
+    return open;
+}
+
+// Grid: blocks of columns x rows (strided), no division per node.  U0, dU0dx, dU0dy: [5][ny][nx];
+// B0, u0: [2][ny][nx] (may be null).
 template <int K, bool HASB>
 __global__ void __launch_bounds__(128) init_kernel(NodeArgs A, const double* __restrict__ U0,
                                                    const double* __restrict__ Ux, const double* __restrict__ Uy,
@@ -787,13 +925,9 @@ __global__ void __launch_bounds__(128) init_kernel(NodeArgs A, const double* __r
     const long long n = (long long)A.nx * A.ny;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= A.nx) return;
-    const double a = A.a, b = A.b;
-    const double s = (A.omega == 2.0) ? 1.0 : -1.0;
-    const double h = s * (0.125 * A.dt), e = h * A.c;
-    const double e4 = 4.0 * e, h4 = 4.0 * h, ha = 0.5 * a, hb = 0.5 * b;
     for (int y = blockIdx.y; y < A.ny; y += gridDim.y) {
         const long long id = (long long)y * A.nx + x;
-        double u[5], ux[5], uy[5], bv[2] = {0.0, 0.0};
+        double u[5], ux[5], uy[5], bv[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
             u[k] = U0[k * n + id];
@@ -804,50 +938,43 @@ __global__ void __launch_bounds__(128) init_kernel(NodeArgs A, const double* __r
             bv[0] = B0[id];
             bv[1] = B0[n + id];
         }
-        // S and D: Phi_x = [cK js + cmu jd, cmu jxy, cK vx, cmu vx, cmu vy],
-        // Phi_y = [cmu jxy, cK js - cmu jd, cK vy, -cmu vy, cmu vx]
-        const double gx = fma(a, ux[2], __dmul_rn(b, ux[3])), gy = fma(a, uy[2], -__dmul_rn(b, uy[3]));
-        const double p = __dadd_rn(ux[0], uy[1]), m = __dadd_rn(ux[0], -uy[1]);
-        const double q = __dadd_rn(ux[1], uy[0]), r = __dadd_rn(ux[1], -uy[0]);
-        const double S[5] = {fma(b, uy[4], gx), fma(b, ux[4], gy), __dmul_rn(a, p), __dmul_rn(b, m), __dmul_rn(b, q)};
-        const double D[5] = {fma(-b, uy[4], gx), fma(b, ux[4], -gy), __dmul_rn(a, m), __dmul_rn(b, p),
-                             __dmul_rn(b, r)};
-        double w[5];
+        double S[4][5], U[5];
+        if constexpr (K == K_F64) {
+            init_node_fused<HASB>(A, u, ux, uy, bv, S);
+            if (A.omega != 2.0) {
+                double f[4][5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) w[k] = fma(-e4, S[k], u[k]);
-        if (HASB) {
-            w[0] = fma(h4, bv[0], w[0]);
-            w[1] = fma(h4, bv[1], w[1]);
-        }
-        const double a2 = __dmul_rn(ha, w[2]), b4 = __dmul_rn(hb, w[4]), b0 = __dmul_rn(hb, w[0]);
-        const double b1 = __dmul_rn(hb, w[1]);
-        const double px[5] = {fma(hb, w[3], a2), b4, __dmul_rn(ha, w[0]), b0, b1};
-        const double py[5] = {b4, fma(-hb, w[3], a2), __dmul_rn(ha, w[1]), -b1, b0};
-        double f[4][5];
+                for (int d = 0; d < 4; ++d)
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            double qu = __dmul_rn(0.25, u[k]);
-            if (HASB && k < 2) qu = fma(h, bv[k], qu);
-            const double cx = fma(e, D[k], qu), cy = fma(-e, D[k], qu);
-            const double tx = fma(e, ux[k], px[k]), ty = fma(e, uy[k], py[k]);
-            f[0][k] = __dadd_rn(cx, tx);
-            f[2][k] = __dadd_rn(cx, -tx);
-            f[1][k] = __dadd_rn(cy, ty);
-            f[3][k] = __dadd_rn(cy, -ty);
-        }
-        if (A.omega == 2.0) {
-            store_node<K>(A, x, y, f);
+                    for (int k = 0; k < 5; ++k) f[d][k] = S[d][k];
+                collide_node(f, bv[0], bv[1], A.dt, A.omega, A.a, A.b, S, U);
+            }
+#pragma unroll
+            for (int k = 0; k < 5; ++k) U[k] = u[k];
         } else {
-            double o[4][5], U[5];
-            collide_node(f, bv[0], bv[1], A.dt, A.omega, a, b, o, U);
-            store_node<K>(A, x, y, o);
+            // The reduced formats store the values of the written order, whose FP64 rounding differs
+            // from the fused form's: about five FP32 values of an 8192^2 lattice would turn, and the
+            // FP32 trajectories part by an ulp from there.  Nodes with a value close to a rounding
+            // boundary, about one in ten thousand, evaluate it in the written order.
+            bool seq = A.omega != 2.0;
+            if (!seq) {
+                init_node_fused<HASB>(A, u, ux, uy, bv, S);
+                seq = init_rounding_open(S);
+#pragma unroll
+                for (int k = 0; k < 5; ++k) U[k] = u[k];
+            }
+#ifdef LBM_INIT_ALWAYS_SEQ
+            seq = true;
+#endif
+            if (seq) init_node_sequence<HASB>(A, u, ux, uy, bv, S, U);
         }
+        store_node<K>(A, x, y, S);
         if (A.w) {
             // u*(dt) = u*(0) + dt v(0) with u*(0) = u0 - dt/2 v(0)  (Eq. trapezoidal)
             const long long off = (long long)(y + A.yo) * A.pitch + x;
             const double u0x = u0 ? u0[id] : 0.0, u0y = u0 ? u0[n + id] : 0.0;
-            A.w[off] = fma(0.5 * A.dt, u[0], u0x);
-            A.w[A.plane + off] = fma(0.5 * A.dt, u[1], u0y);
+            A.w[off] = u0x + 0.5 * A.dt * U[0];
+            A.w[A.plane + off] = u0y + 0.5 * A.dt * U[1];
         }
     }
 }
