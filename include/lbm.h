@@ -112,15 +112,21 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
  * run instead); a remainder of one or two steps runs as a single step or a pair.
  * rows_per_block sets the rows each thread block streams through (0 keeps the
  * format's default: 12 for LBM_F32, 64 for the other reduced formats; for the
- * staged LBM_F64 step of lbm_set_staging 4 at split level 12 and 2 at level 1).
+ * staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
+ * level 1, fewer on small lattices).  By default (this call not made, staging 1)
+ * the steps of one lbm_step call on a small LBM_F64 lattice at split level 12 (up to
+ * about 1800 segments of 32 columns of a row) run in one cooperative launch, with
+ * the same results; a bounded wait of it that runs out (about 2 s) makes the next
+ * lbm_synchronize return LBM_ERR_TIMEOUT.
  * steps_per_pass = 1 always uses one kernel per step. */
 lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t rows_per_block);
 
 /* How the multi-step kernels of lbm_set_step_fusion and the LBM_F64 step at split
- * level 1 read their input (no counterpart in the paper; results are identical
+ * levels 1 and 12 read their input (no counterpart in the paper; results are identical
  * either way).  1 (the default): each multi-step block's input rows are copied into
  * a ring of shared-memory stages by tensor copies (TMA) issued by one producer warp,
- * as far ahead as the ring allows; each thread of the FP64 step copies the 20
+ * as far ahead as the ring allows; each thread of the FP64 step (with a body load at
+ * split level 12) copies the 20
  * populations its node pulls into shared memory by asynchronous copies, one row
  * ahead of the row it computes.  0: each thread loads into registers (the two-step
  * kernel prefetches the next row there).  A bounded wait of the staged

@@ -210,6 +210,7 @@ struct lbm_ctx {
     double neq_scale = 1.0;      // moment-space storage: scale of the stored deviations
     int fuse = 1;                // steps per pass over memory when the fused kernel applies
     int tb_rows = 16;            // rows per block of the fused kernels and the staged FP64 step
+    bool one_step = false;       // one kernel per step asked for (lbm_set_step_fusion with 1)
     bool rows_set = false;       // tb_rows given by lbm_set_step_fusion (else the staged FP64 step's
                                  // rows per block follow its split level)
     int split = 1;               // FP64: split level (which additions run on the integer pipes; 12:
@@ -668,6 +669,7 @@ lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t row
     if (steps_per_pass < 1 || steps_per_pass > 3 || rows_per_block < 0 || rows_per_block > 65535)
         return fail(ctx, LBM_ERR_ARG, "steps_per_pass must be 1, 2 or 3 and rows_per_block in [0, 65535]");
     ctx->fuse = steps_per_pass;
+    ctx->one_step = steps_per_pass == 1;
     if (rows_per_block > 0) {
         ctx->tb_rows = rows_per_block;
         ctx->rows_set = true;
@@ -930,6 +932,24 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
             n -= 2;
         }
     }
+    // small FP64 lattices at the fixed-point level: the steps in one cooperative launch
+    if (split && ctx->split == lbmh::STEP_SPLIT_FIXED && ctx->staging == 1 && !ctx->slab && !ctx->one_step &&
+        !ctx->rows_set && n >= 2 && n <= (1 << 30)) {
+        const long long m = ctx->m;
+        A.src = ctx->buf[ctx->cur];
+        A.dst = ctx->buf[ctx->cur ^ 1];
+        A.T = ctx->R > 0 ? ctx->fT + (m + 1) * 2 * ctx->R : nullptr;
+        A.Tf = nullptr;
+        A.g = ctx->g ? ctx->g + m * 2 * ctx->nwall : nullptr;
+        cudaError_t e = ops->step_multi(A, variant, (int)n, reinterpret_cast<unsigned int*>(ctx->scratch),
+                                        kRedBlocks * 60, reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot), ctx->s);
+        if (e == cudaSuccess) {
+            ctx->cur ^= (int)(n & 1);
+            ctx->m = m + n;
+            return LBM_OK;
+        }
+        if (e != cudaErrorNotSupported) return cuda_fail(ctx, e, "multi-step FP64 kernel");
+    }
     for (int64_t i = 0; i < n; ++i) {
         const long long m = ctx->m;
         A.src = ctx->buf[ctx->cur];
@@ -940,8 +960,12 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
         // FP64 at split level 1: rows staged by asynchronous copies unless staging is off
         cudaError_t e = cudaErrorNotSupported;
         if (split && (ctx->split == 1 || ctx->split == lbmh::STEP_SPLIT_FIXED) && ctx->staging >= 1) {
-            // rows per block measured best at 8192^2: 2 at level 1, 4 for the fixed-point update
-            const int rows = ctx->rows_set ? ctx->tb_rows : (ctx->split == 1 ? 2 : 4);
+            // rows per block measured best at 8192^2: 2 at level 1, 4 for the fixed-point update.  Fewer
+            // where 4 would leave too few blocks (608 are resident): 512 x 256 8.5 us a step with 1 row,
+            // 16.1 with 4; 512 x 512 14.7 and 16.6; 1024 x 512 (4096 row segments) 32.3 and 29.1
+            const long long seg = (long long)((ctx->p.nx + lbmk::SA_THREADS - 1) / lbmk::SA_THREADS) * ctx->p.ny;
+            const int few = seg <= 2048 ? 1 : seg <= 3500 ? 2 : 4;
+            const int rows = ctx->rows_set ? ctx->tb_rows : std::min(few, ctx->split == 1 ? 2 : 4);
             e = ops->step_staged(A, variant, rows, ctx->s);
         }
         if (e == cudaErrorNotSupported) e = ops->step(A, variant, grid, block, ctx->s);

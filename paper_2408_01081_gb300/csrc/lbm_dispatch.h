@@ -50,6 +50,26 @@ constexpr int split_adds(int level)
     return n;
 }
 
+// Launch a kernel that begins with lbmt::grid_dependency_wait(): its blocks may become resident
+// while the previous kernel of the stream drains and run up to that wait, which returns once the
+// previous kernel has completed and its writes are visible.  Saves the launch gap between
+// dependent steps (a few hundred nanoseconds of each step on lattices that fill little of the chip).
+template <typename... P, typename... Q>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Q... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 struct KindOps {
     int kind;
     int vec;                       // nodes per thread in the step kernel
@@ -77,9 +97,15 @@ struct KindOps {
     cudaError_t (*tbt_step)(const CUtensorMap* maps, const lbmk::TbtArgs&, bool dirichlet, dim3 grid, cudaStream_t s);
     // three fused steps (maps with box width Tbt3Geom::WIN, or Tbt3MsGeom::WIN for moment space)
     cudaError_t (*tbt3_step)(const CUtensorMap* maps, const lbmk::TbtArgs&, bool dirichlet, dim3 grid, cudaStream_t s);
-    // one FP64 step at split level 1 or 12 with the rows staged by asynchronous copies, `rows`
-    // rows per block (other formats and variants return cudaErrorNotSupported)
+    // one FP64 step at split level 1, or 12 with or without a body load, with the rows staged by
+    // asynchronous copies, `rows` rows per block (other formats and variants return
+    // cudaErrorNotSupported)
     cudaError_t (*step_staged)(const lbmk::StepArgs&, int variant, int rows, cudaStream_t s);
+    // `steps` FP64 steps of a small lattice in one cooperative launch (split level 12; the variant's
+    // boundary, body load and tracking bits); flags: max_flags words of device scratch.
+    // cudaErrorNotSupported for other formats and for lattices that one launch per step serves better
+    cudaError_t (*step_multi)(const lbmk::StepArgs&, int variant, int steps, unsigned int* flags, int max_flags,
+                              int* timeout, cudaStream_t s);
     // three fused steps over the tiles of a batch (FP32 / BF16 / FP16; others return
     // cudaErrorNotSupported): `ntiles` blocks, all of periodic or all of Dirichlet lattices
     cudaError_t (*batch_tbt3_step)(const lbmk::BatchTbtArgs&, bool dirichlet, int ntiles, cudaStream_t s);

@@ -129,6 +129,28 @@ FX_HD u64 from_fixed(i64 y, int add)
     return ((u64)hi2 << 32) | (u64)(unsigned)d;
 }
 
+// the same value on the integer pipes alone (|y| < 2^63): normalise the magnitude, round its low 11
+// bits to nearest even and add exponent and sign; about 25 integer instructions against one
+// FP64-pipe conversion, which costs 16 cycles of a scheduler's FP64 pipe per warp.  Used for some
+// of a node's outputs where the FP64 pipe has other work (the body load) and is the longer one.
+FX_HD u64 from_fixed_int(i64 y, int add)
+{
+    const unsigned s = (unsigned)((u64)y >> 32) & 0x80000000u;
+    const u64 m = y < 0 ? 0ull - (u64)y : (u64)y;
+    if (m == 0) return 0ull;
+#ifdef __CUDA_ARCH__
+    const int n = __clzll((i64)m);
+#else
+    const int n = __builtin_clzll(m);
+#endif
+    const u64 z = m << n;                             // top bit set
+    const unsigned rem = (unsigned)z & 0x7FFu;
+    u64 q = z >> 11;                                  // 53 bits, the hidden one included
+    q += (rem + ((unsigned)q & 1u)) > 0x400u ? 1ull : 0ull;
+    // y = q 2^(11-n): exponent field 1086 - n, of which the hidden bit adds one
+    return q + ((u64)(unsigned)(((1085 - n) << 20) + add) << 32) + ((u64)s << 32);
+}
+
 // E of a node: the largest exponent field among its 20 inputs
 FX_HD int node_exp(const u64 (&in)[4][5])
 {
@@ -165,7 +187,9 @@ FX_HD bool exp_ok(int E) { return E >= 59 && E <= 2042; }
 // below 46 * 2^(E - 1023) (U below 10, the doubled outputs below 46 times that), inside the
 // 2^63 rho range, and each output is within half an ulp plus 13 rho of the exact update of
 // its inputs (five floors in U, three in a pair sum with h).
-template <bool HASH>
+// NI: how many of the 12 conversions of the (-1,0), (0,-1) outputs and of U's velocity components
+// run on the integer pipes (same bits).
+template <bool HASH, int NI = 0>
 FX_HD void fx_update_h(const u64 (&in)[4][5], const u64 (&h)[2], int E, const Mul& A, const Mul& B,
                        u64 (&out)[4][5], u64 (&Uout)[5])
 {
@@ -212,9 +236,11 @@ FX_HD void fx_update_h(const u64 (&in)[4][5], const u64 (&h)[2], int E, const Mu
         const i64 y1 = U[k] + T[1][k] + T[1][k];      // 2 f*(0,1)
         out[0][k] = from_fixed(y0, add2);
         out[1][k] = from_fixed(y1, add2);
-        out[2][k] = from_fixed(rx[k] + rx[k] - y0, add2);   // 2 f*(-1,0)
-        out[3][k] = from_fixed(ry[k] + ry[k] - y1, add2);   // 2 f*(0,-1)
-        Uout[k] = from_fixed(U[k], add2 + (1 << 20));       // U itself: scale rho
+        const i64 y2 = rx[k] + rx[k] - y0, y3 = ry[k] + ry[k] - y1;
+        out[2][k] = k < NI ? from_fixed_int(y2, add2) : from_fixed(y2, add2);           // 2 f*(-1,0)
+        out[3][k] = 5 + k < NI ? from_fixed_int(y3, add2) : from_fixed(y3, add2);       // 2 f*(0,-1)
+        // U itself: scale rho
+        Uout[k] = 10 + k < NI ? from_fixed_int(U[k], add2 + (1 << 20)) : from_fixed(U[k], add2 + (1 << 20));
     }
 }
 

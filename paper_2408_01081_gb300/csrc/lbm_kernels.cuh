@@ -287,11 +287,22 @@ __device__ __forceinline__ void collide_fixed(const double (&f)[4][5], double a,
     }
 }
 
-// The fixed-point node update with a body load (b_x, b_y at the node, hdt = dt/2): U of the two
-// velocity components gains h = hdt b (Eq. cond_eq).  Nodes outside the fixed-point range run
-// the FP64 sequence of step_kernel's body-load path (the body load folded into the pair sums
-// by fused multiply-adds, then the 47-operation collision).
-__device__ __forceinline__ void collide_fixed_forced(const double (&f)[4][5], double bx, double by, double hdt,
+// One term of the body load's coefficients: dt/2 b_c(x, y) = sum_r X[r][x] body_coef(r, c, y),
+// summed by fused multiply-adds in the order of r (the staged and the register kernel alike).
+// hdt = dt/2, T = [2][R] the row of the time.
+__device__ __forceinline__ double body_coef(const StepArgs& A, const double* T, double hdt, int r, int c, int y)
+{
+    return __dmul_rn(__dmul_rn(hdt, T[c * A.R + r]), A.Y[(long long)r * A.ny + y]);
+}
+
+#ifndef LBM_FX_FORCED_NI
+#define LBM_FX_FORCED_NI 5      // conversions of a node with body load on the integer pipes (0 .. 12)
+#endif
+
+// The fixed-point node update with a body load (hx, hy = dt/2 b at the node): U of the two
+// velocity components gains h (Eq. cond_eq).  Nodes outside the fixed-point range run the
+// FP64 sequence (the body load added to the pair sums, then the 47-operation collision).
+__device__ __forceinline__ void collide_fixed_forced(const double (&f)[4][5], double hx, double hy,
                                                      double a, double b, double (&U)[5], double (&o)[4][5])
 {
     const lbmfx::Mul A = lbmfx::make_mul(lbmemu::bits_of(a)), B = lbmfx::make_mul(lbmemu::bits_of(b));
@@ -300,11 +311,11 @@ __device__ __forceinline__ void collide_fixed_forced(const double (&f)[4][5], do
     for (int d = 0; d < 4; ++d)
 #pragma unroll
         for (int k = 0; k < 5; ++k) in[d][k] = lbmemu::bits_of(f[d][k]);
-    const lbmfx::u64 h[2] = {lbmemu::bits_of(hdt * bx), lbmemu::bits_of(hdt * by)};
+    const lbmfx::u64 h[2] = {lbmemu::bits_of(hx), lbmemu::bits_of(hy)};
     const int E = lbmfx::node_exp_h(in, h);
     const bool ok = lbmfx::exp_ok(E);
     if (__all_sync(0xffffffffu, ok)) {
-        lbmfx::fx_update_h<true>(in, h, E, A, B, out, Uo);
+        lbmfx::fx_update_h<true, LBM_FX_FORCED_NI>(in, h, E, A, B, out, Uo);
     } else {
         double rx[5], ry[5], U2[5], o2[4][5];
 #pragma unroll
@@ -312,10 +323,10 @@ __device__ __forceinline__ void collide_fixed_forced(const double (&f)[4][5], do
             rx[k] = f[1][k] + f[3][k];
             ry[k] = f[0][k] + f[2][k];
         }
-        rx[0] = fma(hdt, bx, rx[0]);
-        rx[1] = fma(hdt, by, rx[1]);
-        ry[0] = fma(hdt, bx, ry[0]);
-        ry[1] = fma(hdt, by, ry[1]);
+        rx[0] += hx;
+        rx[1] += hy;
+        ry[0] += hx;
+        ry[1] += hy;
         U2[0] = rx[0] + (f[0][0] + f[2][0]);
         U2[1] = rx[1] + (f[0][1] + f[2][1]);
 #pragma unroll
@@ -327,7 +338,7 @@ __device__ __forceinline__ void collide_fixed_forced(const double (&f)[4][5], do
 #pragma unroll
             for (int d = 0; d < 4; ++d) out[d][k] = lbmemu::bits_of(o2[d][k]);
         }
-        if (ok) lbmfx::fx_update_h<true>(in, h, E, A, B, out, Uo);
+        if (ok) lbmfx::fx_update_h<true, LBM_FX_FORCED_NI>(in, h, E, A, B, out, Uo);
     }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
@@ -535,16 +546,16 @@ step_kernel(StepArgs A)
         if constexpr (SPLIT > 0 && sizeof(M) == 8 && !FORCING && !OMEGA) {
             collide_split<SPLIT>(f, a, b, U, o);
         } else if constexpr ((SPLIT & kSplitFixed) != 0 && sizeof(M) == 8 && FORCING && !OMEGA) {
-            // body load in FP64 as below, then the fixed-point node update with it
-            double bx = 0.0, by = 0.0;
+            // dt/2 times the body load in FP64, then the fixed-point node update with it
+            double hx = 0.0, hy = 0.0;
             if (x < nx) {
                 for (int r = 0; r < A.R; ++r) {
-                    const double xy = A.X[(long long)r * nx + x] * A.Y[(long long)r * ny + y];
-                    bx = fma(xy, A.T[r], bx);
-                    by = fma(xy, A.T[A.R + r], by);
+                    const double X = A.X[(long long)r * nx + x];
+                    hx = fma(X, body_coef(A, A.T, 0.5 * A.dt, r, 0, y), hx);
+                    hy = fma(X, body_coef(A, A.T, 0.5 * A.dt, r, 1, y), hy);
                 }
             }
-            collide_fixed_forced(f, bx, by, 0.5 * A.dt, a, b, U, o);
+            collide_fixed_forced(f, hx, hy, a, b, U, o);
         } else {
 #pragma unroll
             for (int k = 0; k < 5; ++k) {

@@ -72,37 +72,106 @@ cudaError_t step_split(const lbmk::StepArgs& a, int level, dim3 g, dim3 b, cudaS
 #define LBM_SA_MASK lbmh::split_mask(1)   // the additions of split level 1 on the integer pipes
 #endif
 
-// FP64 at split level 1 or 12 with the rows staged by asynchronous copies (lbm_f64stage.cuh);
-// other formats, levels and variants return cudaErrorNotSupported
-template <bool D, bool T, unsigned long long M>
+// FP64 at split level 1 or 12 with the rows staged by asynchronous copies (lbm_f64stage.cuh),
+// a body load at level 12 only; other formats, levels and variants return cudaErrorNotSupported
+template <bool D, bool T, bool F, unsigned long long M>
 cudaError_t step_staged_dt(const lbmk::StepArgs& a, int rows, cudaStream_t s)
 {
     if constexpr (K != lbmk::K_F64) {
         return cudaErrorNotSupported;
     } else {
         const dim3 g((a.nx + lbmk::SA_THREADS - 1) / lbmk::SA_THREADS, (a.ny + rows - 1) / rows);
-        lbmk::step_f64_staged_kernel<D, T, M><<<g, lbmk::SA_THREADS, 0, s>>>(a, rows);
-        return cudaGetLastError();
+        return lbmh::launch_dependent(lbmk::step_f64_staged_kernel<D, T, F, M>, g, dim3(lbmk::SA_THREADS), 0, s, a, rows);
     }
 }
 
-template <unsigned long long M>
+template <bool F, unsigned long long M>
 cudaError_t step_staged_m(const lbmk::StepArgs& a, bool d, bool t, int rows, cudaStream_t s)
 {
-    return d ? (t ? step_staged_dt<true, true, M>(a, rows, s) : step_staged_dt<true, false, M>(a, rows, s))
-             : (t ? step_staged_dt<false, true, M>(a, rows, s) : step_staged_dt<false, false, M>(a, rows, s));
+    return d ? (t ? step_staged_dt<true, true, F, M>(a, rows, s) : step_staged_dt<true, false, F, M>(a, rows, s))
+             : (t ? step_staged_dt<false, true, F, M>(a, rows, s) : step_staged_dt<false, false, F, M>(a, rows, s));
 }
 
 // split levels 1 (LBM_SA_MASK) and 12 (fixed point)
 cudaError_t step_staged(const lbmk::StepArgs& a, int variant, int rows, cudaStream_t s)
 {
+    constexpr unsigned long long FX = lbmh::split_mask(lbmh::STEP_SPLIT_FIXED);
     const int level = (variant >> lbmh::STEP_SPLIT_SHIFT) & 15;
-    if ((level != 1 && level != lbmh::STEP_SPLIT_FIXED) || (variant & (lbmh::STEP_FORCING | lbmh::STEP_OMEGA)) ||
-        rows < 1)
+    const bool force = variant & lbmh::STEP_FORCING;
+    if ((level != 1 && level != lbmh::STEP_SPLIT_FIXED) || (variant & lbmh::STEP_OMEGA) ||
+        (force && level != lbmh::STEP_SPLIT_FIXED) || rows < 1)
         return cudaErrorNotSupported;
     const bool d = variant & lbmh::STEP_DIRICHLET, t = variant & lbmh::STEP_TRACK;
-    return level == 1 ? step_staged_m<LBM_SA_MASK>(a, d, t, rows, s)
-                      : step_staged_m<lbmh::split_mask(lbmh::STEP_SPLIT_FIXED)>(a, d, t, rows, s);
+    if (level == 1) return step_staged_m<false, LBM_SA_MASK>(a, d, t, rows, s);
+    return force ? step_staged_m<true, FX>(a, d, t, rows, s) : step_staged_m<false, FX>(a, d, t, rows, s);
+}
+
+// `steps` FP64 steps of a small lattice at split level 12 in one cooperative launch
+// (multi_f64_kernel); cudaErrorNotSupported where one launch per step is the better form
+template <bool D, bool T, bool F>
+cudaError_t step_multi_dtf(const lbmk::StepArgs& a, int steps, unsigned int* flags, int max_flags, int* timeout,
+                           cudaStream_t s)
+{
+    if constexpr (K != lbmk::K_F64) {
+        return cudaErrorNotSupported;
+    } else {
+        constexpr int W = lbmk::MULTI_WARPS;
+        lbmk::MultiArgs q;
+        q.A = a;
+        q.steps = steps;
+        q.nseg = (a.nx + 31) / 32;
+        const long long ntask = (long long)q.nseg * a.ny;
+        int dev = 0, sms = 0, occ = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lbmk::multi_f64_kernel<D, T, F>, 32 * W, 0);
+        if (e != cudaSuccess) return e;
+        // up to three blocks per SM: beyond that a launch per step is as fast (us per step, this
+        // kernel / launches: 64^2 3.3 / 5.0, 128^2 3.4 / 5.2, 256^2 5.9 / 5.6; with body load and
+        // tracking 4.1 / 5.1, 4.3 / 6.3, 6.6 / 6.6)
+        const long long cap = std::min((long long)std::min(occ, 3) * sms, (long long)max_flags / lbmk::MULTI_FLAG) * W;
+        if (cap < W || ntask > cap) return cudaErrorNotSupported;
+        q.ntask = (int)ntask;
+        q.nblk = (q.ntask + W - 1) / W;
+        // a node's sources lie within nseg segments of its own, cyclically; one block more for the
+        // shorter last block, one for the rounding
+        q.reach = std::min((q.nseg + W - 1) / W + 2, q.nblk - 1);
+        q.flags = flags;
+        q.timeout = timeout;
+        e = cudaMemsetAsync(flags, 0, (size_t)q.nblk * lbmk::MULTI_FLAG * sizeof(unsigned int), s);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(q.nblk);
+        cfg.blockDim = dim3(32 * W);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, lbmk::multi_f64_kernel<D, T, F>, q);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {       // part of the chip reserved for others
+            cudaGetLastError();
+            return cudaErrorNotSupported;
+        }
+        return e;
+    }
+}
+
+cudaError_t step_multi(const lbmk::StepArgs& a, int variant, int steps, unsigned int* flags, int max_flags,
+                       int* timeout, cudaStream_t s)
+{
+    switch (variant & 7) {
+    case 0: return step_multi_dtf<false, false, false>(a, steps, flags, max_flags, timeout, s);
+    case 1: return step_multi_dtf<true, false, false>(a, steps, flags, max_flags, timeout, s);
+    case 2: return step_multi_dtf<false, false, true>(a, steps, flags, max_flags, timeout, s);
+    case 3: return step_multi_dtf<true, false, true>(a, steps, flags, max_flags, timeout, s);
+    case 4: return step_multi_dtf<false, true, false>(a, steps, flags, max_flags, timeout, s);
+    case 5: return step_multi_dtf<true, true, false>(a, steps, flags, max_flags, timeout, s);
+    case 6: return step_multi_dtf<false, true, true>(a, steps, flags, max_flags, timeout, s);
+    default: return step_multi_dtf<true, true, true>(a, steps, flags, max_flags, timeout, s);
+    }
 }
 
 template <bool O>
@@ -347,7 +416,7 @@ namespace lbmh {
 const KindOps LBM_OPS_NAME(LBM_KIND) = {
     K, V, ELEM, NODE_BYTES,
     step, init, moments, get_pop, set_pop, energy, error, finite, batch_step, batch_occupancy, tb2_step, tbt_step,
-    tbt3_step, step_staged, batch_tbt3_step,
+    tbt3_step, step_staged, step_multi, batch_tbt3_step,
     LBM_VEC_SPLIT, VB,
 };
 

@@ -1,0 +1,59 @@
+"""Step kernels chosen by size, against the same steps taken one kernel at a time: several FP64
+steps in one launch on small lattices, and the FP64 step with a body load on staged rows against the
+register kernel.  All bit for bit."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _lattice(lbm, nx, ny, dirichlet, storage, load, nt=40, seed=0):
+    rng = np.random.default_rng(seed + nx + 1000 * ny)
+    lat = lbm.Lattice(nx, ny, 0.1, 0.1 / 3.2, 1.0, 0.6, dirichlet=dirichlet, storage=storage,
+                      track_displacement=load)
+    if load:
+        R = 3
+        lat.set_forcing(rng.standard_normal((R, nx)), rng.standard_normal((R, ny)),
+                        rng.standard_normal((nt, 2, R)) * 1e-3)
+        if dirichlet:
+            lat.set_dirichlet(rng.standard_normal((nt, 2, 2 * (nx + ny))) * 1e-3)
+    lat.set_populations(rng.standard_normal((4, 5, ny, nx)) * 1e-3, rng.standard_normal((2, ny, nx)) * 1e-3)
+    return lat
+
+
+def _state(lat):
+    lat.synchronize()
+    f, us = lat.populations()
+    lat.close()
+    return f, us
+
+
+# one segment of 32 columns per warp, four per block; the largest still takes one launch
+@pytest.mark.parametrize("load", [False, True])
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 7), (31, 4), (32, 3), (33, 65), (64, 64), (100, 300), (700, 40),
+                                   (2049, 2), (9000, 3)])
+def test_fp64_steps_in_one_launch_equal_single_launches(lbm, nx, ny, dirichlet, load):
+    many = _lattice(lbm, nx, ny, dirichlet, "f64", load)
+    many.step(2)
+    many.step(17)
+    one = _lattice(lbm, nx, ny, dirichlet, "f64", load)
+    for _ in range(19):
+        one.step(1)
+    a, b = _state(many), _state(one)
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("nx,ny,rows", [(2, 2, 1), (127, 5, 0), (129, 6, 4), (130, 9, 3), (1031, 7, 2), (260, 1300, 0)])
+def test_fp64_body_load_staged_equals_register_kernel(lbm, nx, ny, rows, dirichlet):
+    states = []
+    for staging in (1, 0):
+        lat = _lattice(lbm, nx, ny, dirichlet, "f64", True)
+        lat.set_staging(staging)
+        lat.set_step_fusion(1, rows)
+        lat.step(9)
+        states.append(_state(lat))
+    np.testing.assert_array_equal(states[0][0], states[1][0])
+    np.testing.assert_array_equal(states[0][1], states[1][1])
