@@ -99,8 +99,10 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out);
 lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const double* dU0dy,
                     const double* B0, const double* u0, int32_t on_device);
 
-/* Steps per pass over memory: 1, 2 or 3 (3 is the default for every format but
- * LBM_F64, whose step is bound by arithmetic, not memory).  With 2 lbm_step advances
+/* Steps per pass over memory: 1, 2 or 3.  Without this call LBM_F32 takes up to four
+ * steps per pass (results do not depend on the grouping), the other reduced formats
+ * three and LBM_F64, whose step is bound by arithmetic as well as by memory, one.
+ * With 2 lbm_step advances
  * pairs of steps with one kernel that keeps the intermediate state on chip (halving
  * the memory traffic per step), with 3 triples, whenever the lattice stores FP32 / BF16 / FP16
  * populations (or moment-space deviations, with staged rows: lbm_set_staging),
@@ -109,10 +111,11 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
  * step, one kernel per step runs.  FP32 results are bit-identical to single
  * steps; 16-bit and moment-space results skip one rounding per pair and are more
  * accurate.  Three steps per kernel need staged rows (lbm_set_staging 1; with 0 pairs
- * run instead); a remainder of one or two steps runs as a single step or a pair.
+ * run instead); a remainder of one or two steps runs as a single step or a pair
+ * (LBM_F32: passes of equal length instead).
  * rows_per_block sets the rows each thread block streams through (0 keeps the
- * format's default: 12 for LBM_F32, 64 for the other reduced formats; for the
- * staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
+ * default: for the population formats from the lattice's size, 2 to 96; 64 for moment
+ * space; for the staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
  * level 1, fewer on small lattices).  By default (this call not made, staging 1)
  * the steps of one lbm_step call on a small LBM_F64 lattice at split level 12 (up to
  * about 1800 segments of 32 columns of a row) run in one cooperative launch, with
@@ -362,12 +365,14 @@ lbm_status lbm_batch_tune(lbm_batch* b, const char* cache_path);
 
 /* Launch mode: 0 = one launch per step; 1 = one persistent launch per
  * `graph_steps` steps with a grid barrier between steps (cooperative launch);
- * 2 = three steps per pass (FP32 / BF16 / FP16 storage only, LBM_ERR_ARG otherwise):
- * every lattice is cut into tiles of 112 columns and 12 (FP32) or 64 (16-bit) rows,
+ * 2 = several steps per pass, up to four in FP32 and three in BF16 / FP16 (these
+ * storages only, LBM_ERR_ARG otherwise): every lattice is cut into tiles of 168 (FP32)
+ * or 240 (16-bit) columns and 2 to 96 rows (from the batch's sizes),
  * one block per tile stages the tile's input rows with tensor copies and keeps the
- * two intermediate steps on chip (the single-lattice three-step kernel of
+ * intermediate steps on chip (the single-lattice multi-step kernel of
  * lbm_set_step_fusion), one launch for the periodic and one for the Dirichlet
- * tiles per pass; steps beyond a multiple of three run as mode 0;
+ * tiles per pass; FP32 steps are grouped into passes of equal length, 16-bit steps
+ * beyond a multiple of three run as mode 0;
  * 3 = one step per launch on staged rows (FP64 storage only, LBM_ERR_ARG otherwise):
  * tiles of 128 columns and 4 rows (2 for a lattice on the level-1 sequence), one
  * block per tile copying each node's 20 inputs into shared memory one row ahead

@@ -112,7 +112,7 @@ struct lbm_batch {
     bool t3_ok = false;                   // row maps encoded and tile lists built
     int t3_rows = 0;                      // output rows per tile
     lbmk::BatchLatT3* d_lat3 = nullptr;
-    CUtensorMap* d_maps = nullptr;        // [lattice][arena]
+    CUtensorMap* d_maps = nullptr;        // [lattice][arena][2]: row map, wrap map
     int4* d_t3 = nullptr;                 // periodic tiles, then Dirichlet tiles
     int nt3[2] = {0, 0};                  // tile counts: periodic, Dirichlet
     // mode 3: FP64 on staged rows, one step per launch (lbm_batch_f64.cu)
@@ -183,30 +183,35 @@ lbm_status build_tiles(lbm_batch* b)
     return LBM_OK;
 }
 
-#ifndef LBM_BATCH_T3_ROWS4
-#define LBM_BATCH_T3_ROWS4 12     // output rows per mode-2 tile, FP32 (the single-lattice default)
-#endif
-#ifndef LBM_BATCH_T3_ROWS2
-#define LBM_BATCH_T3_ROWS2 64     // the same for BF16 / FP16
-#endif
-
-// Row maps (box width Tbt3Geom::WIN, both arenas) and tile lists of mode 2, for the
+// Row and wrap maps (box widths TbpGeom::WIN and ::WRAP, both arenas) and tile lists of mode 2, for the
 // population formats FP32 / BF16 / FP16 and lattices of at least 2 x 2 nodes; leaves
 // t3_ok false (mode 2 unavailable) where a map cannot be encoded
 lbm_status setup_t3(lbm_batch* b)
 {
     if (b->storage != LBM_F32 && b->storage != LBM_BF16 && b->storage != LBM_F16) return LBM_OK;
     const int es = b->ops->elem_bytes;
-    const int win = es == 4 ? lbmk::Tbt3Geom<4>::WIN : lbmk::Tbt3Geom<2>::WIN;
-    b->t3_rows = es == 4 ? LBM_BATCH_T3_ROWS4 : LBM_BATCH_T3_ROWS2;
-    std::vector<CUtensorMap> maps((size_t)2 * b->count);
+    const int win = es == 4 ? lbmk::TbpGeom<4>::WIN : lbmk::TbpGeom<2>::WIN;
+    const int wrap = es == 4 ? lbmk::TbpGeom<4>::WRAP : lbmk::TbpGeom<2>::WRAP;
+    const int out = es == 4 ? lbmk::TbpGeom<4>::OUT : lbmk::TbpGeom<2>::OUT;
+    // rows per tile: the rule of single lattices over all tiles (two launches of about half each)
+    const int resident = 152 * (es == 4 ? lbmk::TbpGeom<4>::MIN_BLOCKS : lbmk::TbpGeom<2>::MIN_BLOCKS);
+    int ny_max = 0;
+    for (const lbmk::LatDesc& L : b->lat) ny_max = std::max(ny_max, L.ny);
+    b->t3_rows = lbmk::tbp_rows(resident, ny_max, [&](int r) {
+        long long n = 0;
+        for (const lbmk::LatDesc& L : b->lat) n += (long long)((L.nx + out - 1) / out) * ((L.ny + r - 1) / r);
+        return n;
+    });
+    std::vector<CUtensorMap> maps((size_t)4 * b->count);
     std::vector<lbmk::BatchLatT3> l3((size_t)b->count);
     std::vector<int4> tiles[2];
     for (int i = 0; i < b->count; ++i) {
         const lbmk::LatDesc& L = b->lat[i];
         for (int a = 0; a < 2; ++a) {
             void* base = static_cast<char*>(b->arena[a]) + (size_t)L.off * es;
-            if (!lbmh::encode_rows_map(&maps[(size_t)2 * i + a], base, es, L.nx, L.ny, L.pitch, L.plane, 20, win))
+            CUtensorMap* m = &maps[(size_t)4 * i + 2 * a];
+            if (!lbmh::encode_rows_map(m, base, es, L.nx, L.ny, L.pitch, L.plane, 20, win) ||
+                !lbmh::encode_rows_map(m + 1, base, es, L.nx, L.ny, L.pitch, L.plane, 20, wrap))
                 return LBM_OK;
         }
         lbmk::BatchLatT3& q = l3[i];
@@ -219,7 +224,7 @@ lbm_status setup_t3(lbm_batch* b)
         q.bf = (float)L.b;
         q.pad_ = 0;
         for (int y = 0; y < L.ny; y += b->t3_rows)
-            for (int x = 0; x < L.nx; x += lbmk::TBT3_OUT) tiles[L.bc ? 1 : 0].push_back(make_int4(i, x, y, 0));
+            for (int x = 0; x < L.nx; x += out) tiles[L.bc ? 1 : 0].push_back(make_int4(i, x, y, 0));
     }
     b->nt3[0] = (int)tiles[0].size();
     b->nt3[1] = (int)tiles[1].size();
@@ -293,14 +298,33 @@ lbmk::BatchArgs batch_args(const lbm_batch* b, int steps, int parity)
     return A;
 }
 
-// arena swaps of `steps` steps: one per launch (a three-step pass of mode 2 is one launch pair)
-int swaps_of(const lbm_batch* b, long long steps)
+// Mode 2: launch pairs (one arena swap each) that make `steps` steps.  FP32 results do not depend
+// on how the steps are grouped: the fewest passes, of equal length, one more where the number of
+// swaps has to be even (a graph).  The 16-bit formats round once per pass: passes of three steps,
+// then single steps (an even number of swaps exactly when `steps` is even).
+long long mode2_passes(const lbm_batch* b, long long steps, bool even)
 {
-    return (int)((b->mode == 2 ? steps / 3 + steps % 3 : steps) & 1);
+    if (b->storage != LBM_F32) return steps / 3 + steps % 3;
+    const long long count = (steps + lbmk::TbpGeom<4>::NLMAX - 1) / lbmk::TbpGeom<4>::NLMAX;
+    return even && (count & 1) ? count + 1 : count;
 }
 
-// enqueue `steps` steps starting from arena `parity` (no graph)
-cudaError_t enqueue_steps(lbm_batch* b, int steps, int parity)
+// steps of pass p of `count`
+int mode2_pass(const lbm_batch* b, long long steps, long long count, long long p)
+{
+    if (b->storage != LBM_F32) return p < steps / 3 ? 3 : 1;
+    return lbmk::tbp_pass(steps, count, p);
+}
+
+// arena swaps of `steps` steps outside a graph: one per launch or launch pair
+int swaps_of(const lbm_batch* b, long long steps)
+{
+    return (int)((b->mode == 2 ? mode2_passes(b, steps, false) : steps) & 1);
+}
+
+// enqueue `steps` steps starting from arena `parity`; even: with an even number of arena swaps
+// (steps even)
+cudaError_t enqueue_steps(lbm_batch* b, int steps, int parity, bool even)
 {
     if (b->mode == 1) {
         return b->ops->batch_step(batch_args(b, steps, parity), true, b->persistent_grid, b->s);
@@ -326,23 +350,27 @@ cudaError_t enqueue_steps(lbm_batch* b, int steps, int parity)
     }
     int i = 0;
     if (b->mode == 2) {
-        // three steps per pass: the periodic tiles and the Dirichlet tiles, one launch each
-        lbmk::BatchTbtArgs T;
+        // several steps per pass: the periodic tiles and the Dirichlet tiles, one launch each
+        lbmk::BatchTbpArgs T;
         T.lat = b->d_lat3;
         T.maps = b->d_maps;
         T.arenaA = b->arena[0];
         T.arenaB = b->arena[1];
         T.rows = b->t3_rows;
         T.timeout = reinterpret_cast<int*>(b->d_bar + 2);
-        for (; i + 3 <= steps; i += 3) {
+        const long long count = mode2_passes(b, steps, even);
+        for (long long p = 0; p < count; ++p) {
+            const int k = mode2_pass(b, steps, count, p);
+            if (k < 2) break;                  // single steps: below
             T.parity = parity;
             T.tiles = b->d_t3;
-            cudaError_t e = b->ops->batch_tbt3_step(T, false, b->nt3[0], b->s);
+            cudaError_t e = b->ops->batch_tbp_step(T, k, false, b->nt3[0], b->s);
             if (e != cudaSuccess) return e;
             T.tiles = b->d_t3 + b->nt3[0];
-            e = b->ops->batch_tbt3_step(T, true, b->nt3[1], b->s);
+            e = b->ops->batch_tbp_step(T, k, true, b->nt3[1], b->s);
             if (e != cudaSuccess) return e;
             parity ^= 1;
+            i += k;
         }
     }
     for (; i < steps; ++i) {
@@ -358,7 +386,7 @@ lbm_status ensure_graph(lbm_batch* b)
     if (b->graph_valid) return LBM_OK;
     cudaGraph_t g = nullptr;
     B_CUDA(b, cudaStreamBeginCapture(b->s, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = enqueue_steps(b, b->graph_steps, 0);
+    cudaError_t e = enqueue_steps(b, b->graph_steps, 0, true);
     cudaError_t e2 = cudaStreamEndCapture(b->s, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -388,9 +416,12 @@ lbm_status run_steps(lbm_batch* b, long long n)
             n -= b->graph_steps;           // an even number of swaps: the state returns to arena 0
             continue;
         }
-        const int k = (int)std::min<long long>(n, b->cur == 0 ? (n % b->graph_steps) : 1);
+        // a graph starts from arena 0; the grouping of steps into passes matters to the 16-bit formats only
+        const bool free_split = b->storage == LBM_F32 || b->storage == LBM_F64;
+        const int k = (int)std::min<long long>(n, b->cur == 0 ? (n % b->graph_steps)
+                                                              : (free_split && n < b->graph_steps ? n : 1));
         const int kk = std::max(1, k);
-        B_CUDA(b, enqueue_steps(b, kk, b->cur));
+        B_CUDA(b, enqueue_steps(b, kk, b->cur, false));
         b->cur = (b->cur + swaps_of(b, kk)) & 1;
         n -= kk;
     }

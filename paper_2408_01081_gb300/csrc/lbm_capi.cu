@@ -210,6 +210,7 @@ struct lbm_ctx {
     double neq_scale = 1.0;      // moment-space storage: scale of the stored deviations
     int fuse = 1;                // steps per pass over memory when the fused kernel applies
     int tb_rows = 16;            // rows per block of the fused kernels and the staged FP64 step
+    int tbp_rows = 16;           // rows per block of the multi-step population kernels unless rows_set
     bool one_step = false;       // one kernel per step asked for (lbm_set_step_fusion with 1)
     bool rows_set = false;       // tb_rows given by lbm_set_step_fusion (else the staged FP64 step's
                                  // rows per block follow its split level)
@@ -226,9 +227,10 @@ struct lbm_ctx {
     bool slab = false;           // a row slab of a larger lattice (lbm_create_slab)
     int halo_lo = 0, halo_hi = 0;  // halo rows below / above the slab's own rows (0 or 1)
     bool maps_ok = false;        // row maps of both buffers encoded (all formats but FP64)
-    CUtensorMap map[2][2];       // row maps of buf[0], buf[1] for the staged fused kernel
-                                 // ([buffer][part]; moment space: FP32 part, 16-bit part)
-    CUtensorMap map3[2][2];      // row maps of the three-step kernels (narrower box)
+    CUtensorMap map[2][2];       // row maps of buf[0], buf[1] for the staged fused kernels
+                                 // ([buffer][part]; moment space: FP32 part, 16-bit part;
+                                 // populations: row map, wrap map)
+    CUtensorMap map3[2][2];      // moment space: row maps of the three-step kernel (narrower box)
 };
 
 namespace {
@@ -449,7 +451,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out)
     // three steps per pass for every reduced format (measured faster than one or two steps for each
     // of them at 8192^2, and fewer roundings to the storage format); rows per block measured best
     // per format
-    ctx->fuse = (p->storage == LBM_F64) ? 1 : 3;
+    ctx->fuse = (p->storage == LBM_F64) ? 1 : (p->storage == LBM_F32) ? lbmk::TbpGeom<4>::NLMAX : 3;
     ctx->tb_rows = (p->storage == LBM_F64) ? 2 : (p->storage == LBM_F32) ? 12 : 64;
     // FP64: the fixed-point node update by default (within FP64 accuracy, bound by memory
     // instead of the FP64 pipe); the exact integer-pipe sums where its multipliers do not fit
@@ -484,15 +486,20 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out)
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->s);
     if (e == cudaSuccess && (p->storage == LBM_F32 || p->storage == LBM_BF16 || p->storage == LBM_F16)) {
         const int es = ctx->ops->elem_bytes;
-        const int win = es == 4 ? lbmk::TbtGeom<4>::WIN : lbmk::TbtGeom<2>::WIN;
-        const int win3 = es == 4 ? lbmk::Tbt3Geom<4>::WIN : lbmk::Tbt3Geom<2>::WIN;
+        const int win = es == 4 ? lbmk::TbpGeom<4>::WIN : lbmk::TbpGeom<2>::WIN;
+        const int wrap = es == 4 ? lbmk::TbpGeom<4>::WRAP : lbmk::TbpGeom<2>::WRAP;
+        const int out = es == 4 ? lbmk::TbpGeom<4>::OUT : lbmk::TbpGeom<2>::OUT;
+        const int resident = 152 * (es == 4 ? lbmk::TbpGeom<4>::MIN_BLOCKS : lbmk::TbpGeom<2>::MIN_BLOCKS);
+        ctx->tbp_rows = lbmk::tbp_rows(resident, p->ny, [&](int r) {
+            return (long long)((p->nx + out - 1) / out) * ((p->ny + r - 1) / r);
+        });
         ctx->maps_ok = true;
         for (int i = 0; i < 2; ++i)
             ctx->maps_ok = ctx->maps_ok &&
                            encode_rows_map(&ctx->map[i][0], ctx->buf[i], es, p->nx, p->ny, ctx->pitch, ctx->plane, 20,
                                            win) &&
-                           encode_rows_map(&ctx->map3[i][0], ctx->buf[i], es, p->nx, p->ny, ctx->pitch, ctx->plane, 20,
-                                           win3);
+                           encode_rows_map(&ctx->map[i][1], ctx->buf[i], es, p->nx, p->ny, ctx->pitch, ctx->plane, 20,
+                                           wrap);
     }
     if (e == cudaSuccess && (p->storage == LBM_MS_BF16 || p->storage == LBM_MS_F16 || p->storage == LBM_MS_BFP)) {
         const int win = lbmk::TbtMsGeom::WIN;
@@ -883,6 +890,44 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
         const dim3 tblock(128), tgrid((nstrip + 3) / 4, (ctx->p.ny + T.rows - 1) / T.rows);
         if (ctx->staging >= 1) {
             if (!ctx->maps_ok) return fail(ctx, LBM_ERR_CUDA, "tensor maps of the state buffers could not be encoded");
+            if (!ms) {
+                lbmk::TbpArgs P;
+                P.nx = ctx->p.nx;
+                P.ny = ctx->p.ny;
+                P.pitch = ctx->pitch;
+                P.plane = ctx->plane;
+                P.af = (float)ctx->a;
+                P.bf = (float)ctx->b;
+                P.rows = ctx->rows_set ? ctx->tb_rows : ctx->tbp_rows;
+                P.timeout = reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot);
+                P.withhold = ctx->staging == 2 ? 2 : -1;
+                auto pass = [&](int k) {
+                    P.src = ctx->buf[ctx->cur];
+                    P.dst = ctx->buf[ctx->cur ^ 1];
+                    cudaError_t e = ops->tbp_step(ctx->map[ctx->cur], P, k, ctx->p.bc == LBM_DIRICHLET, ctx->s);
+                    if (e != cudaSuccess) return cuda_fail(ctx, e, "staged multi-step kernel");
+                    ctx->cur ^= 1;
+                    ctx->m += k;
+                    return LBM_OK;
+                };
+                lbm_status st;
+                if (ctx->p.storage == LBM_F32 && n >= 2) {
+                    // the fewest passes, of equal length; FP32 results do not depend on the split
+                    const long long count = (n + ctx->fuse - 1) / ctx->fuse, total = n;
+                    for (long long i = 0; i < count; ++i) {
+                        const int k = lbmk::tbp_pass(total, count, i);
+                        if (k < 2) break;                      // a single step: below
+                        if ((st = pass(k)) != LBM_OK) return st;
+                        n -= k;
+                    }
+                }
+                // the 16-bit formats round once per pass: whole passes, then the remainder
+                while (ctx->p.storage != LBM_F32 && n >= 2) {
+                    const int k = (int)std::min<long long>(n, ctx->fuse);
+                    if ((st = pass(k)) != LBM_OK) return st;
+                    n -= k;
+                }
+            }
             lbmk::TbtArgs Q;
             Q.nx = ctx->p.nx;
             Q.ny = ctx->p.ny;
@@ -897,7 +942,7 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
             Q.scale = (float)ctx->neq_scale;
             Q.inv_s = (float)(1.0 / ctx->neq_scale);
             Q.sat = reinterpret_cast<int*>(ctx->scratch + kSatSlot);
-            if (ctx->fuse == 3) {
+            if (ms && ctx->fuse == 3) {
                 // three steps per pass: the remainder below runs as one pair or a single step
                 const dim3 q3grid((ctx->p.nx + lbmk::TBT3_OUT - 1) / lbmk::TBT3_OUT, (ctx->p.ny + Q.rows - 1) / Q.rows);
                 while (n >= 3) {
@@ -911,7 +956,7 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
                 }
             }
             const dim3 qgrid((ctx->p.nx + lbmk::TBT_OUT - 1) / lbmk::TBT_OUT, (ctx->p.ny + Q.rows - 1) / Q.rows);
-            while (n >= 2) {
+            while (ms && n >= 2) {
                 Q.src = ctx->buf[ctx->cur];
                 Q.dst = ctx->buf[ctx->cur ^ 1];
                 cudaError_t e = ops->tbt_step(ctx->map[ctx->cur], Q, ctx->p.bc == LBM_DIRICHLET, qgrid, ctx->s);

@@ -10,6 +10,7 @@
 #include "lbm_kernels.cuh"
 #include "lbm_ms.cuh"
 #include "lbm_tb.cuh"
+#include "lbm_tbp.cuh"
 #include "lbm_tbt.cuh"
 
 namespace lbmh {
@@ -91,12 +92,14 @@ struct KindOps {
     cudaError_t (*batch_occupancy)(int* blocks_per_sm);
     // two fused steps (FP32 / BF16 / FP16 populations only; others return cudaErrorNotSupported)
     cudaError_t (*tb2_step)(const lbmk::TbArgs&, bool dirichlet, dim3 grid, dim3 block, cudaStream_t s);
-    // two fused steps with the input rows staged by tensor copies (FP32 / BF16 / FP16 populations
-    // and the moment-space formats); maps: the row maps of the source buffer, one for the
-    // population formats (box {TbtGeom::WIN, 1, 20}), two for moment space (FP32 part, 16-bit part)
+    // two and three fused steps of the moment-space formats with the input rows staged by tensor
+    // copies; maps: the row maps of the source buffer's FP32 and 16-bit parts (box width
+    // TbtMsGeom::WIN, Tbt3MsGeom::WIN); other formats return cudaErrorNotSupported
     cudaError_t (*tbt_step)(const CUtensorMap* maps, const lbmk::TbtArgs&, bool dirichlet, dim3 grid, cudaStream_t s);
-    // three fused steps (maps with box width Tbt3Geom::WIN, or Tbt3MsGeom::WIN for moment space)
     cudaError_t (*tbt3_step)(const CUtensorMap* maps, const lbmk::TbtArgs&, bool dirichlet, dim3 grid, cudaStream_t s);
+    // two or three fused steps of the FP32 / BF16 / FP16 populations in the same manner; maps: the
+    // row map and the wrap map of the source buffer (20 planes, box widths TbpGeom::WIN and ::WRAP)
+    cudaError_t (*tbp_step)(const CUtensorMap* maps, const lbmk::TbpArgs&, int steps, bool dirichlet, cudaStream_t s);
     // one FP64 step at split level 1, or 12 with or without a body load, with the rows staged by
     // asynchronous copies, `rows` rows per block (other formats and variants return
     // cudaErrorNotSupported)
@@ -108,7 +111,7 @@ struct KindOps {
                               int* timeout, cudaStream_t s);
     // three fused steps over the tiles of a batch (FP32 / BF16 / FP16; others return
     // cudaErrorNotSupported): `ntiles` blocks, all of periodic or all of Dirichlet lattices
-    cudaError_t (*batch_tbt3_step)(const lbmk::BatchTbtArgs&, bool dirichlet, int ntiles, cudaStream_t s);
+    cudaError_t (*batch_tbp_step)(const lbmk::BatchTbpArgs&, int steps, bool dirichlet, int ntiles, cudaStream_t s);
     int vec_split;                 // nodes per thread of the FP64 split-level step kernels
     int batch_vec;                 // nodes per thread of the batch kernel
 };

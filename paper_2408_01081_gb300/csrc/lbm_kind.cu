@@ -323,17 +323,43 @@ cudaError_t tb2_step(const lbmk::TbArgs& a, bool dirichlet, dim3 g, dim3 b, cuda
     return tb2_t<K>(a, dirichlet, g, b, s);
 }
 
+// 2 .. TbpGeom::NLMAX fused steps of the population formats (lbm_tbp.cuh)
+template <int KK, int NL>
+cudaError_t tbp_nl(const CUtensorMap* maps, const lbmk::TbpArgs& a, bool dirichlet, cudaStream_t s)
+{
+    using G = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>;
+    void (*kern)(CUtensorMap, CUtensorMap, lbmk::TbpArgs) =
+        dirichlet ? lbmk::tbp_kernel<KK, NL, true> : lbmk::tbp_kernel<KK, NL, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+    if (e != cudaSuccess) return e;
+    const dim3 g((a.nx + G::OUT - 1) / G::OUT, (a.ny + a.rows - 1) / a.rows);
+    return lbmh::launch_dependent(kern, g, dim3(G::THREADS), G::SMEM, s, maps[0], maps[1], a);
+}
+
+template <int KK>
+cudaError_t tbp_t(const CUtensorMap* maps, const lbmk::TbpArgs& a, int steps, bool dirichlet, cudaStream_t s)
+{
+    if constexpr (KK == lbmk::K_F32 || KK == lbmk::K_BF16 || KK == lbmk::K_F16) {
+        constexpr int MX = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>::NLMAX;
+        switch (steps) {
+        case 2: return tbp_nl<KK, 2>(maps, a, dirichlet, s);
+        case 3: return tbp_nl<KK, 3>(maps, a, dirichlet, s);
+        case 4: if constexpr (MX >= 4) return tbp_nl<KK, 4>(maps, a, dirichlet, s); break;
+        case 5: if constexpr (MX >= 5) return tbp_nl<KK, 5>(maps, a, dirichlet, s); break;
+        }
+    }
+    return cudaErrorNotSupported;
+}
+
+cudaError_t tbp_step(const CUtensorMap* maps, const lbmk::TbpArgs& a, int steps, bool dirichlet, cudaStream_t s)
+{
+    return tbp_t<K>(maps, a, steps, dirichlet, s);
+}
+
 template <int KK>
 cudaError_t tbt_t(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool dirichlet, dim3 g, cudaStream_t s)
 {
-    if constexpr (KK == lbmk::K_F32 || KK == lbmk::K_BF16 || KK == lbmk::K_F16) {
-        using G = lbmk::TbtGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>;
-        void (*kern)(CUtensorMap, lbmk::TbtArgs) = dirichlet ? lbmk::tbt_kernel<KK, true> : lbmk::tbt_kernel<KK, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-        if (e != cudaSuccess) return e;
-        kern<<<g, lbmk::TBT_THREADS, G::SMEM, s>>>(maps[0], a);
-        return cudaGetLastError();
-    } else if constexpr (KK == lbmk::K_MSBF16 || KK == lbmk::K_MSF16 || KK == lbmk::K_MSBFP) {
+    if constexpr (KK == lbmk::K_MSBF16 || KK == lbmk::K_MSF16 || KK == lbmk::K_MSBFP) {
         using G = lbmk::TbtMsGeom;
         void (*kern)(CUtensorMap, CUtensorMap, lbmk::TbtArgs) =
             dirichlet ? lbmk::tbt_ms_kernel<KK, true> : lbmk::tbt_ms_kernel<KK, false>;
@@ -354,14 +380,7 @@ cudaError_t tbt_step(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool diric
 template <int KK>
 cudaError_t tbt3_t(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool dirichlet, dim3 g, cudaStream_t s)
 {
-    if constexpr (KK == lbmk::K_F32 || KK == lbmk::K_BF16 || KK == lbmk::K_F16) {
-        using G = lbmk::Tbt3Geom<(int)sizeof(typename lbmk::Fmt<KK>::E)>;
-        void (*kern)(CUtensorMap, lbmk::TbtArgs) = dirichlet ? lbmk::tbt3_kernel<KK, true> : lbmk::tbt3_kernel<KK, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-        if (e != cudaSuccess) return e;
-        kern<<<g, lbmk::TBT_THREADS, G::SMEM, s>>>(maps[0], a);
-        return cudaGetLastError();
-    } else if constexpr (KK == lbmk::K_MSBF16 || KK == lbmk::K_MSF16 || KK == lbmk::K_MSBFP) {
+    if constexpr (KK == lbmk::K_MSBF16 || KK == lbmk::K_MSF16 || KK == lbmk::K_MSBFP) {
         using G = lbmk::Tbt3MsGeom;
         void (*kern)(CUtensorMap, CUtensorMap, lbmk::TbtArgs) =
             dirichlet ? lbmk::tbt3_ms_kernel<KK, true> : lbmk::tbt3_ms_kernel<KK, false>;
@@ -379,26 +398,36 @@ cudaError_t tbt3_step(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool diri
     return tbt3_t<K>(maps, a, dirichlet, g, s);
 }
 
-template <int KK>
-cudaError_t batch_tbt3_t(const lbmk::BatchTbtArgs& a, bool dirichlet, int ntiles, cudaStream_t s)
+template <int KK, int NL>
+cudaError_t batch_tbp_nl(const lbmk::BatchTbpArgs& a, bool dirichlet, int ntiles, cudaStream_t s)
 {
-    if constexpr (KK == lbmk::K_F32 || KK == lbmk::K_BF16 || KK == lbmk::K_F16) {
-        using G = lbmk::Tbt3Geom<(int)sizeof(typename lbmk::Fmt<KK>::E)>;
-        if (ntiles <= 0) return cudaSuccess;
-        void (*kern)(lbmk::BatchTbtArgs) =
-            dirichlet ? lbmk::batch_tbt3_kernel<KK, true> : lbmk::batch_tbt3_kernel<KK, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-        if (e != cudaSuccess) return e;
-        kern<<<ntiles, lbmk::TBT_THREADS, G::SMEM, s>>>(a);
-        return cudaGetLastError();
-    } else {
-        return cudaErrorNotSupported;
-    }
+    using G = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>;
+    void (*kern)(lbmk::BatchTbpArgs) =
+        dirichlet ? lbmk::batch_tbp_kernel<KK, NL, true> : lbmk::batch_tbp_kernel<KK, NL, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+    if (e != cudaSuccess) return e;
+    return lbmh::launch_dependent(kern, dim3(ntiles), dim3(G::THREADS), G::SMEM, s, a);
 }
 
-cudaError_t batch_tbt3_step(const lbmk::BatchTbtArgs& a, bool dirichlet, int ntiles, cudaStream_t s)
+template <int KK>
+cudaError_t batch_tbp_t(const lbmk::BatchTbpArgs& a, int steps, bool dirichlet, int ntiles, cudaStream_t s)
 {
-    return batch_tbt3_t<K>(a, dirichlet, ntiles, s);
+    if (ntiles <= 0) return cudaSuccess;
+    if constexpr (KK == lbmk::K_F32 || KK == lbmk::K_BF16 || KK == lbmk::K_F16) {
+        constexpr int MX = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>::NLMAX;
+        switch (steps) {
+        case 2: if constexpr (MX >= 4) return batch_tbp_nl<KK, 2>(a, dirichlet, ntiles, s); break;
+        case 3: return batch_tbp_nl<KK, 3>(a, dirichlet, ntiles, s);
+        case 4: if constexpr (MX >= 4) return batch_tbp_nl<KK, 4>(a, dirichlet, ntiles, s); break;
+        case 5: if constexpr (MX >= 5) return batch_tbp_nl<KK, 5>(a, dirichlet, ntiles, s); break;
+        }
+    }
+    return cudaErrorNotSupported;
+}
+
+cudaError_t batch_tbp_step(const lbmk::BatchTbpArgs& a, int steps, bool dirichlet, int ntiles, cudaStream_t s)
+{
+    return batch_tbp_t<K>(a, steps, dirichlet, ntiles, s);
 }
 
 cudaError_t batch_occupancy(int* n)
@@ -416,7 +445,7 @@ namespace lbmh {
 const KindOps LBM_OPS_NAME(LBM_KIND) = {
     K, V, ELEM, NODE_BYTES,
     step, init, moments, get_pop, set_pop, energy, error, finite, batch_step, batch_occupancy, tb2_step, tbt_step,
-    tbt3_step, step_staged, step_multi, batch_tbt3_step,
+    tbt3_step, tbp_step, step_staged, step_multi, batch_tbp_step,
     LBM_VEC_SPLIT, VB,
 };
 

@@ -25,22 +25,10 @@
 #include "lbm_kernels.cuh"
 #include "lbm_ms.cuh"
 #include "lbm_tb.cuh"
+#include "lbm_tbp.cuh"
 #include "lbm_tma.cuh"
 
 namespace lbmk {
-
-// r modulo ny in [0, ny) for r within three rows of the lattice (the staged rows of the
-// three-step kernels): one wrap suffices unless ny = 2, where the remainder is taken
-__device__ __forceinline__ int wrap_row(int r, int ny)
-{
-    if (r < 0) r += ny;
-    else if (r >= ny) r -= ny;
-    if ((unsigned)r >= (unsigned)ny) {
-        const int q = r % ny;
-        r = q < 0 ? q + ny : q;
-    }
-    return r;
-}
 
 struct TbtArgs {
     const void* src;       // f*(t) planes (wrapped edge columns are read here)
@@ -75,215 +63,6 @@ constexpr int TBT_L2_AHEAD = 0;               // default rows the producer prefe
                                               // (measured: any prefetch distance made the kernels slower)
 constexpr int TBT_OUT = TBT_WARPS * TB_OUT;   // output columns per block (120)
 constexpr int TBT_THREADS = 32 * (TBT_WARPS + 1);
-
-template <int ES>
-struct TbtGeom {
-    static constexpr int HL = 16 / ES;                                 // staged columns left of the tile
-    static constexpr int WIN = HL + TBT_OUT + HL;                      // staged columns per row
-    static constexpr int ROW_BYTES = 20 * WIN * ES;                    // one row of the 20 planes
-    static constexpr int STAGE_BYTES = (ROW_BYTES + 127) / 128 * 128;  // stage starts 128-byte aligned
-    static constexpr int NST = (ES == 4) ? LBM_TBT_NST4 : LBM_TBT_NST2; // stages in the ring
-    static constexpr int SMEM = NST * STAGE_BYTES + 128;               // dynamic shared memory per block
-                                                                       // (+128: the ring starts 128-B aligned)
-    static_assert((WIN * ES) % 16 == 0, "staged row width must be a multiple of 16 bytes");
-    static_assert(WIN <= 256, "tensor-copy box width");
-};
-
-template <int K, bool DIRICHLET>
-__global__ void __launch_bounds__(TBT_THREADS, 3) tbt_kernel(const __grid_constant__ CUtensorMap map, TbtArgs A)
-{
-    using E = typename Fmt<K>::E;
-    using G = TbtGeom<(int)sizeof(E)>;
-    constexpr int NST = G::NST, WIN = G::WIN, HL = G::HL;
-    extern __shared__ __align__(128) unsigned char tbt_smem_raw[];
-    __shared__ __align__(8) unsigned long long full_bar[NST], empty_bar[NST];
-    __shared__ int abort_flag;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nx = A.nx, ny = A.ny;
-    const int X0 = blockIdx.x * TBT_OUT;
-    const int y0 = blockIdx.y * A.rows;
-    const int y1 = min(ny, y0 + A.rows);
-    const int nin = (y1 - y0) + 4;                   // staged input rows y0-2 .. y1+1
-    const uint32_t raw = lbmt::smem_u32(tbt_smem_raw);
-    const uint32_t sbase = (raw + 127u) & ~127u;                    // 128-byte aligned ring
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < NST; ++s) {
-            lbmt::mbar_init(lbmt::smem_u32(&full_bar[s]), 1);
-            lbmt::mbar_init(lbmt::smem_u32(&empty_bar[s]), TBT_WARPS);
-        }
-        abort_flag = 0;
-        lbmt::fence_mbar_init();
-    }
-    __syncthreads();
-
-    if (warp == TBT_WARPS) {
-        // ---- producer: one tensor copy per input row, as far ahead as the ring allows ----
-        if (lane == 0) {
-            lbmt::prefetch_map(&map);
-            for (int jp = NST; jp < NST + A.l2_ahead && jp < nin; ++jp) {
-                const int yp = y0 - 2 + jp;
-                if (!DIRICHLET || (yp >= 0 && yp < ny))
-                    lbmt::tma_prefetch_3d(&map, X0 - HL, (yp < 0) ? yp + ny : (yp >= ny ? yp - ny : yp), 0);
-            }
-            int j = 0;
-            for (; j < nin; ++j) {
-                const int s = j % NST;
-                const uint32_t fb = lbmt::smem_u32(&full_bar[s]);
-                if (j == A.withhold) continue;               // test hook: this row never arrives
-                if (j >= NST && !lbmt::mbar_wait(lbmt::smem_u32(&empty_bar[s]), ((j / NST) - 1) & 1, &abort_flag))
-                    break;
-                {
-                    // the row the ring will reach l2_ahead copies later: into L2 now
-                    const int jp = j + A.l2_ahead;
-                    const int yp = y0 - 2 + jp;
-                    if (j >= NST && A.l2_ahead > 0 && jp < nin && (!DIRICHLET || (yp >= 0 && yp < ny)))
-                        lbmt::tma_prefetch_3d(&map, X0 - HL, (yp < 0) ? yp + ny : (yp >= ny ? yp - ny : yp), 0);
-                }
-                int y = y0 - 2 + j;
-                if (DIRICHLET && (y < 0 || y >= ny)) {
-                    lbmt::mbar_arrive(fb);                   // row outside the lattice: never read
-                    continue;
-                }
-                if (!DIRICHLET) y = (y < 0) ? y + ny : (y >= ny ? y - ny : y);
-                lbmt::mbar_arrive_expect_tx(fb, G::ROW_BYTES);
-                lbmt::tma_load_3d(sbase + s * G::STAGE_BYTES, &map, X0 - HL, y, 0, fb);
-            }
-            // every copy issued has landed before the block leaves
-            for (int q = (j > NST ? j - NST : 0); q < j; ++q)
-                if (q != A.withhold) lbmt::mbar_drain(lbmt::smem_u32(&full_bar[q % NST]), (q / NST) & 1);
-            if (abort_flag) atomicExch(A.timeout, 1);
-        }
-        return;
-    }
-
-    // ---- compute warps ----
-    const E* __restrict__ src = static_cast<const E*>(A.src);
-    E* __restrict__ dst = static_cast<E*>(A.dst);
-    const long long plane = A.plane;
-    const int xs = X0 - 1 + TB_OUT * warp + lane;        // this lane's S1 column (may be -1 or >= nx)
-    const int xc = DIRICHLET ? (xs < 0 ? 0 : (xs >= nx ? nx - 1 : xs)) : ((xs % nx) + nx) % nx;
-    const bool out_lane = (lane >= 1) && (lane <= TB_OUT) && (xs >= 0) && (xs < nx);
-    const bool staged = DIRICHLET || (xs >= 1 && xs + 1 <= nx - 1);   // all three columns in the tile
-    const int xl = (xc == 0) ? nx - 1 : xc - 1, xr = (xc == nx - 1) ? 0 : xc + 1;
-    const int idx = xs - X0 + HL;                        // shared-memory column of xs
-    const float fa = A.af, fb = A.bf;
-    const float Dk[5] = {-1.f, -1.f, 1.f, 1.f, 1.f};
-
-    float keep_py[5], prev[4][5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        keep_py[k] = 0.f;
-#pragma unroll
-        for (int d = 0; d < 4; ++d) prev[d][k] = 0.f;
-    }
-    bool ok = lbmt::mbar_wait(lbmt::smem_u32(&full_bar[0]), 0, &abort_flag) &&
-              lbmt::mbar_wait(lbmt::smem_u32(&full_bar[1 % NST]), (1 / NST) & 1, &abort_flag);
-    for (int i = 0; i + 2 < nin; ++i) {
-        const int r = y0 - 1 + i;                        // S1 row, from staged rows i, i+1, i+2
-        {
-            const int j = i + 2;
-            ok = ok && lbmt::mbar_wait(lbmt::smem_u32(&full_bar[j % NST]), (j / NST) & 1, &abort_flag);
-        }
-        if (!__all_sync(0xffffffffu, ok)) break;
-        // shared addresses of this lane's column in the staged rows r-1, r, r+1
-        constexpr uint32_t ES = sizeof(E), PL = WIN * sizeof(E);
-        const uint32_t rm = sbase + (i % NST) * G::STAGE_BYTES + idx * ES;
-        const uint32_t rc = sbase + ((i + 1) % NST) * G::STAGE_BYTES + idx * ES;
-        const uint32_t rp = sbase + ((i + 2) % NST) * G::STAGE_BYTES + idx * ES;
-        // ---- S1(r) at column xc ----
-        float cur[4][5];
-        const bool row_ok = DIRICHLET ? (r >= 0 && r < ny) : true;
-        {
-            float f[4][5];
-            if (staged) {
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    f[0][k] = Fmt<K>::ld(lbmt::lds<E>(rc + (0 * 5 + k) * PL - ES));
-                    f[2][k] = Fmt<K>::ld(lbmt::lds<E>(rc + (2 * 5 + k) * PL + ES));
-                    f[1][k] = Fmt<K>::ld(lbmt::lds<E>(rm + (1 * 5 + k) * PL));
-                    f[3][k] = Fmt<K>::ld(lbmt::lds<E>(rp + (3 * 5 + k) * PL));
-                }
-            } else {
-                // periodic wrap around x = 0 / x = nx - 1: read the wrapped columns directly
-                const int ry = (r < 0) ? r + ny : (r >= ny ? r - ny : r);
-                const int rmy = (ry == 0) ? ny - 1 : ry - 1, rpy = (ry == ny - 1) ? 0 : ry + 1;
-                const long long o = (long long)ry * A.pitch;
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    f[0][k] = sload<K>(src + (0 * 5 + k) * plane + o + xl);
-                    f[2][k] = sload<K>(src + (2 * 5 + k) * plane + o + xr);
-                    f[1][k] = sload<K>(src + (1 * 5 + k) * plane + (long long)rmy * A.pitch + xc);
-                    f[3][k] = sload<K>(src + (3 * 5 + k) * plane + (long long)rpy * A.pitch + xc);
-                }
-            }
-            if (DIRICHLET) {
-                const bool bot = r == 0, top = r == ny - 1;
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    if (xc == 0) f[0][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (2 * 5 + k) * PL));
-                    if (xc == nx - 1) f[2][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (0 * 5 + k) * PL));
-                    if (bot) f[1][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (3 * 5 + k) * PL));
-                    if (top) f[3][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (1 * 5 + k) * PL));
-                }
-            }
-            float U[5], rx[5], ry2[5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                rx[k] = f[1][k] + f[3][k];
-                ry2[k] = f[0][k] + f[2][k];
-                U[k] = rx[k] + ry2[k];
-            }
-            collide<float>(f, U, rx, ry2, fa, fb, cur);
-            if (!row_ok)
-#pragma unroll
-                for (int d = 0; d < 4; ++d)
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) cur[d][k] = 0.f;
-        }
-        // staged row i (row r-1) is not read again
-        __syncwarp();
-        if (lane == 0) lbmt::mbar_arrive(lbmt::smem_u32(&empty_bar[i % NST]));
-        // ---- S2(r-1) from S1(r-2), S1(r-1), S1(r) ----
-        const int q = r - 1;
-        if (q >= y0) {
-            const bool bot = DIRICHLET && q == 0, top = DIRICHLET && q == ny - 1;
-            float f[4][5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                f[0][k] = __shfl_up_sync(0xffffffffu, prev[0][k], 1);
-                f[2][k] = __shfl_down_sync(0xffffffffu, prev[2][k], 1);
-                f[1][k] = bot ? Dk[k] * prev[3][k] : keep_py[k];
-                f[3][k] = top ? Dk[k] * prev[1][k] : cur[3][k];
-                if (DIRICHLET && xs == 0) f[0][k] = Dk[k] * prev[2][k];
-                if (DIRICHLET && xs == nx - 1) f[2][k] = Dk[k] * prev[0][k];
-            }
-            float U[5], rx[5], ry2[5], o[4][5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                rx[k] = f[1][k] + f[3][k];
-                ry2[k] = f[0][k] + f[2][k];
-                U[k] = rx[k] + ry2[k];
-            }
-            collide<float>(f, U, rx, ry2, fa, fb, o);
-            if (out_lane) {
-                const long long off = (long long)q * A.pitch + xs;
-#pragma unroll
-                for (int d = 0; d < 4; ++d)
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) dst[(d * 5 + k) * plane + off] = Fmt<K>::st(o[d][k]);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            keep_py[k] = prev[1][k];
-#pragma unroll
-            for (int d = 0; d < 4; ++d) prev[d][k] = cur[d][k];
-        }
-    }
-    if (lane == 0 && abort_flag) atomicExch(A.timeout, 1);
-}
 
 // ---------------------------------------------------------------------------
 // Moment-space storage (lbm_ms.cuh): the same two-step pass over a state of 5 FP32
@@ -891,268 +670,6 @@ __global__ void __launch_bounds__(TBT_THREADS, LBM_TBT3MS_MIN_BLOCKS) tbt3_ms_ke
         }
     }
     if (lane == 0 && abort_flag) atomicExch(A.timeout, 1);
-}
-
-
-// ---------------------------------------------------------------------------
-// Population formats, three steps per pass (tbt3_kernel): tbt_kernel's staging with the
-// three register levels of tbt3_ms_kernel (S1 from the staged rows, S2, S3 stored by
-// lanes 2..29 of each warp, 112 columns per block, staged rows y0 - 3 .. y1 + 2).  Same
-// arithmetic as single steps, so FP32 results stay bit-identical to them.
-// ---------------------------------------------------------------------------
-#ifndef LBM_TBT3_NST4
-#define LBM_TBT3_NST4 7
-#endif
-#ifndef LBM_TBT3_NST2
-#define LBM_TBT3_NST2 4
-#endif
-
-template <int ES>
-struct Tbt3Geom {
-    static constexpr int HL = 16 / ES;                                 // >= 3 staged columns each side
-    static constexpr int WIN = HL + TBT3_OUT + HL;
-    static constexpr int ROW_BYTES = 20 * WIN * ES;
-    static constexpr int STAGE_BYTES = (ROW_BYTES + 127) / 128 * 128;
-    static constexpr int NST = (ES == 4) ? LBM_TBT3_NST4 : LBM_TBT3_NST2;
-    static constexpr int SMEM = NST * STAGE_BYTES + 128;
-    static_assert((WIN * ES) % 16 == 0 && HL >= 3, "staged row geometry");
-};
-
-#ifndef LBM_TBT3_MIN_BLOCKS
-#define LBM_TBT3_MIN_BLOCKS 3       // 116-127 registers
-#endif
-
-// One block's work: output columns X0 .. X0 + TBT3_OUT - 1 and rows y0 .. y0 + A.rows - 1 of
-// the lattice A describes, its rows staged through `map` (a generic address: a kernel
-// parameter or a map in global memory).
-template <int K, bool DIRICHLET>
-__device__ __forceinline__ void tbt3_body(const CUtensorMap* mapp, const TbtArgs& A, int X0, int y0)
-{
-    using E = typename Fmt<K>::E;
-    using G = Tbt3Geom<(int)sizeof(E)>;
-    constexpr int NST = G::NST, WIN = G::WIN, HL = G::HL;
-    extern __shared__ __align__(128) unsigned char tbt_smem_raw[];
-    __shared__ __align__(8) unsigned long long full_bar[NST], empty_bar[NST];
-    __shared__ int abort_flag;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nx = A.nx, ny = A.ny;
-    const int y1 = min(ny, y0 + A.rows);
-    const int nin = (y1 - y0) + 6;                   // staged input rows y0-3 .. y1+2
-    const uint32_t raw = lbmt::smem_u32(tbt_smem_raw);
-    const uint32_t sbase = (raw + 127u) & ~127u;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < NST; ++s) {
-            lbmt::mbar_init(lbmt::smem_u32(&full_bar[s]), 1);
-            lbmt::mbar_init(lbmt::smem_u32(&empty_bar[s]), TBT_WARPS);
-        }
-        abort_flag = 0;
-        lbmt::fence_mbar_init();
-    }
-    __syncthreads();
-
-    if (warp == TBT_WARPS) {
-        if (lane == 0) {
-            lbmt::prefetch_map(mapp);
-            int j = 0;
-            for (; j < nin; ++j) {
-                const int s = j % NST;
-                const uint32_t fb = lbmt::smem_u32(&full_bar[s]);
-                if (j == A.withhold) continue;
-                if (j >= NST && !lbmt::mbar_wait(lbmt::smem_u32(&empty_bar[s]), ((j / NST) - 1) & 1, &abort_flag))
-                    break;
-                int y = y0 - 3 + j;
-                if (DIRICHLET && (y < 0 || y >= ny)) {
-                    lbmt::mbar_arrive(fb);
-                    continue;
-                }
-                if (!DIRICHLET) y = wrap_row(y, ny);   // rows y0 - 3 .. y1 + 2: more than one wrap when ny = 2
-                lbmt::mbar_arrive_expect_tx(fb, G::ROW_BYTES);
-                lbmt::tma_load_3d(sbase + s * G::STAGE_BYTES, mapp, X0 - HL, y, 0, fb);
-            }
-            for (int q = (j > NST ? j - NST : 0); q < j; ++q)
-                if (q != A.withhold) lbmt::mbar_drain(lbmt::smem_u32(&full_bar[q % NST]), (q / NST) & 1);
-            if (abort_flag) atomicExch(A.timeout, 1);
-        }
-        return;
-    }
-
-    const E* __restrict__ src = static_cast<const E*>(A.src);
-    E* __restrict__ dst = static_cast<E*>(A.dst);
-    const long long plane = A.plane;
-    const int xs = X0 - 2 + TB3_OUT * warp + lane;   // this lane's S1 column
-    const int xc = DIRICHLET ? (xs < 0 ? 0 : (xs >= nx ? nx - 1 : xs)) : ((xs % nx) + nx) % nx;
-    const bool out_lane = (lane >= 2) && (lane < 2 + TB3_OUT) && (xs >= 0) && (xs < nx);
-    const bool staged = DIRICHLET || (xs >= 1 && xs + 1 <= nx - 1);
-    const int xl = (xc == 0) ? nx - 1 : xc - 1, xr = (xc == nx - 1) ? 0 : xc + 1;
-    const int idx = xs - X0 + HL;
-    const float fa = A.af, fb = A.bf;
-    const float Dk[5] = {-1.f, -1.f, 1.f, 1.f, 1.f};
-
-    float p1[4][5], k1[5], p2[4][5], k2[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        k1[k] = k2[k] = 0.f;
-#pragma unroll
-        for (int d = 0; d < 4; ++d) p1[d][k] = p2[d][k] = 0.f;
-    }
-    bool ok = lbmt::mbar_wait(lbmt::smem_u32(&full_bar[0]), 0, &abort_flag) &&
-              lbmt::mbar_wait(lbmt::smem_u32(&full_bar[1 % NST]), (1 / NST) & 1, &abort_flag);
-    for (int i = 0; i + 2 < nin; ++i) {
-        const int r = y0 - 2 + i;                    // S1 row, from staged rows i, i+1, i+2
-        {
-            const int j = i + 2;
-            ok = ok && lbmt::mbar_wait(lbmt::smem_u32(&full_bar[j % NST]), (j / NST) & 1, &abort_flag);
-        }
-        if (!__all_sync(0xffffffffu, ok)) break;
-        constexpr uint32_t ES = sizeof(E), PL = WIN * sizeof(E);
-        const uint32_t rm = sbase + (i % NST) * G::STAGE_BYTES + idx * ES;
-        const uint32_t rc = sbase + ((i + 1) % NST) * G::STAGE_BYTES + idx * ES;
-        const uint32_t rp = sbase + ((i + 2) % NST) * G::STAGE_BYTES + idx * ES;
-        float c1[4][5];
-        {
-            float f[4][5];
-            if (staged) {
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    f[0][k] = Fmt<K>::ld(lbmt::lds<E>(rc + (0 * 5 + k) * PL - ES));
-                    f[2][k] = Fmt<K>::ld(lbmt::lds<E>(rc + (2 * 5 + k) * PL + ES));
-                    f[1][k] = Fmt<K>::ld(lbmt::lds<E>(rm + (1 * 5 + k) * PL));
-                    f[3][k] = Fmt<K>::ld(lbmt::lds<E>(rp + (3 * 5 + k) * PL));
-                }
-            } else {
-                const int ry = (r < 0) ? r + ny : (r >= ny ? r - ny : r);
-                const int rmy = (ry == 0) ? ny - 1 : ry - 1, rpy = (ry == ny - 1) ? 0 : ry + 1;
-                const long long o = (long long)ry * A.pitch;
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    f[0][k] = sload<K>(src + (0 * 5 + k) * plane + o + xl);
-                    f[2][k] = sload<K>(src + (2 * 5 + k) * plane + o + xr);
-                    f[1][k] = sload<K>(src + (1 * 5 + k) * plane + (long long)rmy * A.pitch + xc);
-                    f[3][k] = sload<K>(src + (3 * 5 + k) * plane + (long long)rpy * A.pitch + xc);
-                }
-            }
-            if (DIRICHLET) {
-                const bool bot = r == 0, top = r == ny - 1;
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    if (xc == 0) f[0][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (2 * 5 + k) * PL));
-                    if (xc == nx - 1) f[2][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (0 * 5 + k) * PL));
-                    if (bot) f[1][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (3 * 5 + k) * PL));
-                    if (top) f[3][k] = Dk[k] * Fmt<K>::ld(lbmt::lds<E>(rc + (1 * 5 + k) * PL));
-                }
-            }
-            float U[5], rx[5], ry2[5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                rx[k] = f[1][k] + f[3][k];
-                ry2[k] = f[0][k] + f[2][k];
-                U[k] = rx[k] + ry2[k];
-            }
-            collide<float>(f, U, rx, ry2, fa, fb, c1);
-            if (DIRICHLET && !(r >= 0 && r < ny))
-#pragma unroll
-                for (int d = 0; d < 4; ++d)
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) c1[d][k] = 0.f;
-        }
-        __syncwarp();
-        if (lane == 0) lbmt::mbar_arrive(lbmt::smem_u32(&empty_bar[i % NST]));
-        const int q2 = r - 1;
-        if (q2 >= y0 - 1) {
-            float c2[4][5];
-            level_step<DIRICHLET>(p1, k1, c1[3], q2, xs, nx, ny, fa, fb, c2);
-            if (DIRICHLET && !(q2 >= 0 && q2 < ny))
-#pragma unroll
-                for (int d = 0; d < 4; ++d)
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) c2[d][k] = 0.f;
-            const int q3 = r - 2;
-            if (q3 >= y0) {
-                float o[4][5];
-                level_step<DIRICHLET>(p2, k2, c2[3], q3, xs, nx, ny, fa, fb, o);
-                if (out_lane) {
-                    const long long off = (long long)q3 * A.pitch + xs;
-#pragma unroll
-                    for (int d = 0; d < 4; ++d)
-#pragma unroll
-                        for (int k = 0; k < 5; ++k) dst[(d * 5 + k) * plane + off] = Fmt<K>::st(o[d][k]);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                k2[k] = p2[1][k];
-#pragma unroll
-                for (int d = 0; d < 4; ++d) p2[d][k] = c2[d][k];
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            k1[k] = p1[1][k];
-#pragma unroll
-            for (int d = 0; d < 4; ++d) p1[d][k] = c1[d][k];
-        }
-    }
-    if (lane == 0 && abort_flag) atomicExch(A.timeout, 1);
-}
-
-template <int K, bool DIRICHLET>
-__global__ void __launch_bounds__(TBT_THREADS, LBM_TBT3_MIN_BLOCKS) tbt3_kernel(const __grid_constant__ CUtensorMap map, TbtArgs A)
-{
-    tbt3_body<K, DIRICHLET>(&map, A, blockIdx.x * TBT3_OUT, blockIdx.y * A.rows);
-}
-
-// ---------------------------------------------------------------------------
-// Batches of lattices, three steps per pass (lbm_batch.cu, mode 2): one block per tile
-// {lattice, X0, y0} of a flat list, each running tbt3_body on its lattice with that
-// lattice's row map of the source arena.  The maps live in global memory, written by the
-// host before the launch; a lattice's planes sit at its element offset in each arena.
-// ---------------------------------------------------------------------------
-struct BatchLatT3 {
-    long long off;         // element offset of plane 0 in each arena
-    long long plane;       // elements per plane = ny * pitch
-    int nx, ny, pitch;
-    float af, bf;          // cK / c, cmu / c in FP32
-    int pad_;
-};
-
-struct BatchTbtArgs {
-    const int4* tiles;          // {lattice, X0, y0, 0} per block
-    const BatchLatT3* lat;
-    const CUtensorMap* maps;    // [lattice][arena]: row maps (box width Tbt3Geom::WIN)
-    void* arenaA;
-    void* arenaB;
-    int parity;                 // 0: read arena A, write arena B
-    int rows;                   // output rows per tile
-    int* timeout;               // set when a bounded wait ran out
-};
-
-template <int K, bool DIRICHLET>
-__global__ void __launch_bounds__(TBT_THREADS, LBM_TBT3_MIN_BLOCKS) batch_tbt3_kernel(BatchTbtArgs B)
-{
-    using E = typename Fmt<K>::E;
-    const int4 t = B.tiles[blockIdx.x];
-    const BatchLatT3 L = B.lat[t.x];
-    E* a = static_cast<E*>(B.arenaA) + L.off;
-    E* b = static_cast<E*>(B.arenaB) + L.off;
-    TbtArgs A;
-    A.src = B.parity ? b : a;
-    A.dst = B.parity ? a : b;
-    A.nx = L.nx;
-    A.ny = L.ny;
-    A.pitch = L.pitch;
-    A.plane = L.plane;
-    A.af = L.af;
-    A.bf = L.bf;
-    A.rows = B.rows;
-    A.timeout = B.timeout;
-    A.withhold = -1;
-    A.scale = 1.f;
-    A.inv_s = 1.f;
-    A.sat = nullptr;
-    A.l2_ahead = 0;
-    tbt3_body<K, DIRICHLET>(B.maps + 2 * t.x + B.parity, A, t.y, t.z);
 }
 
 }  // namespace lbmk

@@ -1,6 +1,6 @@
-"""Step kernels chosen by size, against the same steps taken one kernel at a time: several FP64
-steps in one launch on small lattices, and the FP64 step with a body load on staged rows against the
-register kernel.  All bit for bit."""
+"""Step kernels chosen by size, against the same steps taken one kernel at a time: several FP32
+steps per pass (default grouping), several FP64 steps in one launch on small lattices, and the FP64
+step with a body load on staged rows against the register kernel.  All bit for bit."""
 import numpy as np
 import pytest
 
@@ -26,6 +26,35 @@ def _state(lat):
     f, us = lat.populations()
     lat.close()
     return f, us
+
+
+# tiles of 168 columns (56 per warp, 4 halo columns), copies of the wrapped columns for lattices
+# wider than a tile; row blocks from 2 to 96 rows
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("nx,ny,steps", [(2, 2, 4), (3, 5, 9), (55, 3, 5), (57, 9, 6), (112, 2, 7), (167, 11, 13),
+                                         (168, 8, 8), (169, 4, 4), (171, 33, 11), (173, 200, 10), (335, 7, 21),
+                                         (337, 40, 4), (1000, 3, 6), (61, 1500, 8)])
+def test_fp32_default_passes_equal_single_steps(lbm, nx, ny, steps, dirichlet):
+    one = _lattice(lbm, nx, ny, dirichlet, "f32", False)
+    one.set_step_fusion(1)
+    one.step(steps)
+    many = _lattice(lbm, nx, ny, dirichlet, "f32", False)
+    many.step(steps)
+    np.testing.assert_array_equal(_state(one)[0], _state(many)[0])
+
+
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("nx,ny", [(55, 3), (119, 11), (121, 130), (239, 5), (240, 64), (241, 9), (243, 4), (481, 70)])
+def test_bf16_passes_do_not_depend_on_the_row_blocks(lbm, nx, ny, dirichlet):
+    states = []
+    for rows in (0, 2, 5, 64):
+        lat = _lattice(lbm, nx, ny, dirichlet, "bf16", False)
+        if rows:
+            lat.set_step_fusion(3, rows)
+        lat.step(8)
+        states.append(_state(lat)[0])
+    for s in states[1:]:
+        np.testing.assert_array_equal(states[0], s)
 
 
 # one segment of 32 columns per warp, four per block; the largest still takes one launch
