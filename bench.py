@@ -59,7 +59,7 @@ TRAFFIC_CAPTURE = {"sha256": "427275c0b852342612482484dcd6605f8b9ba6a8e2209f6534
                                       "ms_f16_fused3": 105.11, "ms_bfp_fused3": 105.2}}
 KERNEL_SOURCES = ["paper_2408_01081_gb300/csrc/lbm_kernels.cuh", "paper_2408_01081_gb300/csrc/lbm_kind.cu",
                   "paper_2408_01081_gb300/csrc/lbm_tb.cuh", "paper_2408_01081_gb300/csrc/lbm_ms.cuh",
-                  "paper_2408_01081_gb300/csrc/lbm_tbp.cuh", "paper_2408_01081_gb300/csrc/lbm_tbt.cuh", "paper_2408_01081_gb300/csrc/lbm_tma.cuh",
+                  "paper_2408_01081_gb300/csrc/lbm_tbp.cuh", "paper_2408_01081_gb300/csrc/lbm_tbpms.cuh", "paper_2408_01081_gb300/csrc/lbm_tma.cuh",
                   "paper_2408_01081_gb300/csrc/lbm_f64emu.cuh", "paper_2408_01081_gb300/csrc/lbm_mscodec.cuh",
                   "paper_2408_01081_gb300/csrc/lbm_f64stage.cuh", "paper_2408_01081_gb300/csrc/lbm_f64fx.cuh"]
 # Pipe instruction counts of the default FP64 step kernel (step_f64_staged_kernel, split level 12) per node

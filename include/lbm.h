@@ -114,8 +114,7 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
  * run instead); a remainder of one or two steps runs as a single step or a pair
  * (LBM_F32: passes of equal length instead).
  * rows_per_block sets the rows each thread block streams through (0 keeps the
- * default: for the population formats from the lattice's size, 2 to 96; 64 for moment
- * space; for the staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
+ * default: from the lattice's size, 2 to 96; for the staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
  * level 1, fewer on small lattices).  By default (this call not made, staging 1)
  * the steps of one lbm_step call on a small LBM_F64 lattice at split level 12 (up to
  * about 1800 segments of 32 columns of a row) run in one cooperative launch, with

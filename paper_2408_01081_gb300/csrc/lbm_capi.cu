@@ -5,7 +5,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -220,17 +219,14 @@ struct lbm_ctx {
     int echeck_since = 0;        // steps since the last check
     int staging = 1;             // 1 = rows staged in shared memory (tensor copies for the fused kernels,
                                  // asynchronous copies for the FP64 step), 0 = register loads
-    int l2_ahead = lbmk::TBT_L2_AHEAD;   // staged kernel: rows prefetched into L2 ahead of the ring
-                                         // (environment LBM_TBT_L2_AHEAD, 0..64, read at lbm_create)
     int nyi = 0;                 // rows of the lattice's own (a slab: without its halo rows)
     int yo = 0;                  // storage row of own row 0 (1 when a halo row sits below)
     bool slab = false;           // a row slab of a larger lattice (lbm_create_slab)
     int halo_lo = 0, halo_hi = 0;  // halo rows below / above the slab's own rows (0 or 1)
     bool maps_ok = false;        // row maps of both buffers encoded (all formats but FP64)
-    CUtensorMap map[2][2];       // row maps of buf[0], buf[1] for the staged fused kernels
-                                 // ([buffer][part]; moment space: FP32 part, 16-bit part;
-                                 // populations: row map, wrap map)
-    CUtensorMap map3[2][2];      // moment space: row maps of the three-step kernel (narrower box)
+    CUtensorMap map[2][4];       // maps of buf[0], buf[1] for the staged fused kernels: populations: row
+                                 // map, wrap map; moment space: row maps of the FP32 and the 16-bit
+                                 // part, then their wrap maps
 };
 
 namespace {
@@ -436,10 +432,6 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out)
     }
     ctx->p = *p;
     ctx->nyi = p->ny;
-    if (const char* v = std::getenv("LBM_TBT_L2_AHEAD")) {
-        const int a = std::atoi(v);
-        if (a >= 0 && a <= 64) ctx->l2_ahead = a;
-    }
     ctx->s = static_cast<cudaStream_t>(p->stream);
     ctx->ops = ops_for(p->storage);
     ctx->pitch = (p->nx + 63) / 64 * 64;
@@ -502,18 +494,20 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out)
                                            wrap);
     }
     if (e == cudaSuccess && (p->storage == LBM_MS_BF16 || p->storage == LBM_MS_F16 || p->storage == LBM_MS_BFP)) {
-        const int win = lbmk::TbtMsGeom::WIN;
+        using G = lbmk::TbpMsGeom;
+        ctx->tbp_rows = lbmk::tbp_rows(152 * G::MIN_BLOCKS, p->ny, [&](int r) {
+            return (long long)((p->nx + G::OUT - 1) / G::OUT) * ((p->ny + r - 1) / r);
+        });
         ctx->maps_ok = true;
         for (int i = 0; i < 2; ++i) {
             char* b = static_cast<char*>(ctx->buf[i]);
-            const int win3 = lbmk::Tbt3MsGeom::WIN;
+            char* d = b + 20 * ctx->plane;
+            CUtensorMap* m = ctx->map[i];
             ctx->maps_ok = ctx->maps_ok &&
-                           encode_rows_map(&ctx->map[i][0], b, 4, p->nx, p->ny, ctx->pitch, ctx->plane, 5, win) &&
-                           encode_rows_map(&ctx->map[i][1], b + 20 * ctx->plane, 2, p->nx, p->ny, ctx->pitch,
-                                           ctx->plane, 15, win) &&
-                           encode_rows_map(&ctx->map3[i][0], b, 4, p->nx, p->ny, ctx->pitch, ctx->plane, 5, win3) &&
-                           encode_rows_map(&ctx->map3[i][1], b + 20 * ctx->plane, 2, p->nx, p->ny, ctx->pitch,
-                                           ctx->plane, 15, win3);
+                           encode_rows_map(m, b, 4, p->nx, p->ny, ctx->pitch, ctx->plane, 5, G::WIN) &&
+                           encode_rows_map(m + 1, d, 2, p->nx, p->ny, ctx->pitch, ctx->plane, 15, G::WIN) &&
+                           encode_rows_map(m + 2, b, 4, p->nx, p->ny, ctx->pitch, ctx->plane, 5, G::WRAP) &&
+                           encode_rows_map(m + 3, d, 2, p->nx, p->ny, ctx->pitch, ctx->plane, 15, G::WRAP);
         }
     }
     if (e != cudaSuccess) {
@@ -928,43 +922,30 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
                     n -= k;
                 }
             }
-            lbmk::TbtArgs Q;
-            Q.nx = ctx->p.nx;
-            Q.ny = ctx->p.ny;
-            Q.pitch = ctx->pitch;
-            Q.plane = ctx->plane;
-            Q.af = (float)ctx->a;
-            Q.bf = (float)ctx->b;
-            Q.rows = ctx->tb_rows;
-            Q.timeout = reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot);
-            Q.withhold = ctx->staging == 2 ? 2 : -1;
-            Q.l2_ahead = ctx->l2_ahead;
-            Q.scale = (float)ctx->neq_scale;
-            Q.inv_s = (float)(1.0 / ctx->neq_scale);
-            Q.sat = reinterpret_cast<int*>(ctx->scratch + kSatSlot);
-            if (ms && ctx->fuse == 3) {
-                // three steps per pass: the remainder below runs as one pair or a single step
-                const dim3 q3grid((ctx->p.nx + lbmk::TBT3_OUT - 1) / lbmk::TBT3_OUT, (ctx->p.ny + Q.rows - 1) / Q.rows);
-                while (n >= 3) {
-                    Q.src = ctx->buf[ctx->cur];
+            if (ms) {
+                lbmk::TbpMsArgs Q;
+                Q.nx = ctx->p.nx;
+                Q.ny = ctx->p.ny;
+                Q.pitch = ctx->pitch;
+                Q.plane = ctx->plane;
+                Q.af = (float)ctx->a;
+                Q.bf = (float)ctx->b;
+                Q.scale = (float)ctx->neq_scale;
+                Q.inv_s = (float)(1.0 / ctx->neq_scale);
+                Q.rows = ctx->rows_set ? ctx->tb_rows : ctx->tbp_rows;
+                Q.timeout = reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot);
+                Q.sat = reinterpret_cast<int*>(ctx->scratch + kSatSlot);
+                Q.withhold = ctx->staging == 2 ? 2 : -1;
+                // rounded once per pass: whole passes, then a pair or a single step
+                while (n >= 2) {
+                    const int k = (int)std::min<long long>(n, ctx->fuse);
                     Q.dst = ctx->buf[ctx->cur ^ 1];
-                    cudaError_t e = ops->tbt3_step(ctx->map3[ctx->cur], Q, ctx->p.bc == LBM_DIRICHLET, q3grid, ctx->s);
-                    if (e != cudaSuccess) return cuda_fail(ctx, e, "staged three-step kernel");
+                    cudaError_t e = ops->tbpms_step(ctx->map[ctx->cur], Q, k, ctx->p.bc == LBM_DIRICHLET, ctx->s);
+                    if (e != cudaSuccess) return cuda_fail(ctx, e, "staged multi-step kernel");
                     ctx->cur ^= 1;
-                    ctx->m += 3;
-                    n -= 3;
+                    ctx->m += k;
+                    n -= k;
                 }
-            }
-            const dim3 qgrid((ctx->p.nx + lbmk::TBT_OUT - 1) / lbmk::TBT_OUT, (ctx->p.ny + Q.rows - 1) / Q.rows);
-            while (ms && n >= 2) {
-                Q.src = ctx->buf[ctx->cur];
-                Q.dst = ctx->buf[ctx->cur ^ 1];
-                cudaError_t e = ops->tbt_step(ctx->map[ctx->cur], Q, ctx->p.bc == LBM_DIRICHLET, qgrid, ctx->s);
-                if (e == cudaErrorNotSupported) return fail(ctx, LBM_ERR_ARG, "no staged two-step kernel for this format");
-                if (e != cudaSuccess) return cuda_fail(ctx, e, "staged two-step kernel");
-                ctx->cur ^= 1;
-                ctx->m += 2;
-                n -= 2;
             }
         }
         while (n >= 2) {

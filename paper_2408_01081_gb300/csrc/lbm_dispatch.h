@@ -11,7 +11,7 @@
 #include "lbm_ms.cuh"
 #include "lbm_tb.cuh"
 #include "lbm_tbp.cuh"
-#include "lbm_tbt.cuh"
+#include "lbm_tbpms.cuh"
 
 namespace lbmh {
 
@@ -92,14 +92,14 @@ struct KindOps {
     cudaError_t (*batch_occupancy)(int* blocks_per_sm);
     // two fused steps (FP32 / BF16 / FP16 populations only; others return cudaErrorNotSupported)
     cudaError_t (*tb2_step)(const lbmk::TbArgs&, bool dirichlet, dim3 grid, dim3 block, cudaStream_t s);
-    // two and three fused steps of the moment-space formats with the input rows staged by tensor
-    // copies; maps: the row maps of the source buffer's FP32 and 16-bit parts (box width
-    // TbtMsGeom::WIN, Tbt3MsGeom::WIN); other formats return cudaErrorNotSupported
-    cudaError_t (*tbt_step)(const CUtensorMap* maps, const lbmk::TbtArgs&, bool dirichlet, dim3 grid, cudaStream_t s);
-    cudaError_t (*tbt3_step)(const CUtensorMap* maps, const lbmk::TbtArgs&, bool dirichlet, dim3 grid, cudaStream_t s);
-    // two or three fused steps of the FP32 / BF16 / FP16 populations in the same manner; maps: the
-    // row map and the wrap map of the source buffer (20 planes, box widths TbpGeom::WIN and ::WRAP)
+    // 2 .. TbpGeom::NLMAX fused steps of the FP32 / BF16 / FP16 populations with the input rows staged
+    // by tensor copies; maps: the row map and the wrap map of the source buffer (20 planes, box widths
+    // TbpGeom::WIN and ::WRAP); other formats return cudaErrorNotSupported
     cudaError_t (*tbp_step)(const CUtensorMap* maps, const lbmk::TbpArgs&, int steps, bool dirichlet, cudaStream_t s);
+    // two or three fused steps of the moment-space formats in the same manner; maps: the row maps of
+    // the source buffer's FP32 and 16-bit parts (box width TbpMsGeom::WIN), then their wrap maps (::WRAP)
+    cudaError_t (*tbpms_step)(const CUtensorMap* maps, const lbmk::TbpMsArgs&, int steps, bool dirichlet,
+                              cudaStream_t s);
     // one FP64 step at split level 1, or 12 with or without a body load, with the rows staged by
     // asynchronous copies, `rows` rows per block (other formats and variants return
     // cudaErrorNotSupported)

@@ -345,7 +345,6 @@ cudaError_t tbp_t(const CUtensorMap* maps, const lbmk::TbpArgs& a, int steps, bo
         case 2: return tbp_nl<KK, 2>(maps, a, dirichlet, s);
         case 3: return tbp_nl<KK, 3>(maps, a, dirichlet, s);
         case 4: if constexpr (MX >= 4) return tbp_nl<KK, 4>(maps, a, dirichlet, s); break;
-        case 5: if constexpr (MX >= 5) return tbp_nl<KK, 5>(maps, a, dirichlet, s); break;
         }
     }
     return cudaErrorNotSupported;
@@ -356,46 +355,32 @@ cudaError_t tbp_step(const CUtensorMap* maps, const lbmk::TbpArgs& a, int steps,
     return tbp_t<K>(maps, a, steps, dirichlet, s);
 }
 
-template <int KK>
-cudaError_t tbt_t(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool dirichlet, dim3 g, cudaStream_t s)
+// two or three fused steps of the moment-space formats (lbm_tbpms.cuh)
+template <int KK, int NL>
+cudaError_t tbpms_nl(const CUtensorMap* maps, const lbmk::TbpMsArgs& a, bool dirichlet, cudaStream_t s)
 {
-    if constexpr (KK == lbmk::K_MSBF16 || KK == lbmk::K_MSF16 || KK == lbmk::K_MSBFP) {
-        using G = lbmk::TbtMsGeom;
-        void (*kern)(CUtensorMap, CUtensorMap, lbmk::TbtArgs) =
-            dirichlet ? lbmk::tbt_ms_kernel<KK, true> : lbmk::tbt_ms_kernel<KK, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-        if (e != cudaSuccess) return e;
-        kern<<<g, lbmk::TBT_THREADS, G::SMEM, s>>>(maps[0], maps[1], a);
-        return cudaGetLastError();
-    } else {
-        return cudaErrorNotSupported;
-    }
-}
-
-cudaError_t tbt_step(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool dirichlet, dim3 g, cudaStream_t s)
-{
-    return tbt_t<K>(maps, a, dirichlet, g, s);
+    using G = lbmk::TbpMsGeom;
+    void (*kern)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, lbmk::TbpMsArgs) =
+        dirichlet ? lbmk::tbpms_kernel<KK, NL, true> : lbmk::tbpms_kernel<KK, NL, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+    if (e != cudaSuccess) return e;
+    const dim3 g((a.nx + G::OUT - 1) / G::OUT, (a.ny + a.rows - 1) / a.rows);
+    return lbmh::launch_dependent(kern, g, dim3(G::THREADS), G::SMEM, s, maps[0], maps[1], maps[2], maps[3], a);
 }
 
 template <int KK>
-cudaError_t tbt3_t(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool dirichlet, dim3 g, cudaStream_t s)
+cudaError_t tbpms_t(const CUtensorMap* maps, const lbmk::TbpMsArgs& a, int steps, bool dirichlet, cudaStream_t s)
 {
     if constexpr (KK == lbmk::K_MSBF16 || KK == lbmk::K_MSF16 || KK == lbmk::K_MSBFP) {
-        using G = lbmk::Tbt3MsGeom;
-        void (*kern)(CUtensorMap, CUtensorMap, lbmk::TbtArgs) =
-            dirichlet ? lbmk::tbt3_ms_kernel<KK, true> : lbmk::tbt3_ms_kernel<KK, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-        if (e != cudaSuccess) return e;
-        kern<<<g, lbmk::TBT_THREADS, G::SMEM, s>>>(maps[0], maps[1], a);
-        return cudaGetLastError();
-    } else {
-        return cudaErrorNotSupported;
+        if (steps == 3) return tbpms_nl<KK, 3>(maps, a, dirichlet, s);
+        if (steps == 2) return tbpms_nl<KK, 2>(maps, a, dirichlet, s);
     }
+    return cudaErrorNotSupported;
 }
 
-cudaError_t tbt3_step(const CUtensorMap* maps, const lbmk::TbtArgs& a, bool dirichlet, dim3 g, cudaStream_t s)
+cudaError_t tbpms_step(const CUtensorMap* maps, const lbmk::TbpMsArgs& a, int steps, bool dirichlet, cudaStream_t s)
 {
-    return tbt3_t<K>(maps, a, dirichlet, g, s);
+    return tbpms_t<K>(maps, a, steps, dirichlet, s);
 }
 
 template <int KK, int NL>
@@ -419,7 +404,6 @@ cudaError_t batch_tbp_t(const lbmk::BatchTbpArgs& a, int steps, bool dirichlet, 
         case 2: if constexpr (MX >= 4) return batch_tbp_nl<KK, 2>(a, dirichlet, ntiles, s); break;
         case 3: return batch_tbp_nl<KK, 3>(a, dirichlet, ntiles, s);
         case 4: if constexpr (MX >= 4) return batch_tbp_nl<KK, 4>(a, dirichlet, ntiles, s); break;
-        case 5: if constexpr (MX >= 5) return batch_tbp_nl<KK, 5>(a, dirichlet, ntiles, s); break;
         }
     }
     return cudaErrorNotSupported;
@@ -444,8 +428,8 @@ namespace lbmh {
 
 const KindOps LBM_OPS_NAME(LBM_KIND) = {
     K, V, ELEM, NODE_BYTES,
-    step, init, moments, get_pop, set_pop, energy, error, finite, batch_step, batch_occupancy, tb2_step, tbt_step,
-    tbt3_step, tbp_step, step_staged, step_multi, batch_tbp_step,
+    step, init, moments, get_pop, set_pop, energy, error, finite, batch_step, batch_occupancy, tb2_step, tbp_step,
+    tbpms_step, step_staged, step_multi, batch_tbp_step,
     LBM_VEC_SPLIT, VB,
 };
 

@@ -43,12 +43,14 @@ def test_fp32_default_passes_equal_single_steps(lbm, nx, ny, steps, dirichlet):
     np.testing.assert_array_equal(_state(one)[0], _state(many)[0])
 
 
+@pytest.mark.parametrize("storage", ["bf16", "ms_bf16", "ms_f16", "ms_bfp"])
 @pytest.mark.parametrize("dirichlet", [False, True])
-@pytest.mark.parametrize("nx,ny", [(55, 3), (119, 11), (121, 130), (239, 5), (240, 64), (241, 9), (243, 4), (481, 70)])
-def test_bf16_passes_do_not_depend_on_the_row_blocks(lbm, nx, ny, dirichlet):
+@pytest.mark.parametrize("nx,ny", [(55, 3), (119, 11), (121, 130), (167, 4), (168, 9), (173, 5), (239, 5), (240, 64), (241, 9), (243, 4),
+                                   (481, 70)])
+def test_16_bit_passes_do_not_depend_on_the_row_blocks(lbm, nx, ny, dirichlet, storage):
     states = []
     for rows in (0, 2, 5, 64):
-        lat = _lattice(lbm, nx, ny, dirichlet, "bf16", False)
+        lat = _lattice(lbm, nx, ny, dirichlet, storage, False)
         if rows:
             lat.set_step_fusion(3, rows)
         lat.step(8)
