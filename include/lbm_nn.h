@@ -90,6 +90,12 @@ lbm_status lbm_nn_weight_flip(const void* w_bf16, int32_t Cout, int32_t Cin, int
 /* dy[i] = 0 where y[i] <= 0 (y = ReLU output). */
 lbm_status lbm_nn_relu_backward(float* dy, const float* y, int64_t n, void* stream);
 
+/* lbm_nn_relu_backward on dy, y: [P][C], and lbm_nn_bias_grad of the result, in one pass over the
+ * memory where C is a multiple of 4 up to 1024 and the buffers are 16-byte aligned; arguments and
+ * errors as in those calls. */
+lbm_status lbm_nn_relu_bias_backward(float* dy, const float* y, int64_t P, int32_t C, float* db, void* workspace,
+                                     int64_t workspace_bytes, void* stream);
+
 /* 2x2 average pooling [B][H][W][C] -> [B][H/2][W/2][C] and its gradient. */
 lbm_status lbm_nn_pool(const float* x, int32_t B, int32_t H, int32_t W, int32_t C, float* y, void* stream);
 lbm_status lbm_nn_pool_backward(const float* dy, int32_t B, int32_t H, int32_t W, int32_t C, float* dx, int32_t beta,

@@ -20,7 +20,7 @@
 // (two MMAs per tap; one with act_bf16), BF16 weights, FP32 accumulation.
 //
 // Pipeline (conv3_tc_kernel below): persistent CTAs, one per SM, with warp roles.
-// Producer warps copy the FP32 chunks a few steps ahead with cp.async and convert
+// Producer warps load the FP32 chunks a few steps ahead into registers and convert
 // them into the BF16 operand buffers; one warp issues the MMAs; four warps read the
 // accumulators (tcgen05.ld), add the bias, apply ReLU and store FP32 (or add into
 // the destination); one warp streams the weights when they are not resident.  The
@@ -39,8 +39,8 @@
 #ifndef LBM_CONV_TC_STAGES
 #define LBM_CONV_TC_STAGES 0    // BF16 operand buffers; 0 = three
 #endif
-#ifndef LBM_CONV_TC_RAWD
-#define LBM_CONV_TC_RAWD 3      // FP32 chunks in flight per producer thread
+#ifndef LBM_CONV_TC_DEPTH
+#define LBM_CONV_TC_DEPTH 3     // FP32 chunks in flight per producer thread (registers)
 #endif
 
 namespace {
@@ -130,11 +130,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
+// 16 lanes x 32 columns of an accumulator as matrix fragments: v[4 j + 2 h + e] is lane lane/4 + 8 h,
+// column 8 j + 2 (lane % 4) + e
+__device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, float (&v)[16])
 {
     uint32_t r[16];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
         "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
@@ -155,8 +157,7 @@ template <int BN, int MT, bool LO>
 struct TcShape {
     static constexpr int TH = 16, TW = 8 * MT;               // output block (MT tiles of 16 x 8)
     static constexpr int HWD = TW + 2, HP = (TH + 2) * HWD;  // halo block width, pixels
-    static constexpr int NQ = (HP * 4 + 255) / 256;          // 16-byte copies per producer thread per chunk
-    static constexpr int RAW_BYTES = HP * 64;                // one FP32 chunk of the halo block (16 channels)
+    static constexpr int NQ = (HP * 4 + 255) / 256;          // 16-byte loads per producer thread per chunk
     static constexpr int PLANE = HP * 16;                    // 8 channels of every halo pixel (BF16)
     static constexpr int A_HALF = 2 * PLANE;                 // one BF16 half of a 16-channel chunk
     static constexpr int A_BYTES = (LO ? 2 : 1) * A_HALF;
@@ -171,7 +172,7 @@ struct TcShape {
 };
 
 // warp roles
-constexpr int kProducerWarps = 8;       // warps 0-7: activations (cp.async FP32 -> BF16 hi / lo)
+constexpr int kProducerWarps = 8;       // warps 0-7: activations (FP32 -> BF16 hi / lo)
 constexpr int kEpilogueWarp0 = 8;       // warps 8-11: accumulator -> global (TMEM lanes 32 (w % 4) ..)
 constexpr int kMmaWarp = 12;            // warp 12: tensor-memory allocation; the MMA loop (elected lane issues)
 constexpr int kWeightWarp = 13;         // warp 13: weights per chunk when they are not resident
@@ -181,7 +182,6 @@ static_assert(kEpilogueWarp0 % 4 == 0 && kEpilogueWarp0 + 4 == kMmaWarp && kProd
 
 struct TcConf {
     int stages;     // BF16 operand buffers (and weight buffers when not resident)
-    int rawd;       // FP32 chunks in flight per producer thread
     int resident;   // the weights of all chunks stay in shared memory
 };
 
@@ -205,14 +205,6 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
     }
 }
 
-__device__ __forceinline__ void cp_async_wait_upto(int n)   // at most n of this thread's groups pending
-{
-    if (n <= 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
-    else if (n == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
-    else if (n == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
-    else asm volatile("cp.async.wait_group 3;" ::: "memory");
-}
-
 // Persistent, warp-specialised.  CTA b takes the output blocks b, b + gridDim.x, ...
 // (output channels of blockIdx.y) and walks their 16-channel chunks as one sequence
 // g = 0 .. G-1.  Barriers: full[s] (operands of the chunk in buffer s staged: one
@@ -220,7 +212,7 @@ __device__ __forceinline__ void cp_async_wait_upto(int n)   // at most n of this
 // read buffer s completed: tcgen05.commit), acc_full[b] (the MMAs of the block in
 // accumulator b completed), acc_empty[b] (the epilogue warps have read accumulator b:
 // one arrival per warp).
-// Shared memory: [BF16 operand buffers][FP32 chunk ring][weights].
+// Shared memory: [BF16 operand buffers][weights].
 template <int BN, int MT, bool LO>
 __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcConf cf)
 {
@@ -238,10 +230,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
     const int nchunk = Cin / 16;
     const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int G = my_tiles * nchunk;
-    const int stages = cf.stages, rawd = cf.rawd;
+    const int stages = cf.stages;
     uint8_t* const ring = smem;
-    uint8_t* const raw = smem + stages * S::A_BYTES;
-    uint8_t* const wts = raw + rawd * S::RAW_BYTES;
+    uint8_t* const wts = smem + stages * S::A_BYTES;
 
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -291,12 +282,14 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
     };
 
     if (warp < kProducerWarps) {
-        // ---- activations: FP32 chunk g + rawd copied while chunk g is converted ----
-        // pixel indices of this thread's halo elements in the block being copied, the same for
+        // ---- activations: the FP32 loads of chunk g + DEPTH are issued once chunk g is converted ----
+        constexpr int DEPTH = LBM_CONV_TC_DEPTH;
+        // pixel indices of this thread's halo elements in the block being loaded, the same for
         // every channel chunk of the block: full resolution, and halved for an x1 stored at half size
         int cached_t = -1;
         uint32_t pix_full[S::NQ], pix_half[S::NQ];
-        auto issue_raw = [&](int g) {
+        float4 v[DEPTH][S::NQ];
+        auto load = [&](int g, float4 (&u)[S::NQ]) {
             const int t = g / nchunk, ci0 = (g - t * nchunk) * 16;
             if (t != cached_t) {
                 int n, ty0, tx0;
@@ -313,93 +306,103 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
                 cached_t = t;
             }
             const bool from1 = ci0 < a.C1;
-            const float* base = from1 ? a.x1 + ci0 : a.x2 + (ci0 - a.C1);
+            const float* base = (from1 ? a.x1 + ci0 : a.x2 + (ci0 - a.C1)) + (tid & 3) * 4;
             const size_t cstride = (size_t)(from1 ? a.C1 : a.C2);
             const bool half = from1 && a.x1_half;          // nearest upsampling of a half-size x1
-            const uint32_t dst = smem_addr(raw + (g % rawd) * S::RAW_BYTES);
 #pragma unroll
-            for (int i = 0; i < S::NQ; ++i) {
-                const int q = tid + kProducers * i;
-                if (q < S::HP * 4)
-                    cp_async16(dst + q * 16, base + (size_t)(half ? pix_half[i] : pix_full[i]) * cstride + (q & 3) * 4);
-            }
+            for (int i = 0; i < S::NQ; ++i)
+                if (tid + kProducers * i < S::HP * 4)
+                    u[i] = __ldg(reinterpret_cast<const float4*>(base + (size_t)(half ? pix_half[i] : pix_full[i]) * cstride));
         };
-        for (int d = 0; d < rawd; ++d) {
-            if (d < G) issue_raw(d);
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        }
-        for (int g = 0; g < G; ++g) {
-            const int s = g % stages;
-            // (warp-uniform, so that the whole warp leaves together after an abort)
-            if (g >= stages &&
-                !__all_sync(0xffffffffu,
-                            wait_or_abort(smem_addr(&empty[s]), (uint32_t)((g / stages - 1) & 1), abort_v)))
-                break;
-            cp_async_wait_upto(rawd - 1);                  // this thread's copies of chunk g have landed
-            const uint8_t* src = raw + (g % rawd) * S::RAW_BYTES;
-            uint8_t* st = ring + s * S::A_BYTES;
 #pragma unroll
-            for (int i = 0; i < S::NQ; ++i) {
-                const int q = tid + kProducers * i;
-                if (q < S::HP * 4) {
-                    const int hp = q >> 2, c4 = q & 3;
-                    const float4 v = *reinterpret_cast<const float4*>(src + q * 16);
-                    const int off = (c4 >> 1) * S::PLANE + hp * 16 + (c4 & 1) * 8;
-                    const __nv_bfloat162 h01 = __floats2bfloat162_rn(v.x, v.y), h23 = __floats2bfloat162_rn(v.z, v.w);
-                    *reinterpret_cast<uint2*>(st + off) = make_uint2(bf16x2_bits(h01), bf16x2_bits(h23));
-                    if constexpr (LO) {
-                        const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
-                        const __nv_bfloat162 l01 = __floats2bfloat162_rn(v.x - f01.x, v.y - f01.y);
-                        const __nv_bfloat162 l23 = __floats2bfloat162_rn(v.z - f23.x, v.w - f23.y);
-                        *reinterpret_cast<uint2*>(st + S::A_HALF + off) =
-                            make_uint2(bf16x2_bits(l01), bf16x2_bits(l23));
+        for (int d = 0; d < DEPTH; ++d)
+            if (d < G) load(d, v[d]);
+        bool ok = true;
+        for (int g0 = 0; g0 < G && ok; g0 += DEPTH) {
+#pragma unroll
+            for (int d = 0; d < DEPTH; ++d) {
+                const int g = g0 + d;
+                if (g >= G || !ok) break;
+                const int s = g % stages;
+                // (warp-uniform, so that the whole warp leaves together after an abort)
+                if (g >= stages)
+                    ok = __all_sync(0xffffffffu,
+                                    wait_or_abort(smem_addr(&empty[s]), (uint32_t)((g / stages - 1) & 1), abort_v));
+                if (!ok) break;
+                uint8_t* st = ring + s * S::A_BYTES + ((tid & 3) >> 1) * S::PLANE + (tid & 1) * 8;
+#pragma unroll
+                for (int i = 0; i < S::NQ; ++i) {
+                    const int q = tid + kProducers * i;
+                    if (q < S::HP * 4) {
+                        const float4 u = v[d][i];
+                        const int off = (q >> 2) * 16;
+                        const __nv_bfloat162 h01 = __floats2bfloat162_rn(u.x, u.y), h23 = __floats2bfloat162_rn(u.z, u.w);
+                        *reinterpret_cast<uint2*>(st + off) = make_uint2(bf16x2_bits(h01), bf16x2_bits(h23));
+                        if constexpr (LO) {
+                            const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+                            const __nv_bfloat162 l01 = __floats2bfloat162_rn(u.x - f01.x, u.y - f01.y);
+                            const __nv_bfloat162 l23 = __floats2bfloat162_rn(u.z - f23.x, u.w - f23.y);
+                            *reinterpret_cast<uint2*>(st + S::A_HALF + off) =
+                                make_uint2(bf16x2_bits(l01), bf16x2_bits(l23));
+                        }
                     }
                 }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor core
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_addr(&full[s]));              // for the whole warp
+                if (g + DEPTH < G) load(g + DEPTH, v[d]);
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor core
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_addr(&full[s]));              // for the whole warp
-            if (g + rawd < G) issue_raw(g + rawd);          // into the ring slot just converted (own elements)
-            asm volatile("cp.async.commit_group;" ::: "memory");
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
     } else if (warp < kEpilogueWarp0 + 4) {
         // ---- epilogue: accumulator of block t -> bias, ReLU, FP32 stores ----
-        const int q = warp & 3;
-        const int m = q * 32 + lane;                        // pixel of a 128-pixel tile = TMEM lane
+        // Read as matrix fragments (16 pixels x 32 channels per load): four lanes then hold 8 adjacent
+        // channels of a pixel and a store covers whole 32-byte sectors.  One pixel per lane stored
+        // 16-byte pieces of 32 different lines at a time, every sector twice.
+        const int q = warp & 3, gr = lane >> 2, t4 = lane & 3;
+        float2 bias[BN / 8];
+#pragma unroll
+        for (int j = 0; j < BN / 8; ++j)
+            bias[j] = a.bias ? __ldg(reinterpret_cast<const float2*>(a.bias + co0 + 8 * j + 2 * t4)) : make_float2(0.f, 0.f);
         for (int t = 0; t < my_tiles; ++t) {
             const bool ok = wait_or_abort(smem_addr(&acc_full[t & 1]), (uint32_t)((t >> 1) & 1), abort_v);
             if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after();
             int n, ty0, tx0;
             tile_of(t, n, ty0, tx0);
-#pragma unroll
-            for (int j = 0; j < MT; ++j) {
-                const int oy = ty0 + (m >> 3), ox = tx0 + 8 * j + (m & 7);
-                const long long p = ((long long)n * a.H + oy) * a.W + ox;
-                const uint32_t col0 = (uint32_t)((t & 1) * S::ACC + j * BN);
 #pragma unroll 1
-                for (int cc = 0; cc < BN; cc += 16) {
-                    float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + col0 + (uint32_t)cc, v);
-                    const int co = co0 + cc;                // 16 channels, all in y1 or all in y2
-                    float* dst = co < a.Co1 ? a.y1 + p * a.Co1 + co : a.y2 + p * (a.Cout - a.Co1) + (co - a.Co1);
+            for (int jh = 0; jh < 2 * MT; ++jh) {                       // tile, upper or lower 16 TMEM lanes
+                const int j = jh >> 1, hh = jh & 1;
+                const uint32_t row = tmem + ((uint32_t)(q * 32 + hh * 16) << 16) + (uint32_t)((t & 1) * S::ACC + j * BN);
+                // TMEM lane m = pixel (m >> 3, m & 7) of the tile
+                const long long p = ((long long)n * a.H + ty0 + q * 4 + hh * 2) * a.W + tx0 + 8 * j + gr;
 #pragma unroll
-                    for (int e = 0; e < 16; e += 4) {
-                        float4 r = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-                        if (a.bias) {
-                            const float4 b = __ldg(reinterpret_cast<const float4*>(a.bias + co + e));
-                            r.x += b.x; r.y += b.y; r.z += b.z; r.w += b.w;
+                for (int cc = 0; cc < BN; cc += 32) {
+                    float v[16];
+                    tmem_ld_16x32(row + (uint32_t)cc, v);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const long long ph = p + h * a.W;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int co = co0 + cc + 8 * k;            // 8 channels, all in y1 or all in y2
+                            float* dst = (co < a.Co1 ? a.y1 + ph * a.Co1 + co : a.y2 + ph * (a.Cout - a.Co1) + (co - a.Co1)) +
+                                         2 * t4;
+                            float2 r = make_float2(v[4 * k + 2 * h], v[4 * k + 2 * h + 1]);
+                            if (a.bias) {
+                                r.x += bias[cc / 8 + k].x;
+                                r.y += bias[cc / 8 + k].y;
+                            }
+                            if (a.relu) {
+                                r.x = fmaxf(r.x, 0.f);
+                                r.y = fmaxf(r.y, 0.f);
+                            }
+                            if (a.beta) {
+                                const float2 o = *reinterpret_cast<const float2*>(dst);
+                                r.x += o.x;
+                                r.y += o.y;
+                            }
+                            *reinterpret_cast<float2*>(dst) = r;
                         }
-                        if (a.relu) {
-                            r.x = fmaxf(r.x, 0.f); r.y = fmaxf(r.y, 0.f); r.z = fmaxf(r.z, 0.f); r.w = fmaxf(r.w, 0.f);
-                        }
-                        float4* d4 = reinterpret_cast<float4*>(dst + e);
-                        if (a.beta) {
-                            const float4 o = *d4;
-                            r.x += o.x; r.y += o.y; r.z += o.z; r.w += o.w;
-                        }
-                        *d4 = r;
                     }
                 }
             }
@@ -527,19 +530,17 @@ bool launch_variant(const ConvTcArgs& a, cudaStream_t s, int stages, int slot)
         v.ready = 1;
     }
     const int nchunk = (a.C1 + a.C2) / 16;
-    TcConf cf{stages > 0 ? stages : 3, LBM_CONV_TC_RAWD, 1};
-    if (cf.stages < 2 || cf.stages > kMaxStages || cf.rawd < 1 || cf.rawd > 4) return false;
-    // largest configuration that fits: resident weights first, then fewer FP32 chunks in
-    // flight, then fewer operand buffers
+    TcConf cf{stages > 0 ? stages : 3, 1};
+    if (cf.stages < 2 || cf.stages > kMaxStages) return false;
+    // largest configuration that fits: resident weights first, then fewer operand buffers
     long long smem = 0;
     for (;;) {
-        const long long base = (long long)cf.stages * S::A_BYTES + (long long)cf.rawd * S::RAW_BYTES;
+        const long long base = (long long)cf.stages * S::A_BYTES;
         const long long res = base + (long long)nchunk * S::B_BYTES;
         const long long str = base + (long long)cf.stages * S::B_BYTES;
         if (res <= kSmemLimit) { cf.resident = 1; smem = res; break; }
         if (str <= kSmemLimit) { cf.resident = 0; smem = str; break; }
-        if (cf.rawd > 2) --cf.rawd;
-        else if (cf.stages > 2) --cf.stages;
+        if (cf.stages > 2) --cf.stages;
         else return false;
     }
     const int per_sm = ctas_per_sm(v, dev, smem);

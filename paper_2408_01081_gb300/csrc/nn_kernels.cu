@@ -220,6 +220,82 @@ __global__ void __launch_bounds__(256) conv_fwd_kernel(ConvArgs a)
 }
 
 // ---------------------------------------------------------------------------
+// 1x1 convolution 32 -> 32 channels (the network's output layer).  Bound by memory (256 bytes per
+// pixel): a warp takes 16 pixels at a time, its MMA fragments come straight from global memory (8 rows
+// of 32 bytes per load, whole sectors) and leave the same way; the weights stay in registers.  Same
+// products in the same order as conv_fwd_kernel, whose staged tiles of 128 pixels left the memory
+// idle: 16 x 256 x 256 pixels 81 us before, 46 us so.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) conv1_stream_kernel(ConvArgs a)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+    const long long P = (long long)a.B * a.H * a.W, ntile = (P + 15) / 16;
+    const long long nwarp = (long long)gridDim.x * (blockDim.x >> 5);
+    uint32_t fb[2][4][2];
+    float2 bias[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                fb[k][j][h] = *reinterpret_cast<const uint32_t*>(a.w + (j * 8 + g) * 32 + 16 * k + 8 * h + 2 * t4);
+        bias[j] = a.bias ? make_float2(a.bias[j * 8 + 2 * t4], a.bias[j * 8 + 2 * t4 + 1]) : make_float2(0.f, 0.f);
+    }
+    for (long long tile = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); tile < ntile; tile += nwarp) {
+        const long long p0 = tile * 16 + g;
+        float2 v[2][4];                          // [pixel p0, p0 + 8][channels 8 q + 2 t4, + 1]
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                v[h][q] = p0 + 8 * h < P
+                              ? __ldg(reinterpret_cast<const float2*>(a.x1 + (p0 + 8 * h) * 32 + 8 * q + 2 * t4))
+                              : make_float2(0.f, 0.f);
+        float acc[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            uint32_t fh[4], fl[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {        // rows g, g + 8; columns 2 t4 and 8 + 2 t4
+                const float2 u = v[q & 1][2 * k + (q >> 1)];
+                const __nv_bfloat162 hi = __floats2bfloat162_rn(u.x, u.y);
+                const float2 f = __bfloat1622float2(hi);
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(u.x - f.x, u.y - f.y);
+                fh[q] = *reinterpret_cast<const uint32_t*>(&hi);
+                fl[q] = *reinterpret_cast<const uint32_t*>(&lo);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                mma_bf16(acc[j], fh, fb[k][j]);
+                if (!a.act_bf16) mma_bf16(acc[j], fl, fb[k][j]);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (p0 + 8 * h >= P) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float2 r = make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
+                if (a.bias) {
+                    r.x += bias[j].x;
+                    r.y += bias[j].y;
+                }
+                if (a.relu) {
+                    r.x = fmaxf(r.x, 0.f);
+                    r.y = fmaxf(r.y, 0.f);
+                }
+                *reinterpret_cast<float2*>(a.y1 + (p0 + 8 * h) * 32 + 8 * j + 2 * t4) = r;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // 3x3 convolution on an 8 x 16 pixel tile (H >= 8, W >= 16): the input tile with
 // its one-pixel halo (10 x 18 pixels) is staged once per 32-channel chunk as
 // BF16 hi / lo, the weights of all nine taps once per chunk, and every tap reads
@@ -667,14 +743,28 @@ __global__ void __launch_bounds__(G3THREADS, 2) conv_wgrad3_tile_kernel(Wgrad3Ar
         }
 }
 
-// sum the split partials in order into dW (FP32)
-__global__ void sum_splits_kernel(const float* __restrict__ partial, int splits, long long n, float* __restrict__ out,
-                                  int beta)
+// Sum the split partials into dW (FP32) in a fixed order.  A block takes 32 consecutive elements;
+// its warps take every 8th split each (a 128-byte line per load) and their sums are added in warp
+// order.  One thread per element walked all splits before: 32 -> 32 channels has 9216 elements and
+// up to 600 splits, 36 blocks of dependent loads, 55 us for 19 MB; 6 us so.
+__global__ void __launch_bounds__(256) sum_splits_kernel(const float* __restrict__ partial, int splits, long long n,
+                                                         float* __restrict__ out, int beta)
 {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int k = 0; k < splits; ++k) s += partial[(long long)k * n + i];
-        out[i] = beta ? out[i] + s : s;
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long i = blockIdx.x * 32LL + lane;
+    float s = 0.f;
+    if (i < n) {
+#pragma unroll 8
+        for (int k = warp; k < splits; k += 8) s += partial[(long long)k * n + i];
+    }
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && i < n) {
+        float t = red[0][lane];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) t += red[w][lane];
+        out[i] = beta ? out[i] + t : t;
     }
 }
 
@@ -713,6 +803,52 @@ __global__ void bias_grad_partial_kernel(const float* __restrict__ dy, long long
             partial[(long long)blockIdx.x * C + c0 + t] = acc;
         }
         __syncthreads();
+    }
+}
+
+// The ReLU mask and the bias gradient in one pass over dy and y: dy[p][c] = 0 where y[p][c] <= 0, and
+// the block's partial sum of the masked dy per channel (pass 1 of the bias gradient).  Bound by memory:
+// the mask alone is 12 bytes per element, the sums came in a second pass of 4 (29 + 28 us for 8 x 256 x
+// 256 x 32, 30 us so).  A thread keeps four adjacent channels (C a multiple of 4, at most 1024).
+__global__ void __launch_bounds__(256) relu_bias_partial_kernel(float4* __restrict__ dy, const float4* __restrict__ y,
+                                                                long long P, int C4, long long ppb,
+                                                                float4* __restrict__ partial)
+{
+    __shared__ float4 red[256];
+    const int t = threadIdx.x;
+    const int rows = 256 / C4;
+    const int c = t % C4, r = t / C4;
+    const long long p0 = blockIdx.x * ppb, p1 = min(P, p0 + ppb);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < rows) {
+#pragma unroll 4
+        for (long long p = p0 + r; p < p1; p += rows) {
+            const long long i = p * C4 + c;
+            const float4 a = y[i];
+            float4 v = dy[i];
+            if (!(a.x > 0.f)) v.x = 0.f;
+            if (!(a.y > 0.f)) v.y = 0.f;
+            if (!(a.z > 0.f)) v.z = 0.f;
+            if (!(a.w > 0.f)) v.w = 0.f;
+            dy[i] = v;
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    }
+    red[t] = s;
+    __syncthreads();
+    if (t < C4) {
+        float4 a = red[t];
+        for (int q = 1; q < rows; ++q) {
+            const float4 b = red[q * C4 + t];
+            a.x += b.x;
+            a.y += b.y;
+            a.z += b.z;
+            a.w += b.w;
+        }
+        partial[(long long)blockIdx.x * C4 + t] = a;
     }
 }
 
@@ -917,34 +1053,55 @@ __global__ void to_bf16_kernel(const float* __restrict__ x, long long n, __nv_bf
         y[i] = __float2bfloat16_rn(x[i]);
 }
 
+// (float)(u / s) given r = 1 / s rounded, without an FP64 division where the product decides: q = u r is
+// within two units in the last place of u / s, so both round to the same FP32 value unless q lies that
+// close to the middle between two of them (the 29 bits dropped near 2^28) or outside FP32's normal range.
+__device__ __forceinline__ float div_to_f32(double u, double s, double r)
+{
+    const double q = u * r, m = fabs(q);
+    const int low = (int)(__double2loint(q) & 0x1FFFFFFF) - 0x10000000;
+    if (m >= 2.4e-38 && m < 1.7e38 && (low > 8 || low < -8)) return (float)q;
+    return (float)(u / s);
+}
+
 // network input: U fields [B][nf][H][W] (FP64, field-major per sample) scaled by 1/scale[c], plus a
-// constant channel per sample, into [B][H][W][C] FP32 with zero padding channels
-__global__ void pack_input_kernel(const double* __restrict__ U, long long sample_stride, int nf, const double* __restrict__ scale,
-                                  const float* __restrict__ extra, int B, int H, int W, int C, float* __restrict__ x)
+// constant channel per sample, into [B][H][W][C] FP32 with zero padding channels.  nf FP64 divisions per
+// pixel bounded it (16 x 256 x 256, 5 fields: 90 us before, 69 us so, at 26 us of memory traffic).
+__global__ void __launch_bounds__(256) pack_input_kernel(const double* __restrict__ U, long long sample_stride, int nf,
+                                                         const double* __restrict__ scale,
+                                                         const float* __restrict__ extra, int B, int H, int W, int C,
+                                                         float* __restrict__ x)
 {
     // one thread per pixel: the nf fields (coalesced across the warp), the extra
     // channel, zeros up to C; 16-byte stores when C is a multiple of 4
+    __shared__ double rs[64];
+    for (int c = threadIdx.x; c < nf && c < 64; c += blockDim.x) {
+        const double s = scale[c], r = 1.0 / s;
+        rs[c] = fabs(s) >= 1e-290 && fabs(s) <= 1e290 ? r : 0.0;    // 0: every value takes the division
+    }
+    __syncthreads();
     const long long HW = (long long)H * W;
     const long long npix = (long long)B * HW;
     for (long long pix = blockIdx.x * (long long)blockDim.x + threadIdx.x; pix < npix;
          pix += (long long)gridDim.x * blockDim.x) {
         const long long b = pix / HW, q = pix - b * HW;
         float* dst = x + pix * C;
+        const auto value = [&](int c) {
+            if (c >= nf) return c == nf && extra ? extra[b] : 0.f;
+            const double u = U[b * sample_stride + c * HW + q];
+            const double r = c < 64 ? rs[c] : 0.0;
+            if (u == 0.0 && r != 0.0) return (float)(u * r);        // the sign of a zero
+            return div_to_f32(u, scale[c], r);
+        };
         if ((C & 3) == 0) {
             for (int c0 = 0; c0 < C; c0 += 4) {
                 float v[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int c = c0 + e;
-                    v[e] = c < nf ? (float)(U[b * sample_stride + c * HW + q] / scale[c])
-                                  : (c == nf && extra) ? extra[b] : 0.f;
-                }
+                for (int e = 0; e < 4; ++e) v[e] = value(c0 + e);
                 *reinterpret_cast<float4*>(dst + c0) = make_float4(v[0], v[1], v[2], v[3]);
             }
         } else {
-            for (int c = 0; c < C; ++c)
-                dst[c] = c < nf ? (float)(U[b * sample_stride + c * HW + q] / scale[c])
-                                : (c == nf && extra) ? extra[b] : 0.f;
+            for (int c = 0; c < C; ++c) dst[c] = value(c);
         }
     }
 }
@@ -1123,6 +1280,13 @@ lbm_status lbm_nn_conv_forward(const float* x1, int32_t C1, const float* x2, int
 #undef LBM_CONV3
         return launch_status();
     }
+    // one 32-channel input and output, written whole; 8-byte accesses
+    if (KS == 1 && C1 == 32 && C2 == 0 && Cout == 32 && Co1 == 32 && !(flags & LBM_NN_ACCUMULATE) &&
+        !(flags & LBM_NN_X1_HALF) && ((((uintptr_t)x1 | (uintptr_t)y1) & 7) | ((uintptr_t)w_bf16 & 3)) == 0) {
+        const long long blocks = (P + 127) / 128;
+        conv1_stream_kernel<<<(unsigned)(blocks < 152 * 6 ? blocks : 152 * 6), 256, 0, s>>>(a);
+        return launch_status();
+    }
     const int BN = Cout >= 64 ? 64 : (Cout >= 32 ? 32 : 16);
     dim3 grid((unsigned)((P + CBM - 1) / CBM), (unsigned)((Cout + BN - 1) / BN));
     if (KS == 3) {
@@ -1192,7 +1356,7 @@ lbm_status lbm_nn_conv_backward_weight(const float* dy, int32_t Cout, const floa
         conv_wgrad3_tile_kernel<<<dim3((unsigned)(Cout / 32), (unsigned)(Cin / 32), (unsigned)splits), G3THREADS,
                                   conv_wgrad3_smem_bytes(), st>>>(g3);
         const long long n = (long long)Cout * 9 * Cin;
-        sum_splits_kernel<<<grid_for(n), 256, 0, st>>>(static_cast<const float*>(workspace), splits, n, dw, beta);
+        sum_splits_kernel<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(static_cast<const float*>(workspace), splits, n, dw, beta);
         g_conv_launches[2].fetch_add(1, std::memory_order_relaxed);
         return launch_status();
     }
@@ -1206,7 +1370,7 @@ lbm_status lbm_nn_conv_backward_weight(const float* dy, int32_t Cout, const floa
     dim3 grid((unsigned)((Cout + 63) / 64), (unsigned)(KS * KS * ((Cin + 63) / 64)), (unsigned)splits);
     conv_wgrad_kernel<<<grid, 256, 0, s>>>(a);
     const long long n = (long long)Cout * KS * KS * Cin;
-    sum_splits_kernel<<<grid_for(n), 256, 0, s>>>(static_cast<const float*>(workspace), splits, n, dw, beta);
+    sum_splits_kernel<<<(unsigned)((n + 31) / 32), 256, 0, s>>>(static_cast<const float*>(workspace), splits, n, dw, beta);
     return launch_status();
 }
 
@@ -1227,6 +1391,23 @@ lbm_status lbm_nn_bias_grad(const float* dy, int64_t P, int32_t C, float* db, vo
     float* part = static_cast<float*>(workspace);
     bias_grad_partial_kernel<<<nblk, 256, 0, s>>>(dy, P, C, ppb, part);
     bias_grad_finish_kernel<<<C, 256, 0, s>>>(part, nblk, C, db);
+    return launch_status();
+}
+
+lbm_status lbm_nn_relu_bias_backward(float* dy, const float* y, int64_t P, int32_t C, float* db, void* workspace,
+                                     int64_t workspace_bytes, void* stream)
+{
+    if (!dy || !y || !db || !workspace || P <= 0 || C <= 0) return LBM_ERR_ARG;
+    if (workspace_bytes < lbm_nn_bias_grad_workspace_bytes(P, C)) return LBM_ERR_ARG;
+    if (C % 4 || C > 1024 || (((uintptr_t)dy | (uintptr_t)y | (uintptr_t)workspace) & 15)) {   // two passes
+        const lbm_status st = lbm_nn_relu_backward(dy, y, P * C, stream);
+        return st != LBM_OK ? st : lbm_nn_bias_grad(dy, P, C, db, workspace, workspace_bytes, stream);
+    }
+    const int nblk = bias_grad_blocks(P, C);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    relu_bias_partial_kernel<<<nblk, 256, 0, s>>>(reinterpret_cast<float4*>(dy), reinterpret_cast<const float4*>(y), P,
+                                                  C / 4, bias_grad_ppb(P, C), static_cast<float4*>(workspace));
+    bias_grad_finish_kernel<<<C, 256, 0, s>>>(static_cast<const float*>(workspace), nblk, C, db);
     return launch_status();
 }
 

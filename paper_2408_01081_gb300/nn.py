@@ -10,7 +10,7 @@ import ctypes
 from . import lbm as _lbm
 
 EXPORTS = ["lbm_nn_conv_forward", "lbm_nn_check", "lbm_nn_conv_counts", "lbm_nn_wgrad_workspace_bytes", "lbm_nn_conv_backward_weight",
-           "lbm_nn_bias_grad_workspace_bytes", "lbm_nn_bias_grad",
+           "lbm_nn_bias_grad_workspace_bytes", "lbm_nn_bias_grad", "lbm_nn_relu_bias_backward",
            "lbm_nn_weight_flip", "lbm_nn_relu_backward", "lbm_nn_pool", "lbm_nn_pool_backward", "lbm_nn_upsample",
            "lbm_nn_upsample_backward", "lbm_nn_mse", "lbm_nn_adam", "lbm_nn_to_bf16", "lbm_nn_pack_input",
            "lbm_nn_pack_target", "lbm_nn_residual_output", "lbm_nn_gradient"]
@@ -31,6 +31,7 @@ def _lib():
             "lbm_nn_conv_backward_weight": [vp, i32, vp, i32, vp, i32, i32, i32, i32, i32, vp, i32, vp, i64, vp],
             "lbm_nn_bias_grad_workspace_bytes": [i64, i32],
             "lbm_nn_bias_grad": [vp, i64, i32, vp, vp, i64, vp],
+            "lbm_nn_relu_bias_backward": [vp, vp, i64, i32, vp, vp, i64, vp],
             "lbm_nn_weight_flip": [vp, i32, i32, i32, vp, vp],
             "lbm_nn_relu_backward": [vp, vp, i64, vp],
             "lbm_nn_pool": [vp, i32, i32, i32, i32, vp, vp],
@@ -123,6 +124,13 @@ def bias_grad_workspace_bytes(P, C) -> int:
 def bias_grad(dy, P, C, db, workspace):
     _ok("lbm_nn_bias_grad", _lib().lbm_nn_bias_grad(_p(dy), P, C, _p(db), _p(workspace),
                                                     workspace.numel() * workspace.element_size(), _s()))
+
+
+def relu_bias_backward(dy, y, P, C, db, workspace):
+    """relu_backward(dy, y), then bias_grad(dy) into db, in one pass over the memory."""
+    _ok("lbm_nn_relu_bias_backward",
+        _lib().lbm_nn_relu_bias_backward(_p(dy), _p(y), P, C, _p(db), _p(workspace),
+                                         workspace.numel() * workspace.element_size(), _s()))
 
 
 def weight_flip(w_bf16, Cout, Cin, KS, wt_bf16):

@@ -63,11 +63,15 @@ class Conv:
     def backward(self, dy, y, x1, x2, B, H, W, dx1, dx2, workspace, need_dx=True, x1_half=False):
         """dy: gradient w.r.t. this layer's output (overwritten by the ReLU mask); with x1_half
         the data gradient dx1 is at full resolution (the caller folds it back to (H/2, W/2))."""
-        if self.relu:
+        fused = self.relu and dy.numel() == B * H * W * self.cout
+        if fused:
+            K.relu_bias_backward(dy, y, B * H * W, self.cout, self.gb, workspace)
+        elif self.relu:
             K.relu_backward(dy, y)
         K.conv_backward_weight(dy, self.cout, x1, self.cin1, x2, self.cin2, B, H, W, self.ks, self.gw, workspace,
                                x1_half=x1_half)
-        K.bias_grad(dy, B * H * W, self.cout, self.gb, workspace)
+        if not fused:
+            K.bias_grad(dy, B * H * W, self.cout, self.gb, workspace)
         if need_dx:
             K.weight_flip(self.wb, self.cout, self.cin1 + self.cin2, self.ks, self.wt)
             K.conv_forward(dy, self.cout, None, 0, self.wt, None, dx1, self.cin1, dx2, self.cin1 + self.cin2,

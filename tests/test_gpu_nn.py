@@ -355,3 +355,57 @@ def test_conv_half_resolution_input_and_bf16_activations(lbm, H, W, KS):
     K.conv_backward_weight(_t(dy), Cout, _t(xc), C1, _t(x2), C2, B, H, W, KS, dwh, ws, x1_half=True)
     K.conv_backward_weight(_t(dy), Cout, _t(xu), C1, _t(x2), C2, B, H, W, KS, dwf, ws)
     torch.testing.assert_close(dwh, dwf, rtol=0, atol=0)
+
+
+@pytest.mark.parametrize("P,C", [(1, 4), (100, 32), (70001, 64), (513, 1024), (300, 6), (77, 1028)])
+def test_relu_mask_and_bias_gradient_in_one_pass(lbm, P, C):
+    """One block to many, one row of channels per block at 1024, the two-pass forms beyond (C not a
+    multiple of 4 or above 1024); NaN in y masks.  The masked gradient is the input's words or zero."""
+    import torch
+    from paper_2408_01081_gb300 import nn as K
+    y = torch.randn((P, C), dtype=torch.float32, device="cuda")
+    y[P // 2, 0] = float("nan")
+    dy = torch.randn((P, C), dtype=torch.float32, device="cuda")
+    masked = torch.where(y > 0, dy, torch.zeros_like(dy))
+    db = torch.empty(C, dtype=torch.float32, device="cuda")
+    ws = torch.empty(K.bias_grad_workspace_bytes(P, C) // 4 + 4, dtype=torch.float32, device="cuda")
+    K.relu_bias_backward(dy, y, P, C, db, ws)
+    assert torch.equal(dy, masked)
+    ref = masked.double().sum(0)
+    assert torch.max(torch.abs(db.double() - ref)).item() < 1e-5 * max(1.0, P ** 0.5)
+
+
+@pytest.mark.parametrize("B,H,W,relu,bias,act_bf16", [(1, 1, 1, False, True, False), (3, 2, 4, True, True, False),
+                                                       (1, 1, 8, False, False, True), (5, 64, 64, False, True, False)])
+def test_conv1_streamed(lbm, B, H, W, relu, bias, act_bf16):
+    """1x1, 32 -> 32 channels: part of a 16-pixel tile, several tiles, more tiles than warps; the same
+    words as the staged kernel, which accumulation (onto zeros: an exact addition) selects."""
+    import torch
+    from paper_2408_01081_gb300 import nn as K
+    x = torch.randn((B, H, W, 32), dtype=torch.float32, device="cuda")
+    w = _wb(RNG.standard_normal((32, 1, 1, 32)))
+    b = torch.randn(32, dtype=torch.float32, device="cuda") if bias else None
+    y, z = torch.full_like(x, 7.0), torch.zeros_like(x)
+    for out, beta in ((y, False), (z, True)):
+        K.conv_forward(x, 32, None, 0, w, b, out, 32, None, 32, B, H, W, 1, relu=relu, act_bf16=act_bf16, beta=beta)
+    assert torch.equal(y, z)
+
+
+def test_pack_input_rounds_like_the_division(lbm):
+    """Quotients next to the middle between two FP32 numbers, zeros of both signs, values beyond FP32's
+    normal range, infinities and NaN, scales at FP64's ends: the words of float(u / scale)."""
+    import torch
+    from paper_2408_01081_gb300 import nn as K
+    H, W, nf = 64, 64, 5
+    n = H * W
+    scale = torch.tensor([0.1, 3.0, 1e-300, 1e-3 / 3.0, 1.0], dtype=torch.float64, device="cuda")
+    f = torch.rand((nf, n), dtype=torch.float32, device="cuda").double() + 0.5
+    mid = f + 2.0 ** -25                                       # f in [0.5, 1): its spacing is 2^-24
+    U = mid * scale[:, None] * (1.0 + 2.0 ** -52 * torch.randint(-3, 4, (nf, n), device="cuda").double())
+    U[:, :8] = torch.tensor([0.0, -0.0, float("inf"), float("nan"), 1e-41, -3e-46, 1e39, 5e-324], device="cuda").double()
+    x = torch.empty((1, H, W, 32), dtype=torch.float32, device="cuda")
+    K.pack_input(U, nf * n, nf, scale, torch.ones(1, device="cuda"), 1, H, W, 32, x)
+    ref = (U / scale[:, None]).float().T.reshape(1, H, W, nf)
+    assert torch.equal(x[..., :nf].contiguous().view(torch.int32)[~ref.isnan()], ref.contiguous().view(torch.int32)[~ref.isnan()])
+    assert torch.equal(x[..., :nf].isnan(), ref.isnan())
+    assert torch.equal(x[..., nf], torch.ones_like(x[..., nf])) and not x[..., nf + 1:].any()
