@@ -12,6 +12,7 @@
 
 #include "lbm.h"
 #include "lbm_dispatch.h"
+#include "nn_conv_tc.h"
 
 using lbmh::KindOps;
 using lbmh::encode_rows_map;
@@ -128,6 +129,21 @@ EncodeTiledFn encode_tiled()
 }  // namespace
 
 namespace lbmh {
+
+// 3D map of 3x3 convolution weights [cout][9][cin] in 16-bit words: x = input channel, y = output
+// channel, z = tap; box {16, box_co, 9} with the 32-byte swizzle
+bool encode_conv3_weights_map(CUtensorMap* m, const void* w, int cin, int cout, int box_co)
+{
+    EncodeTiledFn fn = encode_tiled();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)cin, (cuuint64_t)cout, 9u};
+    const cuuint64_t strides[2] = {(cuuint64_t)cin * 18, (cuuint64_t)cin * 2};
+    const cuuint32_t box[3] = {16u, (cuuint32_t)box_co, 9u};
+    const cuuint32_t estr[3] = {1u, 1u, 1u};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(w), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 // 3D map of a lattice buffer: x = column (extent nx), y = row (extent ny), z = plane
 // (extent nplanes); box {box_w, 1, nplanes}, out-of-range elements read as zero

@@ -13,8 +13,9 @@
 // descriptor into that same block, started dy halo rows and dx pixels further on,
 // with the stride between 8-row groups (SBO) = one halo row and between the two K
 // halves (LBO) = one plane; no im2col copy is made.  The weights of a chunk's nine
-// taps are copied (cp.async) into the same layout with output channels as rows;
-// they stay resident for the whole kernel when all chunks fit in shared memory.
+// taps arrive by one tensor copy as rows of 32 bytes (an output channel's 16 input
+// channels) in the 32-byte swizzled layout; they stay resident for the whole kernel
+// when all chunks fit in shared memory.
 //
 // Precision is that of the mma.sync kernels: activations split into BF16 hi + lo
 // (two MMAs per tap; one with act_bf16), BF16 weights, FP32 accumulation.
@@ -34,6 +35,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lbm_tma.cuh"
 #include "nn_conv_tc.h"
 
 #ifndef LBM_CONV_TC_STAGES
@@ -54,14 +56,13 @@ constexpr int kTmemColumns = 512;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// shared-memory matrix descriptor: start address, leading-dimension (K) byte offset
-// and stride-dimension (M / N) byte offset, each >> 4 in 14 bits; descriptor
-// version 1 at bits 46-47; base offset 0, no swizzle (bits 61-63 = 0)
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
-{
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
+// Shared-memory matrix descriptor in two words.  Low: start address and leading-dimension (K) byte
+// offset, each >> 4 in 14 bits; high: stride-dimension (M / N) byte offset >> 4 in 14 bits, descriptor
+// version 1 at bits 46-47, swizzle mode at bits 61-63.  Addresses stay below 2^14 * 16 bytes, so a
+// descriptor further on is the low word plus the distance >> 4.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
+constexpr uint32_t kNoSwizzle = 0u, kSwizzle32 = 6u;
+constexpr uint32_t desc_hi(uint32_t sbo, uint32_t swizzle) { return (sbo >> 4) | (1u << 14) | (swizzle << 29); }
 
 // instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), A and B BF16
 // (bits 7-9 = 1, 10-12 = 1), no negation, both K-major (bits 15, 16 = 0), dense,
@@ -74,16 +75,18 @@ constexpr uint32_t idesc_bf16_f32(int M, int N)
 // D (+)= A B^T with A, B in shared memory (descriptors) and D in tensor memory.  Executed by a
 // whole converged warp: one lane (elect.sync) issues the instruction, so that the operands can
 // stay in warp-uniform registers.
-__device__ __forceinline__ void mma_bf16_ss_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                  uint32_t accumulate)
+template <uint32_t A_HI, uint32_t B_HI, uint32_t IDESC>
+__device__ __forceinline__ void mma_bf16_ss_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p, e;\n\t"
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\t"
         "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "setp.ne.b32 p, %3, 0;\n\t"
+        "mov.b64 da, {%1, %4};\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, p;\n\t"
         "}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "r"(a_lo), "r"(b_lo), "r"(accumulate), "n"(A_HI), "n"(B_HI), "r"(IDESC)
         : "memory");
 }
 
@@ -131,54 +134,58 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // 16 lanes x 32 columns of an accumulator as matrix fragments: v[4 j + 2 h + e] is lane lane/4 + 8 h,
-// column 8 j + 2 (lane % 4) + e
-__device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, float (&v)[16])
+// column 8 j + 2 (lane % 4) + e.  Two of them per wait.
+__device__ __forceinline__ void tmem_ld_16x32_pair(uint32_t taddr0, uint32_t taddr1, uint32_t (&r)[2][16])
 {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    for (int i = 0; i < 2; ++i)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[i][0]), "=r"(r[i][1]), "=r"(r[i][2]), "=r"(r[i][3]), "=r"(r[i][4]), "=r"(r[i][5]), "=r"(r[i][6]),
+              "=r"(r[i][7]), "=r"(r[i][8]), "=r"(r[i][9]), "=r"(r[i][10]), "=r"(r[i][11]), "=r"(r[i][12]),
+              "=r"(r[i][13]), "=r"(r[i][14]), "=r"(r[i][15])
+            : "r"(i ? taddr1 : taddr0)
+            : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 2; ++i)          // uses stay behind the wait
+        asm volatile("" : "+r"(r[i][0]), "+r"(r[i][1]), "+r"(r[i][2]), "+r"(r[i][3]), "+r"(r[i][4]), "+r"(r[i][5]),
+                          "+r"(r[i][6]), "+r"(r[i][7]), "+r"(r[i][8]), "+r"(r[i][9]), "+r"(r[i][10]), "+r"(r[i][11]),
+                          "+r"(r[i][12]), "+r"(r[i][13]), "+r"(r[i][14]), "+r"(r[i][15]));
 }
 
 __device__ __forceinline__ uint32_t bf16x2_bits(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+
+// warp roles
+constexpr int kProducerWarps = 12;      // warps 0-11: activations (FP32 -> BF16 hi / lo)
+constexpr int kEpilogueWarp0 = 12;      // warps 12-15: accumulator -> global (TMEM lanes 32 (w % 4) ..)
+constexpr int kMmaWarp = 16;            // warp 16: tensor-memory allocation; the MMA loop (elected lane issues)
+constexpr int kWeightWarp = 17;         // warp 17: tensor copies of the weights
+constexpr int kThreads = 18 * 32;
+constexpr int kProducers = kProducerWarps * 32;
+static_assert(kEpilogueWarp0 % 4 == 0 && kEpilogueWarp0 == kProducerWarps && kEpilogueWarp0 + 4 == kMmaWarp, "warp roles");
 
 template <int BN, int MT, bool LO>
 struct TcShape {
     static constexpr int TH = 16, TW = 8 * MT;               // output block (MT tiles of 16 x 8)
     static constexpr int HWD = TW + 2, HP = (TH + 2) * HWD;  // halo block width, pixels
-    static constexpr int NQ = (HP * 4 + 255) / 256;          // 16-byte loads per producer thread per chunk
+    static constexpr int NQ = (HP * 2 + kProducers - 1) / kProducers;   // 8-channel items per producer thread per chunk
     static constexpr int PLANE = HP * 16;                    // 8 channels of every halo pixel (BF16)
     static constexpr int A_HALF = 2 * PLANE;                 // one BF16 half of a 16-channel chunk
     static constexpr int A_BYTES = (LO ? 2 : 1) * A_HALF;
-    static constexpr int B_PLANE = BN * 16;                  // 8 input channels of BN weight rows
-    static constexpr int B_TAP = 2 * B_PLANE;
+    static constexpr int B_TAP = BN * 32;                    // BN weight rows of 16 input channels, 32-byte swizzle
     static constexpr int B_BYTES = 9 * B_TAP;                // weights of one 16-channel chunk
     static constexpr int ACC = MT * BN;                      // accumulator columns of one block
     static constexpr int COLS = 2 * ACC <= 32 ? 32 : 2 * ACC <= 64 ? 64 : 2 * ACC <= 128 ? 128
                                 : 2 * ACC <= 256 ? 256 : 512;   // two accumulators
     static constexpr uint32_t IDESC = idesc_bf16_f32(128, BN);
+    static constexpr uint32_t A_HI = desc_hi(HWD * 16, kNoSwizzle), B_HI = desc_hi(256, kSwizzle32);
+    // operand buffers rounded up so that the weights start on a 256-byte boundary (the swizzle's period)
+    static constexpr int ring_bytes(int stages) { return (stages * A_BYTES + 255) / 256 * 256; }
     static_assert(BN % 16 == 0 && BN >= 32 && BN <= 128 && MT >= 1 && MT <= 2, "tile");
 };
 
-// warp roles
-constexpr int kProducerWarps = 8;       // warps 0-7: activations (FP32 -> BF16 hi / lo)
-constexpr int kEpilogueWarp0 = 8;       // warps 8-11: accumulator -> global (TMEM lanes 32 (w % 4) ..)
-constexpr int kMmaWarp = 12;            // warp 12: tensor-memory allocation; the MMA loop (elected lane issues)
-constexpr int kWeightWarp = 13;         // warp 13: weights per chunk when they are not resident
-constexpr int kThreads = 14 * 32;
-constexpr int kProducers = kProducerWarps * 32;
-static_assert(kEpilogueWarp0 % 4 == 0 && kEpilogueWarp0 + 4 == kMmaWarp && kProducers == 256, "warp roles");
+template <int I> struct Const { static constexpr int value = I; };
 
 struct TcConf {
     int stages;     // BF16 operand buffers (and weight buffers when not resident)
@@ -207,23 +214,35 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
 
 // Persistent, warp-specialised.  CTA b takes the output blocks b, b + gridDim.x, ...
 // (output channels of blockIdx.y) and walks their 16-channel chunks as one sequence
-// g = 0 .. G-1.  Barriers: full[s] (operands of the chunk in buffer s staged: one
-// arrival per producer warp, and one from the weight warp when weights stream), empty[s] (the MMAs that
-// read buffer s completed: tcgen05.commit), acc_full[b] (the MMAs of the block in
-// accumulator b completed), acc_empty[b] (the epilogue warps have read accumulator b:
-// one arrival per warp).
+// g = 0 .. G-1.  Barriers: full[s] (activations of the chunk in buffer s staged: one
+// arrival per producer warp), wfull[s] (weights of the chunk in buffer s landed; resident weights:
+// wfull[0], all of them), empty[s] (the MMAs that read buffer s completed: tcgen05.commit),
+// acc_full[b] (the MMAs of the block in accumulator b completed), acc_empty[b] (the epilogue warps
+// have read accumulator b: one arrival per warp).
 // Shared memory: [BF16 operand buffers][weights].
+//
+// What bounds it: an MMA takes max(32 + BN / 4, BN / 2) clocks (128 rows of A and BN of B read from
+// shared memory at 128 bytes per clock, or the arithmetic), measured alike for every operand layout and
+// alignment: 1450 clocks per chunk at BN = 32, 2300 at 128.  At BN = 128 the MMAs take three quarters
+// of the time (the rest: the first chunk's way in and the last block's way out, one or two blocks per
+// CTA); at BN = 32 shared memory is shared with the conversion and the stores (about 2000 clocks per
+// chunk).  Before, the weights came by one warp's 16-byte copies (2.4 us per chunk at BN = 128; now one
+// tensor copy, box 16 channels x BN x 9 taps), and eight warps converted 4-channel items (1.5 us per
+// chunk).  16 samples: 32 -> 32 channels at 256^2 100 -> 76 us, 64 + 32 -> 32 229 -> 170, 128 + 64 -> 64
+// at 128^2 146 -> 100, 256 + 128 -> 128 at 64^2 117 -> 78, 256 -> 256 at 32^2 47 -> 35.
 template <int BN, int MT, bool LO>
-__global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcConf cf)
+__global__ void __launch_bounds__(kThreads, 1)
+    conv3_tc_kernel(const __grid_constant__ CUtensorMap wmap, ConvTcArgs a, TcConf cf)
 {
     using S = TcShape<BN, MT, LO>;
-    extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2];
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], wfull[kMaxStages], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     volatile int* abort_v = &abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = a.W / S::TW, tiles_y = a.H / S::TH;
+    const int tiles_x = a.W / S::TW, tiles_y = a.H / S::TH;      // powers of two
+    const int ltx = 31 - __clz(tiles_x), lty = 31 - __clz(tiles_y);
     const int ntiles = a.B * tiles_x * tiles_y;
     const int co0 = blockIdx.y * BN;
     const int Cin = a.C1 + a.C2;
@@ -231,8 +250,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
     const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int G = my_tiles * nchunk;
     const int stages = cf.stages;
-    uint8_t* const ring = smem;
-    uint8_t* const wts = smem + stages * S::A_BYTES;
+    uint8_t* const ring = smem_raw + (0u - smem_addr(smem_raw) & 255u);
+    const uint32_t wts = smem_addr(ring) + S::ring_bytes(stages);
 
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -244,30 +263,15 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
     if (tid == 0) {
         abort_flag = 0;
         for (int i = 0; i < stages; ++i) {
-            mbar_init(smem_addr(&full[i]), kProducerWarps + (cf.resident ? 0 : 1));   // one arrival per warp
+            mbar_init(smem_addr(&full[i]), kProducerWarps);   // one arrival per warp
             mbar_init(smem_addr(&empty[i]), 1);
+            mbar_init(smem_addr(&wfull[i]), 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_addr(&acc_full[i]), 1);
             mbar_init(smem_addr(&acc_empty[i]), 4);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    // weights of one chunk c into `dst`: row co, plane p = input channels 16 c + 8 p .. + 7, nine taps
-    auto copy_b = [&](int c, uint8_t* dst, int first, int step) {
-        const uint32_t bs = smem_addr(dst);
-        const int ci0 = c * 16;
-        for (int q = first; q < 9 * BN * 2; q += step) {
-            const int plane = q & 1, r = q >> 1;         // r = co * 9 + tap
-            const int co = r / 9, tap = r - co * 9;
-            cp_async16(bs + tap * S::B_TAP + plane * S::B_PLANE + co * 16,
-                       a.w + ((long long)(co0 + co) * 9 + tap) * Cin + ci0 + plane * 8);
-        }
-    };
-    if (cf.resident && G > 0) {
-        for (int c = 0; c < nchunk; ++c) copy_b(c, wts + c * S::B_BYTES, tid, kThreads);
-        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
@@ -276,81 +280,102 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
 
     auto tile_of = [&](int t, int& n, int& ty0, int& tx0) {
         const int tile = (int)blockIdx.x + t * (int)gridDim.x;
-        n = tile / (tiles_x * tiles_y);
-        ty0 = ((tile / tiles_x) % tiles_y) * S::TH;
-        tx0 = (tile % tiles_x) * S::TW;
+        n = tile >> (ltx + lty);
+        ty0 = ((tile >> ltx) & (tiles_y - 1)) * S::TH;
+        tx0 = (tile & (tiles_x - 1)) * S::TW;
     };
 
     if (warp < kProducerWarps) {
-        // ---- activations: the FP32 loads of chunk g + DEPTH are issued once chunk g is converted ----
+        // ---- activations: the FP32 loads of chunk g + DEPTH are issued once chunk g is converted.
+        // An item is one pixel's 8 channels of a plane: 32 bytes read, 16 bytes of hi and of lo written
+        // (the two planes lie 64 bytes apart modulo 128, so eight lanes' stores share no bank).  This
+        // loop paced the kernel with 4-channel items on eight warps and divisions per chunk: 1.5 us per
+        // chunk, with one MMA per tap as with two. ----
         constexpr int DEPTH = LBM_CONV_TC_DEPTH;
-        // pixel indices of this thread's halo elements in the block being loaded, the same for
-        // every channel chunk of the block: full resolution, and halved for an x1 stored at half size
-        int cached_t = -1;
+        static_assert(S::PLANE % 128 == 64, "planes half a line apart");
+        // element offsets of this thread's halo pixels in the block being loaded: full resolution, and
+        // halved for an x1 stored at half size
         uint32_t pix_full[S::NQ], pix_half[S::NQ];
-        float4 v[DEPTH][S::NQ];
-        auto load = [&](int g, float4 (&u)[S::NQ]) {
-            const int t = g / nchunk, ci0 = (g - t * nchunk) * 16;
-            if (t != cached_t) {
+        float4 v[DEPTH][S::NQ][2];
+        int lt = 0, lc = 0;                                // block and chunk of the next load
+        auto load = [&](float4 (&u)[S::NQ][2]) {
+            if (lt == my_tiles) return;
+            if (lc == 0) {
                 int n, ty0, tx0;
-                tile_of(t, n, ty0, tx0);
+                tile_of(lt, n, ty0, tx0);
 #pragma unroll
                 for (int i = 0; i < S::NQ; ++i) {
-                    const int hp = (tid + kProducers * i) >> 2;
+                    const int hp = (tid + kProducers * i) >> 1;
                     const int hy = hp / S::HWD, hx = hp - hy * S::HWD;
                     const int sy = (ty0 + hy - 1) & (a.H - 1), sx = (tx0 + hx - 1) & (a.W - 1);
                     pix_full[i] = ((uint32_t)n * (uint32_t)a.H + (uint32_t)sy) * (uint32_t)a.W + (uint32_t)sx;
                     pix_half[i] = ((uint32_t)n * (uint32_t)(a.H >> 1) + (uint32_t)(sy >> 1)) * (uint32_t)(a.W >> 1) +
                                   (uint32_t)(sx >> 1);
                 }
-                cached_t = t;
             }
+            const int ci0 = lc * 16;
             const bool from1 = ci0 < a.C1;
-            const float* base = (from1 ? a.x1 + ci0 : a.x2 + (ci0 - a.C1)) + (tid & 3) * 4;
-            const size_t cstride = (size_t)(from1 ? a.C1 : a.C2);
+            const float* base = (from1 ? a.x1 + ci0 : a.x2 + (ci0 - a.C1)) + (tid & 1) * 8;
+            const uint32_t cstride = (uint32_t)(from1 ? a.C1 : a.C2);
             const bool half = from1 && a.x1_half;          // nearest upsampling of a half-size x1
 #pragma unroll
             for (int i = 0; i < S::NQ; ++i)
-                if (tid + kProducers * i < S::HP * 4)
-                    u[i] = __ldg(reinterpret_cast<const float4*>(base + (size_t)(half ? pix_half[i] : pix_full[i]) * cstride));
+                if (tid + kProducers * i < S::HP * 2) {
+                    const float4* p = reinterpret_cast<const float4*>(
+                        base + (unsigned long long)(half ? pix_half[i] : pix_full[i]) * cstride);
+                    u[i][0] = __ldg(p);
+                    u[i][1] = __ldg(p + 1);
+                }
+            if (++lc == nchunk) {
+                lc = 0;
+                ++lt;
+            }
         };
 #pragma unroll
-        for (int d = 0; d < DEPTH; ++d)
-            if (d < G) load(d, v[d]);
+        for (int d = 0; d < DEPTH; ++d) load(v[d]);
         bool ok = true;
+        int s = 0;
+        uint32_t ph = 1;                                   // the first round of buffers is free
         for (int g0 = 0; g0 < G && ok; g0 += DEPTH) {
 #pragma unroll
             for (int d = 0; d < DEPTH; ++d) {
                 const int g = g0 + d;
-                if (g >= G || !ok) break;
-                const int s = g % stages;
+                if (g >= G) break;
                 // (warp-uniform, so that the whole warp leaves together after an abort)
-                if (g >= stages)
-                    ok = __all_sync(0xffffffffu,
-                                    wait_or_abort(smem_addr(&empty[s]), (uint32_t)((g / stages - 1) & 1), abort_v));
+                if (g >= stages) ok = __all_sync(0xffffffffu, wait_or_abort(smem_addr(&empty[s]), ph, abort_v));
                 if (!ok) break;
-                uint8_t* st = ring + s * S::A_BYTES + ((tid & 3) >> 1) * S::PLANE + (tid & 1) * 8;
+                uint8_t* st = ring + s * S::A_BYTES + (tid & 1) * S::PLANE;
 #pragma unroll
                 for (int i = 0; i < S::NQ; ++i) {
                     const int q = tid + kProducers * i;
-                    if (q < S::HP * 4) {
-                        const float4 u = v[d][i];
-                        const int off = (q >> 2) * 16;
-                        const __nv_bfloat162 h01 = __floats2bfloat162_rn(u.x, u.y), h23 = __floats2bfloat162_rn(u.z, u.w);
-                        *reinterpret_cast<uint2*>(st + off) = make_uint2(bf16x2_bits(h01), bf16x2_bits(h23));
-                        if constexpr (LO) {
-                            const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
-                            const __nv_bfloat162 l01 = __floats2bfloat162_rn(u.x - f01.x, u.y - f01.y);
-                            const __nv_bfloat162 l23 = __floats2bfloat162_rn(u.z - f23.x, u.w - f23.y);
-                            *reinterpret_cast<uint2*>(st + S::A_HALF + off) =
-                                make_uint2(bf16x2_bits(l01), bf16x2_bits(l23));
+                    if (q < S::HP * 2) {
+                        uint32_t hi[4], lo[4];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float4 u = v[d][i][e];
+                            const __nv_bfloat162 h01 = __floats2bfloat162_rn(u.x, u.y), h23 = __floats2bfloat162_rn(u.z, u.w);
+                            hi[2 * e] = bf16x2_bits(h01);
+                            hi[2 * e + 1] = bf16x2_bits(h23);
+                            if constexpr (LO) {
+                                const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+                                lo[2 * e] = bf16x2_bits(__floats2bfloat162_rn(u.x - f01.x, u.y - f01.y));
+                                lo[2 * e + 1] = bf16x2_bits(__floats2bfloat162_rn(u.z - f23.x, u.w - f23.y));
+                            }
                         }
+                        const int off = (q >> 1) * 16;
+                        *reinterpret_cast<uint4*>(st + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                        if constexpr (LO)
+                            *reinterpret_cast<uint4*>(st + S::A_HALF + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor core
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_addr(&full[s]));              // for the whole warp
-                if (g + DEPTH < G) load(g + DEPTH, v[d]);
+                load(v[d]);
+                if (++s == stages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
         }
     } else if (warp < kEpilogueWarp0 + 4) {
@@ -358,7 +383,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
         // Read as matrix fragments (16 pixels x 32 channels per load): four lanes then hold 8 adjacent
         // channels of a pixel and a store covers whole 32-byte sectors.  One pixel per lane stored
         // 16-byte pieces of 32 different lines at a time, every sector twice.
+        // With one warp per scheduler the loop is bound by its own instructions' latency, so addresses
+        // are one base per block plus 32-bit offsets and the bias stays in registers.
         const int q = warp & 3, gr = lane >> 2, t4 = lane & 3;
+        constexpr int NC = BN / 32;                          // 32-column pieces of a tile's accumulator
+        const int Co2 = a.Cout - a.Co1;
         float2 bias[BN / 8];
 #pragma unroll
         for (int j = 0; j < BN / 8; ++j)
@@ -369,40 +398,61 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
             tc_fence_after();
             int n, ty0, tx0;
             tile_of(t, n, ty0, tx0);
-#pragma unroll 1
-            for (int jh = 0; jh < 2 * MT; ++jh) {                       // tile, upper or lower 16 TMEM lanes
-                const int j = jh >> 1, hh = jh & 1;
-                const uint32_t row = tmem + ((uint32_t)(q * 32 + hh * 16) << 16) + (uint32_t)((t & 1) * S::ACC + j * BN);
-                // TMEM lane m = pixel (m >> 3, m & 7) of the tile
-                const long long p = ((long long)n * a.H + ty0 + q * 4 + hh * 2) * a.W + tx0 + 8 * j + gr;
+            // TMEM lane m = pixel (m >> 3, m & 7) of a tile; this lane's first pixel
+            const long long p0 = ((long long)n * a.H + ty0 + q * 4) * a.W + tx0 + gr;
+            float* const y1 = a.y1 + p0 * a.Co1 + 2 * t4;
+            float* const y2 = a.y2 + p0 * Co2 + 2 * t4 - a.Co1;
+            const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((t & 1) * S::ACC);
+            // 16 lanes (half hh) x 32 columns (piece c) of tile j
+            auto put = [&](const uint32_t (&v)[16], int j, int hh, auto piece) {
+                constexpr int c = decltype(piece)::value;
 #pragma unroll
-                for (int cc = 0; cc < BN; cc += 32) {
-                    float v[16];
-                    tmem_ld_16x32(row + (uint32_t)cc, v);
+                for (int h = 0; h < 2; ++h) {
+                    const int dp = (2 * hh + h) * a.W + 8 * j;
+                    float* const r1 = y1 + dp * a.Co1;
+                    float* const r2 = y2 + dp * Co2;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const long long ph = p + h * a.W;
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int co = co0 + cc + 8 * k;            // 8 channels, all in y1 or all in y2
-                            float* dst = (co < a.Co1 ? a.y1 + ph * a.Co1 + co : a.y2 + ph * (a.Cout - a.Co1) + (co - a.Co1)) +
-                                         2 * t4;
-                            float2 r = make_float2(v[4 * k + 2 * h], v[4 * k + 2 * h + 1]);
-                            if (a.bias) {
-                                r.x += bias[cc / 8 + k].x;
-                                r.y += bias[cc / 8 + k].y;
-                            }
-                            if (a.relu) {
-                                r.x = fmaxf(r.x, 0.f);
-                                r.y = fmaxf(r.y, 0.f);
-                            }
-                            if (a.beta) {
-                                const float2 o = *reinterpret_cast<const float2*>(dst);
-                                r.x += o.x;
-                                r.y += o.y;
-                            }
-                            *reinterpret_cast<float2*>(dst) = r;
+                    for (int k = 0; k < 4; ++k) {
+                        const int co = co0 + 32 * c + 8 * k;            // 8 channels, all in y1 or all in y2
+                        float* const dst = (co < a.Co1 ? r1 : r2) + co;
+                        float2 r = make_float2(__uint_as_float(v[4 * k + 2 * h]), __uint_as_float(v[4 * k + 2 * h + 1]));
+                        if (a.bias) {
+                            r.x += bias[4 * c + k].x;
+                            r.y += bias[4 * c + k].y;
                         }
+                        if (a.relu) {
+                            r.x = fmaxf(r.x, 0.f);
+                            r.y = fmaxf(r.y, 0.f);
+                        }
+                        if (a.beta) {
+                            const float2 o = *reinterpret_cast<const float2*>(dst);
+                            r.x += o.x;
+                            r.y += o.y;
+                        }
+                        *reinterpret_cast<float2*>(dst) = r;
+                    }
+                }
+            };
+            uint32_t v[2][16];
+            if constexpr (NC == 1) {
+#pragma unroll 1
+                for (int j = 0; j < MT; ++j) {
+                    tmem_ld_16x32_pair(acc + j * BN, acc + (16u << 16) + j * BN, v);
+                    put(v[0], j, 0, Const<0>());
+                    put(v[1], j, 1, Const<0>());
+                }
+            } else {
+#pragma unroll 1
+                for (int jh = 0; jh < 2 * MT; ++jh) {
+                    const int j = jh >> 1, hh = jh & 1;
+                    const uint32_t at = acc + ((uint32_t)(16 * hh) << 16) + j * BN;
+                    tmem_ld_16x32_pair(at, at + 32, v);
+                    put(v[0], j, hh, Const<0>());
+                    put(v[1], j, hh, Const<1>());
+                    if constexpr (NC == 4) {
+                        tmem_ld_16x32_pair(at + 64, at + 96, v);
+                        put(v[0], j, hh, Const<2>());
+                        put(v[1], j, hh, Const<3>());
                     }
                 }
             }
@@ -413,63 +463,79 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(ConvTcArgs a, TcC
     } else if (warp == kMmaWarp) {
         // ---- MMAs: the whole warp runs the loop (warp-uniform control flow and operands),
         //      one elected lane issues each instruction ----
-        int last = -1;
-        for (int g = 0; g < G; ++g) {
-            const int t = g / nchunk, c = g - t * nchunk, s = g % stages;
-            // accumulator t & 1 was last read by the epilogue of block t - 2
-            if (c == 0 && t >= 2 &&
-                !__all_sync(0xffffffffu, wait_or_abort(smem_addr(&acc_empty[t & 1]),
-                                                       (uint32_t)(((t >> 1) - 1) & 1), abort_v)))
-                break;
-            if (!__all_sync(0xffffffffu, wait_or_abort(smem_addr(&full[s]), (uint32_t)((g / stages) & 1), abort_v)))
-                break;
+        int last = -1, t = 0, c = 0, s = 0;
+        uint32_t ph = 0;
+        // Operands of chunk g (buffer s, phase ph) staged, and the accumulator of a new block read by the
+        // epilogue of the block two before.  A look at a barrier takes some 200 clocks while the MMAs
+        // read shared memory, which idled the tensor core between chunks: the first look at the next
+        // chunk's barriers comes before the last taps of this one, and only a failed one waits.
+        auto ready = [&](int g, int t, int c, int s, uint32_t ph, auto wait) {
+            return !(c == 0 && t >= 2 && !wait(smem_addr(&acc_empty[t & 1]), (uint32_t)(((t >> 1) - 1) & 1))) &&
+                   ((cf.resident && g > 0) || wait(smem_addr(&wfull[s]), ph)) && wait(smem_addr(&full[s]), ph);
+        };
+        auto look = [](uint32_t bar, uint32_t parity) { return mbar_try(bar, parity); };
+        auto block = [&](uint32_t bar, uint32_t parity) { return wait_or_abort(bar, parity, abort_v); };
+        bool ok = G == 0 || __all_sync(0xffffffffu, ready(0, 0, 0, 0, 0, block));
+        for (int g = 0; g < G && ok; ++g) {
             tc_fence_after();
-            const uint32_t ab = smem_addr(ring + s * S::A_BYTES);
-            const uint32_t bb = smem_addr(wts + (cf.resident ? c : s) * S::B_BYTES);
+            const uint32_t ad = desc_lo(smem_addr(ring) + s * S::A_BYTES, S::PLANE);
+            const uint32_t bd = desc_lo(wts + (cf.resident ? c : s) * S::B_BYTES, 0);
             const uint32_t acc = tmem + (uint32_t)((t & 1) * S::ACC);
+            const uint32_t empty_bar = smem_addr(&empty[s]), acc_bar = smem_addr(&acc_full[t & 1]);
+            const uint32_t first = (uint32_t)c;
+            if (++s == stages) {
+                s = 0;
+                ph ^= 1u;
+            }
+            const bool block_done = ++c == nchunk;
+            if (block_done) {
+                c = 0;
+                ++t;
+            }
+            bool next = false;
 #pragma unroll
             for (int tap = 0; tap < 9; ++tap) {
                 const int dy = tap / 3, dx = tap - dy * 3;
-                const uint64_t bd = smem_desc(bb + tap * S::B_TAP, S::B_PLANE, 128);
+                if (tap == 6 && g + 1 < G) next = __all_sync(0xffffffffu, ready(g + 1, t, c, s, ph, look));
 #pragma unroll
                 for (int j = 0; j < MT; ++j) {
-                    const uint32_t aoff = (uint32_t)((dy * S::HWD + 8 * j + dx) * 16);
+                    const uint32_t aoff = (uint32_t)(dy * S::HWD + 8 * j + dx);     // 16-byte pixels
                     const uint32_t d = acc + (uint32_t)(j * BN);
-                    mma_bf16_ss_elect(d, smem_desc(ab + aoff, S::PLANE, S::HWD * 16), bd, S::IDESC,
-                                      (c | tap) != 0);
+                    mma_bf16_ss_elect<S::A_HI, S::B_HI, S::IDESC>(d, ad + aoff, bd + tap * (S::B_TAP / 16),
+                                                                  tap != 0 ? 1u : first);
                     if constexpr (LO)
-                        mma_bf16_ss_elect(d, smem_desc(ab + S::A_HALF + aoff, S::PLANE, S::HWD * 16), bd,
-                                          S::IDESC, 1u);
+                        mma_bf16_ss_elect<S::A_HI, S::B_HI, S::IDESC>(d, ad + S::A_HALF / 16 + aoff,
+                                                                      bd + tap * (S::B_TAP / 16), 1u);
                 }
             }
-            mma_commit_elect(smem_addr(&empty[s]));
-            if (c == nchunk - 1) mma_commit_elect(smem_addr(&acc_full[t & 1]));
+            mma_commit_elect(empty_bar);
+            if (block_done) mma_commit_elect(acc_bar);
             last = g;
+            if (!next && g + 1 < G) ok = __all_sync(0xffffffffu, ready(g + 1, t, c, s, ph, block));
         }
         // after an abort: wait (bounded) for the MMAs in flight before the memory is freed
         if (*abort_v && last >= 0) mbar_wait(smem_addr(&empty[last % stages]), (uint32_t)((last / stages) & 1));
         __syncwarp();
-    } else if (warp == kWeightWarp && !cf.resident) {
-        // ---- weights of chunk g + 1 copied while chunk g is consumed ----
-        if (G > 0) copy_b(0, wts, lane, 32);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        for (int g = 0; g < G; ++g) {
-            const int s = g % stages;
-            bool ok = true;
-            if (g + 1 < G) {
-                const int g1 = g + 1, s1 = g1 % stages;
-                if (g1 >= stages)
-                    ok = __all_sync(0xffffffffu,
-                                    wait_or_abort(smem_addr(&empty[s1]), (uint32_t)((g1 / stages - 1) & 1), abort_v));
-                if (ok) copy_b(g1 % nchunk, wts + s1 * S::B_BYTES, lane, 32);
+    } else if (warp == kWeightWarp && lane == 0 && G > 0) {
+        // ---- weights: all chunks once, or chunk g as soon as buffer g % stages is free ----
+        lbmt::prefetch_map(&wmap);
+        if (cf.resident) {
+            lbmt::mbar_arrive_expect_tx(smem_addr(&wfull[0]), (uint32_t)(nchunk * S::B_BYTES));
+            for (int c = 0; c < nchunk; ++c)
+                lbmt::tma_load_3d(wts + c * S::B_BYTES, &wmap, 16 * c, co0, 0, smem_addr(&wfull[0]));
+            lbmt::mbar_drain(smem_addr(&wfull[0]), 0);
+        } else {
+            int g = 0;
+            for (; g < G; ++g) {
+                const int s = g % stages;
+                if (g >= stages && !wait_or_abort(smem_addr(&empty[s]), (uint32_t)((g / stages - 1) & 1), abort_v)) break;
+                lbmt::mbar_arrive_expect_tx(smem_addr(&wfull[s]), (uint32_t)S::B_BYTES);
+                lbmt::tma_load_3d(wts + s * S::B_BYTES, &wmap, 16 * (g % nchunk), co0, 0, smem_addr(&wfull[s]));
             }
-            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");   // chunk g landed
-            if (!ok) break;
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_addr(&full[s]));
+            // every copy issued has landed before the block leaves
+            for (int q = g > stages ? g - stages : 0; q < g; ++q)
+                lbmt::mbar_drain(smem_addr(&wfull[q % stages]), (uint32_t)((q / stages) & 1));
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
@@ -530,12 +596,14 @@ bool launch_variant(const ConvTcArgs& a, cudaStream_t s, int stages, int slot)
         v.ready = 1;
     }
     const int nchunk = (a.C1 + a.C2) / 16;
+    CUtensorMap wmap;
+    if (!lbmh::encode_conv3_weights_map(&wmap, a.w, a.C1 + a.C2, a.Cout, BN)) return false;
     TcConf cf{stages > 0 ? stages : 3, 1};
     if (cf.stages < 2 || cf.stages > kMaxStages) return false;
     // largest configuration that fits: resident weights first, then fewer operand buffers
     long long smem = 0;
     for (;;) {
-        const long long base = (long long)cf.stages * S::A_BYTES;
+        const long long base = 256 + S::ring_bytes(cf.stages);       // 256: alignment
         const long long res = base + (long long)nchunk * S::B_BYTES;
         const long long str = base + (long long)cf.stages * S::B_BYTES;
         if (res <= kSmemLimit) { cf.resident = 1; smem = res; break; }
@@ -552,7 +620,7 @@ bool launch_variant(const ConvTcArgs& a, cudaStream_t s, int stages, int slot)
     long long gx = ((long long)per_sm * g_sms[dev] + cob - 1) / cob;
     if (gx > ntiles) gx = ntiles;
     if (gx < 1) gx = 1;
-    conv3_tc_kernel<BN, MT, LO><<<dim3((unsigned)gx, (unsigned)cob), kThreads, (size_t)smem, s>>>(a, cf);
+    conv3_tc_kernel<BN, MT, LO><<<dim3((unsigned)gx, (unsigned)cob), kThreads, (size_t)smem, s>>>(wmap, a, cf);
     return true;
 }
 

@@ -2,6 +2,7 @@
 // the convolution entry point of nn_kernels.cu.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -26,3 +27,9 @@ bool conv3_tc_launch(const ConvTcArgs& a, cudaStream_t s, int stages);
 // Reads and clears the flag that a bounded wait inside the kernel ran out
 // (the output of that launch is invalid); synchronises `s`.
 bool conv3_tc_take_timeout(cudaStream_t s);
+
+namespace lbmh {
+// tensor map of BF16 weights [cout][3][3][cin]: box {16 input channels, box_co, 9 taps} with the
+// 32-byte swizzle, defined in lbm_capi.cu
+bool encode_conv3_weights_map(CUtensorMap* m, const void* w, int cin, int cout, int box_co);
+}  // namespace lbmh
