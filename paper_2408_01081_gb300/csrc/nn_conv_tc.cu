@@ -35,6 +35,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "lbm_tma.cuh"
 #include "nn_conv_tc.h"
 
@@ -133,25 +135,39 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+__device__ __forceinline__ void tmem_ld_16x32_issue(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+// keeps the uses of loaded registers behind the wait
+__device__ __forceinline__ void behind_the_wait(uint32_t (&r)[16])
+{
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                      "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                      "+r"(r[15]));
+}
+
 // 16 lanes x 32 columns of an accumulator as matrix fragments: v[4 j + 2 h + e] is lane lane/4 + 8 h,
 // column 8 j + 2 (lane % 4) + e.  Two of them per wait.
 __device__ __forceinline__ void tmem_ld_16x32_pair(uint32_t taddr0, uint32_t taddr1, uint32_t (&r)[2][16])
 {
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        asm volatile(
-            "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(r[i][0]), "=r"(r[i][1]), "=r"(r[i][2]), "=r"(r[i][3]), "=r"(r[i][4]), "=r"(r[i][5]), "=r"(r[i][6]),
-              "=r"(r[i][7]), "=r"(r[i][8]), "=r"(r[i][9]), "=r"(r[i][10]), "=r"(r[i][11]), "=r"(r[i][12]),
-              "=r"(r[i][13]), "=r"(r[i][14]), "=r"(r[i][15])
-            : "r"(i ? taddr1 : taddr0)
-            : "memory");
+    tmem_ld_16x32_issue(taddr0, r[0]);
+    tmem_ld_16x32_issue(taddr1, r[1]);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 2; ++i)          // uses stay behind the wait
-        asm volatile("" : "+r"(r[i][0]), "+r"(r[i][1]), "+r"(r[i][2]), "+r"(r[i][3]), "+r"(r[i][4]), "+r"(r[i][5]),
-                          "+r"(r[i][6]), "+r"(r[i][7]), "+r"(r[i][8]), "+r"(r[i][9]), "+r"(r[i][10]), "+r"(r[i][11]),
-                          "+r"(r[i][12]), "+r"(r[i][13]), "+r"(r[i][14]), "+r"(r[i][15]));
+    behind_the_wait(r[0]);
+    behind_the_wait(r[1]);
+}
+
+__device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, uint32_t (&r)[16])
+{
+    tmem_ld_16x32_issue(taddr, r);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    behind_the_wait(r);
 }
 
 __device__ __forceinline__ uint32_t bf16x2_bits(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t*>(&v); }
@@ -547,6 +563,232 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
+// ---------------------------------------------------------------------------
+// 3x3 weight gradient, dW[co][dy][dx][ci] = sum over pixels of dY[p][co] X[p + (dy, dx) - 1][ci], on
+// 16 x 16 pixel blocks.  A CTA takes CB output x 32 input channels, all nine taps and a range of blocks
+// (gridDim.z ranges; partials summed in fixed order by the caller).
+//
+// Both operands have their channels contiguous and the pixels as the K index: the M / N-major layout
+// without swizzle, 16-byte rows of 8 channels, 16 pixels of an image row per MMA.  A block's dY lies in
+// shared memory as [row][8-channel plane][16 pixels], X with its halo as [row][plane][18 pixels], both
+// with 288 bytes per plane, so that the planes of consecutive rows follow each other at one stride and
+//   A = dY of 2 rows x CB channels (M = 2 CB),  B = X of the 4 halo rows around them x 32 channels (N = 128):
+// block (i, j) of the product, dY row i against X row j, is the tap dy = j - i: six of the eight blocks
+// are taps.  The tap dx is B started dx pixels further on, each with its own accumulator D_dx (128
+// columns).  Per row pair and dx three MMAs: dY_hi X_hi + dY_hi X_lo + dY_lo X_hi.
+//
+// What bounds it: 72 MMAs of 64 clocks per block (M = 64 takes as long as 128): 33 us of the 43 us that
+// 32 x 32 channels take at 8 x 256 x 256 (20 us of memory traffic).  The mma.sync kernel before, one warp
+// per tap reading its fragments with ldmatrix, took 104 us there at half of mma.sync's rate (47 us);
+// 384 -> 128 channels at 16 x 64 x 64, whole layer: 855 -> 377 us.
+// Sixteen warps load, split into BF16 halves and stage a block while the MMAs of the one before run.
+// ---------------------------------------------------------------------------
+constexpr int kWgProducerWarps = 16;
+constexpr int kWgEpilogueWarp0 = 16;     // four warps: accumulators -> partials
+constexpr int kWgMmaWarp = 20;
+constexpr int kWgThreads = 21 * 32;
+constexpr int kWgProducers = kWgProducerWarps * 32;
+
+template <int CB>
+struct WgShape {
+    static constexpr int PLANE = 288;                                   // bytes of 8 channels of a row
+    static constexpr int Y_BYTES = 16 * (CB / 8) * PLANE;               // one BF16 half of dY
+    static constexpr int X_BYTES = 18 * 4 * PLANE;                      // one BF16 half of X
+    static constexpr int STAGE = 2 * (Y_BYTES + X_BYTES);
+    static constexpr int SMEM = 2 * STAGE + 128;
+    static constexpr int YQ = 256 * (CB / 8) / kWgProducers;            // 8-channel items per thread: dY
+    static constexpr int XQ = (18 * 18 * 4 + kWgProducers - 1) / kWgProducers;   // and X
+    static constexpr int M = 2 * CB;
+    // both operands M / N-major (bits 15, 16)
+    static constexpr uint32_t IDESC = idesc_bf16_f32(M, 128) | (1u << 15) | (1u << 16);
+    static constexpr uint32_t HI = desc_hi(PLANE, kNoSwizzle);          // 8 channels further: one plane
+    static_assert(256 * (CB / 8) % kWgProducers == 0, "dY items per thread");
+};
+
+template <int CB>
+__global__ void __launch_bounds__(kWgThreads, 1) conv3_wgrad_tc_kernel(ConvTcWgradArgs a)
+{
+    using S = WgShape<CB>;
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full[2], empty[2], acc_full, acc_empty;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    volatile int* abort_v = &abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int Cin = a.C1 + a.C2;
+    const int co0 = blockIdx.x * CB, ci0 = blockIdx.y * 32;
+    const int lbx = 31 - __clz(a.W / 16), lby = 31 - __clz(a.H / 16);   // powers of two
+    const int nblocks = a.B << (lbx + lby);
+    // range z of gridDim.z, in a.subs parts of at least one block each: part u ends before block end(u)
+    const int b0 = (int)((long long)nblocks * blockIdx.z / gridDim.z);
+    const int G = (int)((long long)nblocks * (blockIdx.z + 1) / gridDim.z) - b0;
+    auto end = [&](int u) { return (int)((long long)G * (u + 1) / a.subs); };
+    uint8_t* const ring = smem_raw + ((0u - smem_addr(smem_raw)) & 127u);
+
+    if (warp == kWgMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(&tmem_slot))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        abort_flag = 0;
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_addr(&full[i]), kWgProducerWarps);
+            mbar_init(smem_addr(&empty[i]), 1);
+        }
+        mbar_init(smem_addr(&acc_full), 1);
+        mbar_init(smem_addr(&acc_empty), 4);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp < kWgProducerWarps) {
+        // input channels ci0 .. ci0 + 31 lie in x1 or in x2 (C1 is a multiple of 32)
+        const bool from1 = ci0 < a.C1;
+        const int half = (from1 && a.x1_half) ? 1 : 0;                  // nearest upsampling of a half-size x1
+        const int xc = from1 ? a.C1 : a.C2;
+        const float* const xs = (from1 ? a.x1 + ci0 : a.x2 + (ci0 - a.C1)) + (tid & 3) * 8;
+        const float* const ys = a.dy + co0 + (tid & (CB / 8 - 1)) * 8;
+        float4 vy[S::YQ][2], vx[S::XQ][2];
+        auto load = [&](int b) {
+            const int n = b >> (lbx + lby), ty0 = ((b >> lbx) & ((1 << lby) - 1)) * 16, tx0 = (b & ((1 << lbx) - 1)) * 16;
+#pragma unroll
+            for (int i = 0; i < S::YQ; ++i) {
+                const int p = (tid + kWgProducers * i) / (CB / 8);
+                const long long q = ((long long)n * a.H + ty0 + (p >> 4)) * a.W + tx0 + (p & 15);
+                const float4* src = reinterpret_cast<const float4*>(ys + q * a.Cout);
+                vy[i][0] = __ldg(src);
+                vy[i][1] = __ldg(src + 1);
+            }
+#pragma unroll
+            for (int i = 0; i < S::XQ; ++i) {
+                const int hp = (tid + kWgProducers * i) >> 2;
+                if (hp < 18 * 18) {
+                    const int hy = hp / 18, hx = hp - hy * 18;
+                    const int sy = (ty0 + hy - 1) & (a.H - 1), sx = (tx0 + hx - 1) & (a.W - 1);
+                    const long long q = ((long long)n * (a.H >> half) + (sy >> half)) * (a.W >> half) + (sx >> half);
+                    const float4* src = reinterpret_cast<const float4*>(xs + q * xc);
+                    vx[i][0] = __ldg(src);
+                    vx[i][1] = __ldg(src + 1);
+                }
+            }
+        };
+        auto put = [&](uint8_t* dst, int lo_off, const float4 (&u)[2]) {
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const __nv_bfloat162 h01 = __floats2bfloat162_rn(u[e].x, u[e].y), h23 = __floats2bfloat162_rn(u[e].z, u[e].w);
+                const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+                hi[2 * e] = bf16x2_bits(h01);
+                hi[2 * e + 1] = bf16x2_bits(h23);
+                lo[2 * e] = bf16x2_bits(__floats2bfloat162_rn(u[e].x - f01.x, u[e].y - f01.y));
+                lo[2 * e + 1] = bf16x2_bits(__floats2bfloat162_rn(u[e].z - f23.x, u[e].w - f23.y));
+            }
+            *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(dst + lo_off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        };
+        load(b0);
+        for (int g = 0; g < G; ++g) {
+            const int s = g & 1;
+            if (g >= 2 &&
+                !__all_sync(0xffffffffu, wait_or_abort(smem_addr(&empty[s]), (uint32_t)(((g >> 1) - 1) & 1), abort_v)))
+                break;
+            uint8_t* const y = ring + s * S::STAGE;
+            uint8_t* const x = y + 2 * S::Y_BYTES;
+#pragma unroll
+            for (int i = 0; i < S::YQ; ++i) {
+                const int q = tid + kWgProducers * i, p = q / (CB / 8), c = q & (CB / 8 - 1);
+                put(y + ((p >> 4) * (CB / 8) + c) * S::PLANE + (p & 15) * 16, S::Y_BYTES, vy[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < S::XQ; ++i) {
+                const int q = tid + kWgProducers * i, hp = q >> 2;
+                if (hp < 18 * 18) {
+                    const int hy = hp / 18, hx = hp - hy * 18;
+                    put(x + (hy * 4 + (q & 3)) * S::PLANE + hx * 16, S::X_BYTES, vx[i]);
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor core
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&full[s]));
+            if (g + 1 < G) load(b0 + g + 1);
+        }
+    } else if (warp < kWgMmaWarp) {
+        // ---- accumulators -> partials: dY row i of the pairs is a partial of its own ----
+        // M rows 32 w .. 32 w + 31 in this warp's 32 lanes (M = 128), or 16 w .. in its first 16
+        constexpr int HALVES = CB / 32;
+        const int w = warp - kWgEpilogueWarp0, gr = lane >> 2, t4 = lane & 3;
+        for (int u = 0; u < a.subs; ++u) {
+            if (!__all_sync(0xffffffffu, wait_or_abort(smem_addr(&acc_full), (uint32_t)(u & 1), abort_v))) break;
+            tc_fence_after();
+#pragma unroll 1
+            for (int hh = 0; hh < HALVES; ++hh) {
+                const int m = w * 16 * HALVES + 16 * hh, i = m / CB, co = co0 + m % CB;
+                float* const out = a.partial + (2LL * (blockIdx.z * a.subs + u) + i) * a.Cout * 9 * Cin + ci0 + 2 * t4;
+#pragma unroll 1
+                for (int tap = 0; tap < 9; ++tap) {
+                    const int dy = tap / 3, dx = tap - 3 * dy;
+                    uint32_t v[16];
+                    tmem_ld_16x32(tmem + ((uint32_t)(32 * w + 16 * hh) << 16) + 128 * dx + 32 * (i + dy), v);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            *reinterpret_cast<float2*>(out + ((long long)(co + gr + 8 * h) * 9 + tap) * Cin + 8 * k) =
+                                make_float2(__uint_as_float(v[4 * k + 2 * h]), __uint_as_float(v[4 * k + 2 * h + 1]));
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&acc_empty));
+        }
+    } else {
+        // ---- MMAs ----
+        bool ok = true;
+        int last = -1, u = 0, g0 = 0;                       // part and its first block
+        for (int g = 0; g < G; ++g) {
+            const int s = g & 1;
+            ok = __all_sync(0xffffffffu, wait_or_abort(smem_addr(&full[s]), (uint32_t)((g >> 1) & 1), abort_v));
+            if (ok && g == g0 && u > 0)                     // the epilogue has read the part before
+                ok = __all_sync(0xffffffffu, wait_or_abort(smem_addr(&acc_empty), (uint32_t)((u - 1) & 1), abort_v));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t y = desc_lo(smem_addr(ring) + s * S::STAGE, 128);   // 8 pixels further: 128 bytes
+            const uint32_t x = y + 2 * S::Y_BYTES / 16;
+#pragma unroll
+            for (int r = 0; r < 16; r += 2)
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    const uint32_t yr = y + r * (CB / 8) * (S::PLANE / 16), xr = x + r * 4 * (S::PLANE / 16) + dx;
+                    const uint32_t d = tmem + 128 * dx;
+                    mma_bf16_ss_elect<S::HI, S::HI, S::IDESC>(d, yr, xr, r > 0 ? 1u : (uint32_t)(g - g0));
+                    mma_bf16_ss_elect<S::HI, S::HI, S::IDESC>(d, yr, xr + S::X_BYTES / 16, 1u);
+                    mma_bf16_ss_elect<S::HI, S::HI, S::IDESC>(d, yr + S::Y_BYTES / 16, xr, 1u);
+                }
+            mma_commit_elect(smem_addr(&empty[s]));
+            if (g + 1 == end(u)) {
+                mma_commit_elect(smem_addr(&acc_full));
+                ++u;
+                g0 = g + 1;
+            }
+            last = g;
+        }
+        // after an abort: wait (bounded) for the MMAs in flight before the memory is freed
+        if (!ok && last >= 0) mbar_wait(smem_addr(&empty[last & 1]), (uint32_t)((last >> 1) & 1));
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (tid == 0 && *abort_v) atomicExch(&g_tc_timeout, 1);
+    if (warp == kWgMmaWarp) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    }
+}
+
 constexpr int kMaxDevices = 64;
 
 struct VariantInfo {
@@ -634,6 +876,23 @@ bool launch_bn(const ConvTcArgs& a, cudaStream_t s, int stages, int mt)
                       : launch_variant<BN, 1, true>(a, s, stages, base + 3);
 }
 
+template <int CB>
+bool launch_wgrad(const ConvTcWgradArgs& a, int ranges, cudaStream_t s)
+{
+    static bool ready[kMaxDevices] = {};    // racing first launches set the same attribute
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+    if (!ready[dev]) {
+        if (cudaFuncSetAttribute(conv3_wgrad_tc_kernel<CB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 WgShape<CB>::SMEM) != cudaSuccess)
+            return false;
+        ready[dev] = true;
+    }
+    const dim3 grid((unsigned)(a.Cout / CB), (unsigned)((a.C1 + a.C2) / 32), (unsigned)ranges);
+    conv3_wgrad_tc_kernel<CB><<<grid, kWgThreads, WgShape<CB>::SMEM, s>>>(a);
+    return true;
+}
+
 }  // namespace
 
 bool conv3_tc_launch(const ConvTcArgs& a, cudaStream_t s, int stages)
@@ -654,6 +913,28 @@ bool conv3_tc_launch(const ConvTcArgs& a, cudaStream_t s, int stages)
     if (bn == 128) return launch_bn<128>(a, s, stages, mt);
     if (bn == 64) return launch_bn<64>(a, s, stages, mt);
     return launch_bn<32>(a, s, stages, mt);
+}
+
+// One CTA per SM: ranges of blocks for 152 of them.  The tensor core's FP32 sums round towards zero, so
+// their error grows with the number of MMAs in a row; a part of a range is at most twice the blocks that
+// fill 4 x 152 CTAs of 32 x 32 channels (each of a pair's two rows has its own sums, 24 MMAs per block),
+// the length that the kernel before had (relative error of a 32-channel layer's gradients at 8 x 256 x
+// 256: 5.1e-6 then, 6.5e-6 with one part per range, 4.9e-6 so).
+ConvTcWgradSplit conv3_wgrad_tc_split(int Cin, int Cout, int B, int H, int W)
+{
+    const long long nblocks = (long long)B * (H / 16) * (W / 16);
+    const long long tiles32 = (long long)(Cout / 32) * (Cin / 32), tiles = Cout % 64 == 0 ? tiles32 / 2 : tiles32;
+    const long long ranges = std::max(1LL, std::min(152 / tiles, nblocks));
+    const long long splits = std::min((4 * 152 + tiles32 - 1) / tiles32, nblocks);
+    const long long part = 2 * ((nblocks + splits - 1) / splits), per = (nblocks + ranges - 1) / ranges;
+    return {(int)ranges, (int)((per + part - 1) / part)};
+}
+
+bool conv3_wgrad_tc_launch(ConvTcWgradArgs a, cudaStream_t s)
+{
+    const ConvTcWgradSplit sp = conv3_wgrad_tc_split(a.C1 + a.C2, a.Cout, a.B, a.H, a.W);
+    a.subs = sp.parts;
+    return a.Cout % 64 == 0 ? launch_wgrad<64>(a, sp.ranges, s) : launch_wgrad<32>(a, sp.ranges, s);
 }
 
 bool conv3_tc_take_timeout(cudaStream_t s)

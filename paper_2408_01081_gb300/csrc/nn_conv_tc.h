@@ -24,6 +24,26 @@ struct ConvTcArgs {
 // another kernel.  `stages` = 0 picks the pipeline depth.
 bool conv3_tc_launch(const ConvTcArgs& a, cudaStream_t s, int stages);
 
+struct ConvTcWgradArgs {
+    const float* dy;            // [B][H][W][Cout]
+    const float* x1;            // as in ConvTcArgs
+    const float* x2;
+    int C1, C2, Cout;           // multiples of 32
+    int B, H, W;                // H, W powers of two, at least 16
+    int x1_half;
+    float* partial;             // [ranges][parts][2][Cout][3][3][C1 + C2]
+    int subs;                   // parts per range, set by the launch
+};
+
+// 3x3 weight gradient: ranges of 16 x 16 pixel blocks the work is split into and parts per range (two
+// partial sums each), and the launch (false: the device refused the kernel's attributes)
+struct ConvTcWgradSplit {
+    int ranges, parts;
+    int partials() const { return 2 * ranges * parts; }
+};
+ConvTcWgradSplit conv3_wgrad_tc_split(int Cin, int Cout, int B, int H, int W);
+bool conv3_wgrad_tc_launch(ConvTcWgradArgs a, cudaStream_t s);
+
 // Reads and clears the flag that a bounded wait inside the kernel ran out
 // (the output of that launch is invalid); synchronises `s`.
 bool conv3_tc_take_timeout(cudaStream_t s);
