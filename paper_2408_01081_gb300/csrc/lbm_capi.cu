@@ -849,7 +849,11 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
     const int vec = split ? ops->vec_split : ops->vec;
     const int nchunk = (ctx->p.nx + vec - 1) / vec;
     int bx = (nchunk + 31) / 32 * 32;
-    if (bx > 256) bx = 256;
+    // populations in FP32 arithmetic: small blocks fill the registers and the last wave better (us per
+    // step with body load and tracking, blocks of 256 / 128 / 64: 1021 x 515 19.5 / 17.9 / 17.6, 4096^2
+    // 547 / 532 / 528)
+    const int most = ctx->p.storage == LBM_F32 || ctx->p.storage == LBM_BF16 || ctx->p.storage == LBM_F16 ? 64 : 256;
+    if (bx > most) bx = most;
     const dim3 block(bx), grid((nchunk + bx - 1) / bx, ctx->p.ny);
     lbmk::StepArgs A;
     A.w = ctx->w;

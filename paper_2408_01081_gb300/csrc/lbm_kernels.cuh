@@ -24,6 +24,7 @@
 
 #include "lbm_f64emu.cuh"
 #include "lbm_f64fx.cuh"
+#include "lbm_tma.cuh"
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -408,19 +409,28 @@ __device__ __forceinline__ void wall_source(int i, int j, double gx, double gy, 
 // fused pull-collide step: one thread = V consecutive nodes of one row
 // grid: (ceil(ceil(nx/V) / blockDim.x), ny)
 // ---------------------------------------------------------------------------
-#ifndef LBM_STEP_MIN_BLOCKS
-#define LBM_STEP_MIN_BLOCKS 1
+// What bounds the single step in FP32 arithmetic (with a body load, tracking, wall data or omega other
+// than 2, which the kernels of several steps per pass do not take): memory, 192 bytes per node with
+// tracking in FP32, once enough warps are in flight.  Four nodes per thread took 204 registers, so 8
+// warps per SM loaded, waited and stored in turn, and read the body load's factors once per node: 2048 x
+// 1024 92 us, 4096^2 732 us.  Two nodes, 80 registers, 24 warps: 66 and 528 us (0.9 of the copy
+// bandwidth), 1021 x 515 28.9 -> 17.6; one node: 69 and 536, 16.6.
+#ifndef LBM_STEP_MIN_BLOCKS_F32
+#define LBM_STEP_MIN_BLOCKS_F32 3       // blocks of 256
 #endif
 #ifndef LBM_SPLIT_MIN_BLOCKS
 #define LBM_SPLIT_MIN_BLOCKS 3      // 80 registers: more warps to overlap the two pipes
 #endif
 
 template <int K, int V, bool DIRICHLET, bool FORCING, bool TRACK, bool OMEGA = false, unsigned long long SPLIT = 0>
-__global__ void __launch_bounds__(256, SPLIT > 0 ? LBM_SPLIT_MIN_BLOCKS : LBM_STEP_MIN_BLOCKS)
+__global__ void __launch_bounds__(256, SPLIT > 0 ? LBM_SPLIT_MIN_BLOCKS
+                                       : sizeof(typename Fmt<K>::M) == 4 ? LBM_STEP_MIN_BLOCKS_F32 : 1)
 step_kernel(StepArgs A)
 {
     using E = typename Fmt<K>::E;
     using M = typename Fmt<K>::M;
+    // FP32 arithmetic: launched while the step before drains; what that step writes is read past L1
+    constexpr bool CG = sizeof(M) == 4;
     const int y = blockIdx.y;
     const int cx = blockIdx.x * blockDim.x + threadIdx.x;
     const int nchunk = (A.nx + V - 1) / V;
@@ -439,17 +449,19 @@ step_kernel(StepArgs A)
     const int ym = (y == 0) ? ny - 1 : y - 1;
     const int yp = (y == ny - 1) ? 0 : y + 1;
 
+    if constexpr (CG) lbmt::grid_dependency_wait();
+
     M P0[5][V], P1[5][V], P2[5][V], P3[5][V];   // pulled f_d (edge links patched below)
     M own0[5][V], own2[5][V];                    // f*_{(1,0)}, f*_{(-1,0)} of the own chunk
     const long long row = (long long)y * A.pitch + x0;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        vload<K, V>(src + (0 * 5 + k) * plane + row, own0[k]);
-        vload<K, V>(src + (2 * 5 + k) * plane + row, own2[k]);
-        if (bot) vload<K, V>(src + (3 * 5 + k) * plane + row, P1[k]);
-        else     vload<K, V>(src + (1 * 5 + k) * plane + (long long)ym * A.pitch + x0, P1[k]);
-        if (top) vload<K, V>(src + (1 * 5 + k) * plane + row, P3[k]);
-        else     vload<K, V>(src + (3 * 5 + k) * plane + (long long)yp * A.pitch + x0, P3[k]);
+        vload<K, V, CG>(src + (0 * 5 + k) * plane + row, own0[k]);
+        vload<K, V, CG>(src + (2 * 5 + k) * plane + row, own2[k]);
+        if (bot) vload<K, V, CG>(src + (3 * 5 + k) * plane + row, P1[k]);
+        else     vload<K, V, CG>(src + (1 * 5 + k) * plane + (long long)ym * A.pitch + x0, P1[k]);
+        if (top) vload<K, V, CG>(src + (1 * 5 + k) * plane + row, P3[k]);
+        else     vload<K, V, CG>(src + (3 * 5 + k) * plane + (long long)yp * A.pitch + x0, P3[k]);
     }
     // x-planes: shift by one node through the neighbouring lanes
     const int xl = (x0 == 0) ? nx - 1 : x0 - 1;        // source of P0[0]
@@ -460,8 +472,8 @@ step_kernel(StepArgs A)
     for (int k = 0; k < 5; ++k) {
         M l = __shfl_up_sync(0xffffffffu, own0[k][V - 1], 1);
         M r = __shfl_down_sync(0xffffffffu, own2[k][0], 1);
-        if (!left_in_lane) l = sload<K>(src + (0 * 5 + k) * plane + (long long)y * A.pitch + xl);
-        if (!right_in_lane) r = sload<K>(src + (2 * 5 + k) * plane + (long long)y * A.pitch + xr);
+        if (!left_in_lane) l = sload<K, CG>(src + (0 * 5 + k) * plane + (long long)y * A.pitch + xl);
+        if (!right_in_lane) r = sload<K, CG>(src + (2 * 5 + k) * plane + (long long)y * A.pitch + xr);
         P0[k][0] = l;
 #pragma unroll
         for (int e = 1; e < V; ++e) P0[k][e] = own0[k][e - 1];
@@ -474,7 +486,7 @@ step_kernel(StepArgs A)
         const int e = nx - 1 - x0;
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
-            const M r0 = sload<K>(src + (2 * 5 + k) * plane + (long long)y * A.pitch + 0);
+            const M r0 = sload<K, CG>(src + (2 * 5 + k) * plane + (long long)y * A.pitch + 0);
 #pragma unroll
             for (int q = 0; q < V; ++q)
                 if (q == e) P2[k][q] = r0;
@@ -488,6 +500,24 @@ step_kernel(StepArgs A)
     } else {
         a = A.a;
         b = A.b;
+    }
+    // body load of the reduced formats (FP32 tables): the factors of a row and of the time are read
+    // once per thread, not once per node
+    float bxf[V], byf[V];
+    if constexpr (FORCING && sizeof(M) == 4) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) bxf[e] = byf[e] = 0.f;
+        for (int r = 0; r < A.R; ++r) {
+            const float Y = A.Yf[(long long)r * ny + y], Tx = A.Tf[r], Ty = A.Tf[A.R + r];
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                if (x0 + e < nx) {
+                    const float xy = A.Xf[(long long)r * nx + x0 + e] * Y;
+                    bxf[e] = fmaf(xy, Tx, bxf[e]);
+                    byf[e] = fmaf(xy, Ty, byf[e]);
+                }
+            }
+        }
     }
     M out[4][5][V];
     double wv[2][V];
@@ -565,22 +595,19 @@ step_kernel(StepArgs A)
                 ry[k] = sx;
             }
             if (FORCING) {
-                // body load in the arithmetic type (FP32 tables for the reduced formats)
+                // body load in the arithmetic type
                 M bx = M(0), by = M(0);
-                if (x < nx) {
-                    if constexpr (sizeof(M) == 8) {
+                if constexpr (sizeof(M) == 8) {
+                    if (x < nx) {
                         for (int r = 0; r < A.R; ++r) {
                             const M xy = A.X[(long long)r * nx + x] * A.Y[(long long)r * ny + y];
                             bx = fma(xy, A.T[r], bx);
                             by = fma(xy, A.T[A.R + r], by);
                         }
-                    } else {
-                        for (int r = 0; r < A.R; ++r) {
-                            const M xy = A.Xf[(long long)r * nx + x] * A.Yf[(long long)r * ny + y];
-                            bx = fma(xy, A.Tf[r], bx);
-                            by = fma(xy, A.Tf[A.R + r], by);
-                        }
                     }
+                } else {
+                    bx = bxf[e];
+                    by = byf[e];
                 }
                 bxs[e] = (double)bx;
                 bys[e] = (double)by;
@@ -636,7 +663,7 @@ step_kernel(StepArgs A)
             double* wp = A.w + (long long)c * plane + row;
 #pragma unroll
             for (int e = 0; e < V; ++e)
-                if (x0 + e < nx) wp[e] = fma(A.dt, wv[c][e], wp[e]);
+                if (x0 + e < nx) wp[e] = fma(A.dt, wv[c][e], CG ? __ldcg(wp + e) : wp[e]);
         }
     }
 }

@@ -28,6 +28,11 @@ constexpr int K = LBM_KIND;
 constexpr bool MS = (K >= lbmk::K_MSBF16);
 // nodes per thread in the step kernel (one vector access per plane and thread)
 constexpr int V = (K == lbmk::K_F64) ? LBM_VEC_F64 : (K == lbmk::K_F32) ? LBM_VEC_F32 : MS ? 4 : LBM_VEC_F16;
+#ifndef LBM_VEC_STEP
+#define LBM_VEC_STEP 2
+#endif
+// nodes per thread of the single step (measured beside step_kernel)
+constexpr int VS = (K == lbmk::K_F64 || MS) ? V : LBM_VEC_STEP;
 constexpr int ELEM = (K == lbmk::K_F64) ? 8 : (K == lbmk::K_F32) ? 4 : 2;
 // nodes per thread in the batch kernel (FP64 runs the split collision, at its width)
 constexpr int VB = (K == lbmk::K_F64) ? LBM_VEC_SPLIT : V;
@@ -38,7 +43,8 @@ cudaError_t step_v(const lbmk::StepArgs& a, dim3 g, dim3 b, cudaStream_t s)
 {
     if constexpr (MS) lbmk::ms_step_kernel<K, V, D, F, T, O><<<g, b, 0, s>>>(a);
     else if constexpr (SPLIT > 0) lbmk::step_kernel<K, LBM_VEC_SPLIT, D, F, T, O, SPLIT><<<g, b, 0, s>>>(a);
-    else lbmk::step_kernel<K, V, D, F, T, O><<<g, b, 0, s>>>(a);
+    else if constexpr (K == lbmk::K_F64) lbmk::step_kernel<K, V, D, F, T, O><<<g, b, 0, s>>>(a);
+    else return lbmh::launch_dependent(lbmk::step_kernel<K, VS, D, F, T, O>, g, b, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -427,7 +433,7 @@ namespace lbmh {
 #define LBM_OPS_NAME(k) LBM_OPS_NAME2(k)
 
 const KindOps LBM_OPS_NAME(LBM_KIND) = {
-    K, V, ELEM, NODE_BYTES,
+    K, VS, ELEM, NODE_BYTES,
     step, init, moments, get_pop, set_pop, energy, error, finite, batch_step, batch_occupancy, tb2_step, tbp_step,
     tbpms_step, step_staged, step_multi, batch_tbp_step,
     LBM_VEC_SPLIT, VB,

@@ -88,3 +88,27 @@ def test_fp64_body_load_staged_equals_register_kernel(lbm, nx, ny, rows, dirichl
         states.append(_state(lat))
     np.testing.assert_array_equal(states[0][0], states[1][0])
     np.testing.assert_array_equal(states[0][1], states[1][1])
+
+
+# two nodes per thread, blocks of 64 threads: 128 columns per block
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 5), (127, 4), (128, 3), (129, 7), (257, 2), (1021, 9)])
+def test_fp32_arithmetic_with_body_load(lbm, nx, ny, dirichlet, storage):
+    """Steps launched one behind the other against a host wait after each (same words), and in FP32
+    against FP64: 12 steps of some ten roundings of 2^-24 of the largest population each."""
+    many = _lattice(lbm, nx, ny, dirichlet, storage, True)
+    many.step(12)
+    one = _lattice(lbm, nx, ny, dirichlet, storage, True)
+    for _ in range(12):
+        one.step(1)
+        one.synchronize()
+    a, b = _state(many), _state(one)
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+    if storage == "f32":
+        ref = _lattice(lbm, nx, ny, dirichlet, "f64", True)
+        ref.step(12)
+        f, us = _state(ref)
+        assert np.max(np.abs(a[0] - f)) < 120 * 2.0 ** -24 * np.max(np.abs(f))
+        assert np.max(np.abs(a[1] - us)) < 120 * 2.0 ** -24 * np.max(np.abs(us))
