@@ -927,55 +927,83 @@ __global__ void to_bf16_kernel(const float* __restrict__ x, long long n, __nv_bf
         y[i] = __float2bfloat16_rn(x[i]);
 }
 
-// (float)(u / s) given r = 1 / s rounded, without an FP64 division where the product decides: q = u r is
-// within two units in the last place of u / s, so both round to the same FP32 value unless q lies that
-// close to the middle between two of them (the 29 bits dropped near 2^28) or outside FP32's normal range.
+// (float)(u / s) given r = 1 / s rounded (0 where r is of no use), with one FP64 operation where the
+// product decides: q = u r is within two units in the last place of u / s, so both round to the same FP32
+// value unless q lies that close to the middle between two of them (the 29 bits dropped near 2^28) or
+// outside FP32's normal range.  The rounding and the tests are integer operations (two FP64 operations a
+// clock per SM, comparisons and conversions among them, bounded the loop).
 __device__ __forceinline__ float div_to_f32(double u, double s, double r)
 {
-    const double q = u * r, m = fabs(q);
-    const int low = (int)(__double2loint(q) & 0x1FFFFFFF) - 0x10000000;
-    if (m >= 2.4e-38 && m < 1.7e38 && (low > 8 || low < -8)) return (float)q;
+    const unsigned long long ub = (unsigned long long)__double_as_longlong(u), rb = (unsigned long long)__double_as_longlong(r);
+    const unsigned long long q = (unsigned long long)__double_as_longlong(u * r);
+    const unsigned sign = (unsigned)(q >> 32) & 0x80000000u;
+    const int e = (int)(q >> 52) & 0x7FF, low = (int)((unsigned)q & 0x1FFFFFFFu) - 0x10000000;
+    if (e >= 1023 - 125 && e <= 1023 + 126 && (low > 8 || low < -8))
+        return __uint_as_float(sign | ((unsigned)((q & 0x7FFFFFFFFFFFFFFFull) >> 29) - (896u << 23) + (low > 0 ? 1u : 0u)));
+    if ((ub << 1) == 0 && rb != 0) return __uint_as_float(sign);
     return (float)(u / s);
 }
 
 // network input: U fields [B][nf][H][W] (FP64, field-major per sample) scaled by 1/scale[c], plus a
-// constant channel per sample, into [B][H][W][C] FP32 with zero padding channels.  nf FP64 divisions per
-// pixel bounded it (16 x 256 x 256, 5 fields: 90 us before, 69 us so, at 26 us of memory traffic).
+// constant channel per sample, into [B][H][W][C] FP32 with zero padding channels.  A block takes 256
+// pixels: a thread per pixel computes its values (field reads coalesced across the warp) into shared
+// memory, up to 32 channels at a time, then the block writes whole lines.  Memory-bound (172 bytes per
+// pixel at 5 fields, C = 32: 26 us for 16 x 256 x 256): 90 us with nf FP64 divisions per pixel and
+// 16-byte stores a pixel apart, 69 without the divisions, 41 so.
+constexpr int kPackCh = 32;
+
 __global__ void __launch_bounds__(256) pack_input_kernel(const double* __restrict__ U, long long sample_stride, int nf,
                                                          const double* __restrict__ scale,
                                                          const float* __restrict__ extra, int B, int H, int W, int C,
                                                          float* __restrict__ x)
 {
-    // one thread per pixel: the nf fields (coalesced across the warp), the extra
-    // channel, zeros up to C; 16-byte stores when C is a multiple of 4
     __shared__ double rs[64];
+    __shared__ float val[kPackCh][256 + 1];
     for (int c = threadIdx.x; c < nf && c < 64; c += blockDim.x) {
         const double s = scale[c], r = 1.0 / s;
         rs[c] = fabs(s) >= 1e-290 && fabs(s) <= 1e290 ? r : 0.0;    // 0: every value takes the division
     }
-    __syncthreads();
     const long long HW = (long long)H * W;
     const long long npix = (long long)B * HW;
-    for (long long pix = blockIdx.x * (long long)blockDim.x + threadIdx.x; pix < npix;
-         pix += (long long)gridDim.x * blockDim.x) {
+    for (long long first = blockIdx.x * 256LL; first < npix; first += gridDim.x * 256LL) {
+        const long long pix = first + threadIdx.x;
         const long long b = pix / HW, q = pix - b * HW;
-        float* dst = x + pix * C;
-        const auto value = [&](int c) {
-            if (c >= nf) return c == nf && extra ? extra[b] : 0.f;
-            const double u = U[b * sample_stride + c * HW + q];
-            const double r = c < 64 ? rs[c] : 0.0;
-            if (u == 0.0 && r != 0.0) return (float)(u * r);        // the sign of a zero
-            return div_to_f32(u, scale[c], r);
-        };
-        if ((C & 3) == 0) {
-            for (int c0 = 0; c0 < C; c0 += 4) {
-                float v[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = value(c0 + e);
-                *reinterpret_cast<float4*>(dst + c0) = make_float4(v[0], v[1], v[2], v[3]);
+        const int n = (int)min(256LL, npix - first);
+        for (int c0 = 0; c0 < C; c0 += kPackCh) {
+            const int nc = min(kPackCh, C - c0);
+            const int used = max(0, min(nc, nf + 1 - c0));           // channels that are not padding
+            __syncthreads();
+            if (pix < npix) {
+                for (int k = 0; k < used; ++k) {
+                    const int c = c0 + k;
+                    float v;
+                    if (c >= nf) {
+                        v = extra ? extra[b] : 0.f;
+                    } else {
+                        const double u = U[b * sample_stride + c * HW + q];
+                        v = div_to_f32(u, scale[c], c < 64 ? rs[c] : 0.0);
+                    }
+                    val[k][threadIdx.x] = v;
+                }
             }
-        } else {
-            for (int c = 0; c < C; ++c) dst[c] = value(c);
+            __syncthreads();
+            if ((C & 3) == 0) {
+                const int n4 = nc / 4;
+                for (int i = threadIdx.x; i < n * n4; i += 256) {
+                    const int p = i / n4, k = (i - p * n4) * 4;
+                    float4 v;
+                    v.x = k < used ? val[k][p] : 0.f;
+                    v.y = k + 1 < used ? val[k + 1][p] : 0.f;
+                    v.z = k + 2 < used ? val[k + 2][p] : 0.f;
+                    v.w = k + 3 < used ? val[k + 3][p] : 0.f;
+                    *reinterpret_cast<float4*>(x + (first + p) * C + c0 + k) = v;
+                }
+            } else {
+                for (int i = threadIdx.x; i < n * nc; i += 256) {
+                    const int p = i / nc, k = i - p * nc;
+                    x[(first + p) * C + c0 + k] = k < used ? val[k][p] : 0.f;
+                }
+            }
         }
     }
 }

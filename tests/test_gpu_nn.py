@@ -409,3 +409,21 @@ def test_pack_input_rounds_like_the_division(lbm):
     assert torch.equal(x[..., :nf].contiguous().view(torch.int32)[~ref.isnan()], ref.contiguous().view(torch.int32)[~ref.isnan()])
     assert torch.equal(x[..., :nf].isnan(), ref.isnan())
     assert torch.equal(x[..., nf], torch.ones_like(x[..., nf])) and not x[..., nf + 1:].any()
+
+
+@pytest.mark.parametrize("B,H,W,nf,C,extra", [(1, 3, 5, 5, 6, True), (2, 7, 37, 3, 3, False), (3, 16, 32, 33, 40, True),
+                                              (1, 1, 257, 5, 34, False)])
+def test_pack_input_sizes(lbm, B, H, W, nf, C, extra):
+    """Part of a block of 256 pixels, blocks across samples, more than 32 channels, no padding, odd C."""
+    import torch
+    from paper_2408_01081_gb300 import nn as K
+    U = torch.randn((B, nf + 2, H, W), dtype=torch.float64, device="cuda")
+    scale = torch.rand(nf, dtype=torch.float64, device="cuda") + 0.5
+    e = torch.randn(B, dtype=torch.float32, device="cuda") if extra else None
+    x = torch.full((B, H, W, C), 3.0, dtype=torch.float32, device="cuda")
+    K.pack_input(U, (nf + 2) * H * W, nf, scale, e, B, H, W, C, x)
+    ref = torch.zeros_like(x)
+    ref[..., :nf] = (U[:, :nf] / scale[:, None, None]).float().permute(0, 2, 3, 1)
+    if extra:
+        ref[..., nf] = e[:, None, None]
+    assert torch.equal(x, ref)
