@@ -577,8 +577,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // are taps.  The tap dx is B started dx pixels further on, each with its own accumulator D_dx (128
 // columns).  Per row pair and dx three MMAs: dY_hi X_hi + dY_hi X_lo + dY_lo X_hi.
 //
-// What bounds it: 72 MMAs of 64 clocks per block (M = 64 takes as long as 128): 33 us of the 43 us that
-// 32 x 32 channels take at 8 x 256 x 256 (20 us of memory traffic).  The mma.sync kernel before, one warp
+// What bounds it: 72 MMAs of 64 clocks per block (M = 64 takes as long as 128): 33 us of the 50 us that
+// 32 x 32 channels take at 8 x 256 x 256 (20 us of memory traffic; 43 us with one part per range).  The mma.sync kernel before, one warp
 // per tap reading its fragments with ldmatrix, took 104 us there at half of mma.sync's rate (47 us);
 // 384 -> 128 channels at 16 x 64 x 64, whole layer: 855 -> 377 us.
 // Sixteen warps load, split into BF16 halves and stage a block while the MMAs of the one before run.
