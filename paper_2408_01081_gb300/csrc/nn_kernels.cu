@@ -4,10 +4,10 @@
 // and every convolution pads circularly (the lattices are periodic).  Weights
 // are BF16, [Cout][KS][KS][Cin], with FP32 master copies for the optimiser.
 //
-// 3x3 forward convolutions go to the tcgen05 kernel of nn_conv_tc.cu where its tiling
-// applies; the kernels here are implicit GEMMs with mma.sync m16n8k16 (BF16 inputs,
-// FP32 accumulation) for the forward sizes that tiling does not take (the data
-// gradient is a forward convolution too) and for the weight gradients.  An FP32
+// 3x3 convolutions and their weight gradients go to the tcgen05 kernels of nn_conv_tc.cu
+// where their tilings apply; the kernels here are implicit GEMMs with mma.sync m16n8k16
+// (BF16 inputs, FP32 accumulation) for the sizes those do not take (the data
+// gradient is a forward convolution too).  An FP32
 // activation a is split into
 // a_hi = bf16(a) and a_lo = bf16(a - a_hi); products use both halves, so the
 // only rounding of the forward pass is the BF16 weights themselves:
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(256) conv_wgrad_kernel(WgradArgs a)
 // Sum the split partials into dW (FP32) in a fixed order.  A block takes 32 consecutive elements;
 // its warps take every 8th split each (a 128-byte line per load) and their sums are added in warp
 // order.  One thread per element walked all splits before: 32 -> 32 channels has 9216 elements and
-// up to 600 splits, 36 blocks of dependent loads, 55 us for 19 MB; 6 us so.
+// up to 600 splits, 36 blocks of dependent loads, 55 us for 19 MB; 9 us so.
 __global__ void __launch_bounds__(256) sum_splits_kernel(const float* __restrict__ partial, int splits, long long n,
                                                          float* __restrict__ out, int beta)
 {
