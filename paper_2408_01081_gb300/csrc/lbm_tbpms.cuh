@@ -4,8 +4,18 @@
 // is the rebuilding of a row's populations, done once per node, and level l + 1 is pulled from
 // level l's last three rows exactly as there (shuffles for the x-neighbours at every level, so a
 // warp loses one column per level and side: 56 of its 64 columns are stored).  The last level is
-// stored as moments; nothing in between is rounded to 16 bits.  Same operations as the scalar
-// kernel of one column per thread that this one replaces, hence the same words.
+// stored as moments; nothing in between is rounded to 16 bits.
+//
+// Words.  The words a pass stores are those of the scalar kernel that came before this one, whose
+// roundings the compiler chose: every sum with one product fused, but (all formats except periodic
+// block floating point) Phi_x[4] = b m0[1] and Phi_y[3] = -b m0[1], one product used twice, rounded
+// before the deviation was added.  Its warps each took 28 columns (30 in the two-step kernel) and
+// rebuilt f_x of the columns just outside their halo alone, with that sum fused: so at each seam
+// (a column c that is a multiple of 28, of 30 in two steps) the value pulled into c from the left and
+// into c - 1 from the right starts from a fused Phi_x[4] + dx[4] three (two) columns away.  Only
+// components 1 and 4 of those two chains differ (tbpms_seam_update); the last level takes them at the
+// seams.  Without them the 16-bit roundings part from there on within a few hundred steps: the fields
+// of a run differ by as much as the format's own error (1e-5).  About a tenth more instructions.
 //
 // What bounds it: instruction issue (decoding, rebuilding, encoding).  One column per thread took
 // about 470 thread instructions per node and step in block floating point at 3 blocks per SM.
@@ -109,9 +119,15 @@ template <> struct PairCodec<MsBfpCodec> {
     }
 };
 
-// populations of two columns from their moments (ms_dir)
+// populations of two columns from their moments (ms_dir).  SPLIT (see tbpms_compute): Phi_x[4] =
+// b m0[1] and Phi_y[3] = -b m0[1] are rounded before the deviation is added, and f0h, f2h return
+// f[0][4], f[2][4] with the fused sum instead; else every sum with one product is fused.  The
+// separate roundings are scalar: a packed product and a packed sum are merged into one packed
+// multiply-add whatever their rounding modifiers (seen in the results).
+template <bool SPLIT>
 __device__ __forceinline__ void tbpms_rebuild(const f32x2 (&m0)[5], const f32x2 (&dx)[5], const f32x2 (&dy)[5],
-                                              const f32x2 (&dd)[5], const TbpConst& C, f32x2 (&f)[4][5])
+                                              const f32x2 (&dd)[5], const TbpConst& C, f32x2 (&f)[4][5], f32x2& f0h,
+                                              f32x2& f2h)
 {
     const f32x2 two = dup2(2.f), mtwo = dup2(-2.f), quarter = dup2(.25f);
     // T = Phi/c + deviation, per axis
@@ -126,12 +142,40 @@ __device__ __forceinline__ void tbpms_rebuild(const f32x2 (&m0)[5], const f32x2 
     ty[2] = fma2(C.a, m0[1], dy[2]);
     ty[3] = fma2(C.nb, m0[1], dy[3]);
     ty[4] = fma2(C.b, m0[0], dy[4]);
+    if (SPLIT) {
+        f0h = mul2(quarter, add2(fma2(two, tx[4], m0[4]), dd[4]));
+        f2h = mul2(quarter, add2(fma2(mtwo, tx[4], m0[4]), dd[4]));
+        const float pl = __fmul_rn(lo_of(C.b), lo_of(m0[1])), ph = __fmul_rn(lo_of(C.b), hi_of(m0[1]));
+        tx[4] = pk(__fadd_rn(pl, lo_of(dx[4])), __fadd_rn(ph, hi_of(dx[4])));
+        ty[3] = pk(__fsub_rn(lo_of(dy[3]), pl), __fsub_rn(hi_of(dy[3]), ph));
+    }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
         f[0][k] = mul2(quarter, add2(fma2(two, tx[k], m0[k]), dd[k]));
         f[2][k] = mul2(quarter, add2(fma2(mtwo, tx[k], m0[k]), dd[k]));
         f[1][k] = mul2(quarter, fma2(C.m1, dd[k], fma2(two, ty[k], m0[k])));
         f[3][k] = mul2(quarter, fma2(C.m1, dd[k], fma2(mtwo, ty[k], m0[k])));
+    }
+}
+
+// Components 1 and 4 of the directions (1,0) and (-1,0) of tbp_update with X0, X2 in the place of
+// x0, x2 in those components ([0]: component 1, [1]: component 4; the others do not enter)
+template <bool NEG>
+__device__ __forceinline__ void tbpms_seam_update(const TbpConst& C, const f32x2 (&X0)[2], const f32x2 (&x1)[5],
+                                                  const f32x2 (&X2)[2], const f32x2 (&x3)[5], f32x2 (&o0)[2],
+                                                  f32x2 (&o2)[2])
+{
+    f32x2 rx[2], U[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int k = j ? 4 : 1;
+        rx[j] = NEG ? fma2(C.m1, x1[k], x3[k]) : add2(x1[k], x3[k]);
+        U[j] = add2(rx[j], NEG ? fma2(C.m1, X0[j], X2[j]) : add2(X0[j], X2[j]));
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        o0[j] = fma2(NEG ? C.h : C.nh, U[j], fma2(NEG ? C.b : C.nb, U[1 - j], X0[j]));
+        o2[j] = NEG ? fma2(C.m1, o0[j], rx[j]) : add2(rx[j], o0[j]);
     }
 }
 
@@ -210,6 +254,8 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
     using G = TbpMsGeom;
     using Codec = PairCodec<typename Ms<K>::C>;
     constexpr int NST = G::NST, WIN = G::WIN;
+    constexpr bool SPLIT = !(K == K_MSBFP && !DIRICHLET);
+    constexpr int SEAM = NL == 3 ? 28 : 30;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nx = A.nx, ny = A.ny;
     const int nin = (y1 - y0) + 2 * NL;
@@ -245,6 +291,13 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
     const bool wl = EDGE && DIRICHLET && xs == 0;
     const bool wr0 = EDGE && DIRICHLET && xs == nx - 1, wr1 = EDGE && DIRICHLET && xs + 1 == nx - 1;
 
+    // The columns of a seam (header) this lane holds: c - 1 in its upper half, c in its lower half
+    const bool seam_r = SPLIT && (xs + 2) % SEAM == 0, seam_l = SPLIT && xs % SEAM == 0;
+    // [level][0, 1]: components 1, 4 that the level's seam update reads (level 0: component 4 only)
+    f32x2 seam[NL - 1][2];
+#pragma unroll
+    for (int l = 0; l < NL - 1; ++l) seam[l][0] = seam[l][1] = 0ull;
+
     // per level as in tbp_compute; level 0 is the rebuilt state itself
     f32x2 s0[NL][5], s2[NL][5], k1[NL][5], c1[NL][5];
 #pragma unroll
@@ -261,7 +314,7 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
         const bool ok = lbmt::mbar_wait(lbmt::smem_u32(&full_bar[st]), ph, abort_flag);
         if (!__all_sync(0xffffffffu, ok)) break;
         const uint32_t sb = sbase + st * G::STAGE_BYTES;
-        f32x2 cur[4][5];
+        f32x2 cur[4][5], sr[2], sl[2];                     // sr, sl: the seam values of cur (directions 0, 2)
         {
             f32x2 m0[5], dx[5], dy[5], dd[5];
 #pragma unroll
@@ -281,7 +334,7 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
                 }
                 Codec::decode(w[0], w[1], w[2], A.inv_s, dx[k], dy[k], dd[k]);
             }
-            tbpms_rebuild(m0, dx, dy, dd, C, cur);
+            tbpms_rebuild<SPLIT>(m0, dx, dy, dd, C, cur, sr[1], sl[1]);
         }
         __syncwarp();
         if (lane == 0) lbmt::mbar_arrive(lbmt::smem_u32(&empty_bar[st]));
@@ -294,7 +347,7 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
         for (int l = 0; l < NL; ++l) {
             const int q = R - 1 - l;
             const bool neg = (l & 1) != 0;                 // cur[0], cur[1], s0, k1, c1 hold -f
-            f32x2 out[4][5];
+            f32x2 out[4][5], nr[2], nl[2];
             {
                 f32x2 x3[5];
 #pragma unroll
@@ -304,11 +357,44 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
                     for (int k = 0; k < 5; ++k) x3[k] = ((k < 2) != neg) ? neg2(c1[l][k]) : c1[l][k];
                 if (neg) tbp_update<true>(C, s0[l], k1[l], s2[l], x3, out);
                 else tbp_update<false>(C, s0[l], k1[l], s2[l], x3, out);
+                if (SPLIT && l < NL - 1) {
+                    // level 1 of three: column c - 2 (lower half) pulls the seam value rightwards, c + 1
+                    // (upper) leftwards; the level before the last: c - 1 (upper), c (lower)
+                    const bool outer = NL == 3 && l == 0;
+                    f32x2 p0[2], p2[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int k = j ? 4 : 1;
+                        const f32x2 v = seam[l][j];
+                        p0[j] = s0[l][k];
+                        p2[j] = s2[l][k];
+                        if (l == 0 && j == 0) continue;
+                        if (outer) {
+                            p0[j] = pk(lo_of(v), hi_of(p0[j]));
+                            if (!wr1) p2[j] = pk(lo_of(p2[j]), hi_of(v));
+                        } else {
+                            p0[j] = pk(lo_of(p0[j]), hi_of(v));
+                            if (!wr0) p2[j] = pk(lo_of(v), hi_of(p2[j]));
+                        }
+                    }
+                    if (neg) tbpms_seam_update<true>(C, p0, k1[l], p2, x3, nr, nl);
+                    else tbpms_seam_update<false>(C, p0, k1[l], p2, x3, nr, nl);
+                }
             }
+            if (SPLIT && l == 0 && NL == 3)
+                seam[0][1] = pk(__shfl_up_sync(0xffffffffu, hi_of(sr[1]), 1), __shfl_down_sync(0xffffffffu, lo_of(sl[1]), 1));
+            else if (SPLIT && l < NL - 1)
+#pragma unroll
+                for (int j = l == 0 ? 1 : 0; j < 2; ++j) seam[l][j] = pk(hi_of(sl[j]), lo_of(sr[j]));
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                const float up = __shfl_up_sync(0xffffffffu, hi_of(cur[0][k]), 1);
-                const float dn = __shfl_down_sync(0xffffffffu, lo_of(cur[2][k]), 1);
+                float r0 = hi_of(cur[0][k]), l2 = lo_of(cur[2][k]);
+                if (SPLIT && l == NL - 1 && (k == 1 || k == 4)) {
+                    if (seam_r) r0 = hi_of(sr[k / 4]);
+                    if (seam_l) l2 = lo_of(sl[k / 4]);
+                }
+                const float up = __shfl_up_sync(0xffffffffu, r0, 1);
+                const float dn = __shfl_down_sync(0xffffffffu, l2, 1);
                 s0[l][k] = pk(up, lo_of(cur[0][k]));
                 s2[l][k] = pk(hi_of(cur[2][k]), dn);
                 if (EDGE && DIRICHLET) {
@@ -327,6 +413,12 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
             for (int d = 0; d < 4; ++d)
 #pragma unroll
                 for (int k = 0; k < 5; ++k) cur[d][k] = out[d][k];
+            if (SPLIT && l < NL - 1)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    sr[j] = nr[j];
+                    sl[j] = nl[j];
+                }
         }
         const int q = R - NL;
         if (q >= y0) {
