@@ -403,10 +403,12 @@ __global__ void __launch_bounds__(256, 2) ms_step_kernel(StepArgs A)
         }
         float m0[5], dx[5], dy[5], dd[5];
         ms_moments(o, fa, fb, m0, dx, dy, dd);
+        // block floating point: the last thread's nodes beyond the row must not count as saturated
+        const float se = Codec::kJoint && x >= nx ? 0.f : sc;
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
             m0o[k][e] = m0[k];
-            Codec::encode(dx[k] * sc, dy[k] * sc, dd[k] * sc, wxo[k][e], wyo[k][e], wzo[k][e], sat);
+            Codec::encode(dx[k] * se, dy[k] * se, dd[k] * se, wxo[k][e], wyo[k][e], wzo[k][e], sat);
         }
         if (TRACK) {
             wv[0][e] = (double)U[0];

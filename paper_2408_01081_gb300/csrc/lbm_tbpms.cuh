@@ -54,7 +54,7 @@ template <int H> struct PairCodec<MsFloatCodec<H>> {
         return (uint32_t)Fmt<H>::st(a) | ((uint32_t)Fmt<H>::st(b) << 16);
     }
     static __device__ __forceinline__ void encode(f32x2 x, f32x2 y, f32x2 z, uint32_t& wx, uint32_t& wy, uint32_t& wz,
-                                                  bool&)
+                                                  bool&, bool&)
     {
         wx = word(x);
         wy = word(y);
@@ -105,12 +105,13 @@ template <> struct PairCodec<MsBfpCodec> {
         const uint32_t p = (uint32_t)(unsigned short)i | ((uint32_t)(unsigned short)j << 16);
         return __vmaxs2(__vmins2(p, 0x3FFF3FFFu), 0xC001C001u);
     }
+    // satl, sath: set when the lower / upper column's block saturated
     static __device__ __forceinline__ void encode(f32x2 x, f32x2 y, f32x2 z, uint32_t& wx, uint32_t& wy, uint32_t& wz,
-                                                  bool& sat)
+                                                  bool& satl, bool& sath)
     {
         float fl, fh;
-        const uint32_t el = block(lo_of(x), lo_of(y), lo_of(z), fl, sat);
-        const uint32_t eh = block(hi_of(x), hi_of(y), hi_of(z), fh, sat);
+        const uint32_t el = block(lo_of(x), lo_of(y), lo_of(z), fl, satl);
+        const uint32_t eh = block(hi_of(x), hi_of(y), hi_of(z), fh, sath);
         const uint32_t t = (el >> 23) | (eh >> 7);                     // e of both columns in bits 0.., 16..
         const f32x2 f = pk(fl, fh);
         wx = ((mants(x, f) << 1) & 0xFFFEFFFEu) | (t & 0x00010001u);
@@ -433,11 +434,11 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
             if (out_lane) {
                 const f32x2 sc = dup2(A.scale);
                 const long long off = (long long)q * A.pitch + xs;
-                bool clip = false;
+                bool clipl = false, cliph = false;
 #pragma unroll
                 for (int k = 0; k < 5; ++k) {
                     uint32_t w[3];
-                    Codec::encode(mul2(dx[k], sc), mul2(dy[k], sc), mul2(dd[k], sc), w[0], w[1], w[2], clip);
+                    Codec::encode(mul2(dx[k], sc), mul2(dy[k], sc), mul2(dd[k], sc), w[0], w[1], w[2], clipl, cliph);
                     if (both) {
                         *reinterpret_cast<f32x2*>(m0p + k * A.plane + off) = m0[k];
 #pragma unroll
@@ -449,7 +450,7 @@ __device__ __forceinline__ void tbpms_compute(const TbpMsArgs& A, int X0, int y0
                         for (int j = 0; j < 3; ++j) dvp[(5 * j + k) * A.plane + off] = (unsigned short)(w[j] & 0xFFFFu);
                     }
                 }
-                sat |= clip;
+                sat |= clipl || (both && cliph);           // column nx of an odd width is not stored
             }
         }
     }
