@@ -691,34 +691,47 @@ __global__ void __launch_bounds__(256) relu_bias_partial_kernel(float4* __restri
     const int rows = 256 / C4;
     const int c = t % C4, r = t / C4;
     const long long p0 = blockIdx.x * ppb, p1 = min(P, p0 + ppb);
+    auto add = [](float4& u, const float4& v) {
+        u.x += v.x;
+        u.y += v.y;
+        u.z += v.z;
+        u.w += v.w;
+    };
+    auto take = [&](long long p, float4& u) {     // mask one value and add it
+        const long long i = p * C4 + c;
+        const float4 a = y[i];
+        float4 v = dy[i];
+        if (!(a.x > 0.f)) v.x = 0.f;
+        if (!(a.y > 0.f)) v.y = 0.f;
+        if (!(a.z > 0.f)) v.z = 0.f;
+        if (!(a.w > 0.f)) v.w = 0.f;
+        dy[i] = v;
+        add(u, v);
+    };
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < rows) {
+    if (r < rows && rows >= 4) {
 #pragma unroll 4
-        for (long long p = p0 + r; p < p1; p += rows) {
-            const long long i = p * C4 + c;
-            const float4 a = y[i];
-            float4 v = dy[i];
-            if (!(a.x > 0.f)) v.x = 0.f;
-            if (!(a.y > 0.f)) v.y = 0.f;
-            if (!(a.z > 0.f)) v.z = 0.f;
-            if (!(a.w > 0.f)) v.w = 0.f;
-            dy[i] = v;
-            s.x += v.x;
-            s.y += v.y;
-            s.z += v.z;
-            s.w += v.w;
+        for (long long p = p0 + r; p < p1; p += rows) take(p, s);
+    } else if (r < rows) {                        // more than 256 channels: four sums a thread, or its chain of
+        float4 s1 = s, s2 = s, s3 = s;            // additions would be two to four times as long
+        long long p = p0 + r;
+        for (; p + 3 * rows < p1; p += 4 * rows) {
+            take(p, s);
+            take(p + rows, s1);
+            take(p + 2 * rows, s2);
+            take(p + 3 * rows, s3);
         }
+        for (; p < p1; p += rows) take(p, s);
+        add(s, s1);
+        add(s2, s3);
+        add(s, s2);
     }
     red[t] = s;
     for (int n = rows; n > 1;) {                  // rows added in pairs: rounding grows with their logarithm
         const int h = (n + 1) / 2;
         __syncthreads();
         if (r < n - h) {
-            const float4 b = red[t + h * C4];
-            s.x += b.x;
-            s.y += b.y;
-            s.z += b.z;
-            s.w += b.w;
+            add(s, red[t + h * C4]);
             red[t] = s;
         }
         n = h;
