@@ -232,7 +232,7 @@ def batch_accounting(mode, storage, descs, steps, ntiles_one_step, passes_per_gr
 
     Bytes: one read and one write of the state per launch (FP32 160 B per node, FP64 320); mode 2
     runs 33 three-step passes and one single step per 100 steps, or passes_per_graph passes.  Launches: mode 1 one per graph,
-    mode 2 two per pass (periodic and Dirichlet tiles) and one per single step, mode 3 one per step
+    mode 2 one per pass with passes_per_graph (two without: periodic and Dirichlet tiles) and one per single step, mode 3 one per step
     and boundary kind present (every lattice of the benchmark's workload has cK/c and cmu/c in
     [2^-60, 1/2), so all take the fixed-point update, whose lists are the two used).  Tiles: the
     library's one-step work-list (modes 0 and 1, `ntiles_one_step`), else the mode's own tiles,
@@ -243,7 +243,7 @@ def batch_accounting(mode, storage, descs, steps, ntiles_one_step, passes_per_gr
         passes, singles = passes_per_graph * steps // 100, 0
     bpn = (320 if storage == "f64" else 160) * (passes + singles) / steps
     kinds = len({d[2] for d in descs})
-    launches = {1: steps // 100, 2: 2 * passes + singles, 3: kinds * steps}.get(mode, steps)
+    launches = {1: steps // 100, 2: (1 if passes_per_graph is not None else 2) * passes + singles, 3: kinds * steps}.get(mode, steps)
     tile_shape = {2: (112, 12), 3: (128, 4)}.get(mode)
     tiles = ntiles_one_step if tile_shape is None else sum(
         math.ceil(d[0] / tile_shape[0]) * math.ceil(d[1] / tile_shape[1]) for d in descs)
@@ -303,8 +303,7 @@ def run_batch(args, lbm, torch, stream, dev, max_over_ranks, barrier, ws):
             "nodes": nodes, "steps": steps, "ms_per_step": round(ms, 4),
             "mlups": round(nodes * ws / (ms * 1e-3) / 1e6, 1),
             "mode": {0: "launch per step", 1: "persistent",
-                     2: "several steps per pass (tiles with staged rows), one launch each for periodic and "
-                        "Dirichlet tiles",
+                     2: "several steps per pass (tiles with staged rows), one launch over all tiles",
                      3: "FP64 tiles with staged rows, one launch per step each for periodic and Dirichlet "
                         "tiles"}[mode],
             "graph_replays": steps // 100, "gpu_launches": launches,

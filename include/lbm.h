@@ -365,12 +365,11 @@ lbm_status lbm_batch_tune(lbm_batch* b, const char* cache_path);
 /* Launch mode: 0 = one launch per step; 1 = one persistent launch per
  * `graph_steps` steps with a grid barrier between steps (cooperative launch);
  * 2 = several steps per pass, up to four in FP32 and three in BF16 / FP16 (these
- * storages only, LBM_ERR_ARG otherwise): every lattice is cut into tiles of 168 (FP32)
- * or 240 (16-bit) columns and 2 to 96 rows (from the batch's sizes),
+ * storages only, LBM_ERR_ARG otherwise): every lattice is cut into tiles of 168 columns
+ * and 2 to 96 rows (from the batch's sizes),
  * one block per tile stages the tile's input rows with tensor copies and keeps the
  * intermediate steps on chip (the single-lattice multi-step kernel of
- * lbm_set_step_fusion), one launch for the periodic and one for the Dirichlet
- * tiles per pass; FP32 steps are grouped into passes of equal length, 16-bit steps
+ * lbm_set_step_fusion), one launch over all tiles per pass; FP32 steps are grouped into passes of equal length, 16-bit steps
  * beyond a multiple of three run as mode 0;
  * 3 = one step per launch on staged rows (FP64 storage only, LBM_ERR_ARG otherwise):
  * tiles of 128 columns and 4 rows (2 for a lattice on the level-1 sequence), one

@@ -114,7 +114,7 @@ struct lbm_batch {
     lbmk::BatchLatT3* d_lat3 = nullptr;
     CUtensorMap* d_maps = nullptr;        // [lattice][arena][2]: row map, wrap map
     int4* d_t3 = nullptr;                 // periodic tiles, then Dirichlet tiles
-    int nt3[2] = {0, 0};                  // tile counts: periodic, Dirichlet
+    int nt3 = 0;                          // tiles
     // mode 3: FP64 on staged rows, one step per launch (lbm_batch_f64.cu)
     bool f64s_ok = false;                 // tile lists built (FP64 storage)
     int4* d_f64s = nullptr;               // the four lists, one after the other
@@ -190,11 +190,11 @@ lbm_status setup_t3(lbm_batch* b)
 {
     if (b->storage != LBM_F32 && b->storage != LBM_BF16 && b->storage != LBM_F16) return LBM_OK;
     const int es = b->ops->elem_bytes;
-    const int win = es == 4 ? lbmk::TbpGeom<4>::WIN : lbmk::TbpGeom<2>::WIN;
-    const int wrap = es == 4 ? lbmk::TbpGeom<4>::WRAP : lbmk::TbpGeom<2>::WRAP;
-    const int out = es == 4 ? lbmk::TbpGeom<4>::OUT : lbmk::TbpGeom<2>::OUT;
-    // rows per tile: the rule of single lattices over all tiles (two launches of about half each)
-    const int resident = 152 * (es == 4 ? lbmk::TbpGeom<4>::MIN_BLOCKS : lbmk::TbpGeom<2>::MIN_BLOCKS);
+    const int win = es == 4 ? lbmk::TbpGeom<4, true>::WIN : lbmk::TbpGeom<2, true>::WIN;
+    const int wrap = es == 4 ? lbmk::TbpGeom<4, true>::WRAP : lbmk::TbpGeom<2, true>::WRAP;
+    const int out = es == 4 ? lbmk::TbpGeom<4, true>::OUT : lbmk::TbpGeom<2, true>::OUT;
+    // rows per tile: the rule of single lattices over all tiles
+    const int resident = 152 * (es == 4 ? lbmk::TbpGeom<4, true>::MIN_BLOCKS : lbmk::TbpGeom<2, true>::MIN_BLOCKS);
     int ny_max = 0;
     for (const lbmk::LatDesc& L : b->lat) ny_max = std::max(ny_max, L.ny);
     b->t3_rows = lbmk::tbp_rows(resident, ny_max, [&](int r) {
@@ -224,12 +224,11 @@ lbm_status setup_t3(lbm_batch* b)
         q.bf = (float)L.b;
         q.pad_ = 0;
         for (int y = 0; y < L.ny; y += b->t3_rows)
-            for (int x = 0; x < L.nx; x += out) tiles[L.bc ? 1 : 0].push_back(make_int4(i, x, y, 0));
+            for (int x = 0; x < L.nx; x += out) tiles[L.bc ? 1 : 0].push_back(make_int4(i, x, y, L.bc ? 1 : 0));
     }
-    b->nt3[0] = (int)tiles[0].size();
-    b->nt3[1] = (int)tiles[1].size();
     std::vector<int4> all(tiles[0]);
     all.insert(all.end(), tiles[1].begin(), tiles[1].end());
+    b->nt3 = (int)all.size();
     B_CUDA(b, cudaMalloc((void**)&b->d_lat3, l3.size() * sizeof(lbmk::BatchLatT3)));
     B_CUDA(b, cudaMalloc((void**)&b->d_maps, maps.size() * sizeof(CUtensorMap)));
     B_CUDA(b, cudaMalloc((void**)&b->d_t3, std::max<size_t>(1, all.size()) * sizeof(int4)));
@@ -298,14 +297,14 @@ lbmk::BatchArgs batch_args(const lbm_batch* b, int steps, int parity)
     return A;
 }
 
-// Mode 2: launch pairs (one arena swap each) that make `steps` steps.  FP32 results do not depend
+// Mode 2: launches (one arena swap each) that make `steps` steps.  FP32 results do not depend
 // on how the steps are grouped: the fewest passes, of equal length, one more where the number of
 // swaps has to be even (a graph).  The 16-bit formats round once per pass: passes of three steps,
 // then single steps (an even number of swaps exactly when `steps` is even).
 long long mode2_passes(const lbm_batch* b, long long steps, bool even)
 {
     if (b->storage != LBM_F32) return steps / 3 + steps % 3;
-    const long long count = (steps + lbmk::TbpGeom<4>::NLMAX - 1) / lbmk::TbpGeom<4>::NLMAX;
+    const long long count = (steps + lbmk::TbpGeom<4, true>::NLMAX - 1) / lbmk::TbpGeom<4, true>::NLMAX;
     return even && (count & 1) ? count + 1 : count;
 }
 
@@ -316,7 +315,7 @@ int mode2_pass(const lbm_batch* b, long long steps, long long count, long long p
     return lbmk::tbp_pass(steps, count, p);
 }
 
-// arena swaps of `steps` steps outside a graph: one per launch or launch pair
+// arena swaps of `steps` steps outside a graph: one per launch (mode 3: per step)
 int swaps_of(const lbm_batch* b, long long steps)
 {
     return (int)((b->mode == 2 ? mode2_passes(b, steps, false) : steps) & 1);
@@ -350,8 +349,9 @@ cudaError_t enqueue_steps(lbm_batch* b, int steps, int parity, bool even)
     }
     int i = 0;
     if (b->mode == 2) {
-        // several steps per pass: the periodic tiles and the Dirichlet tiles, one launch each
+        // several steps per pass, one launch over all tiles
         lbmk::BatchTbpArgs T;
+        T.tiles = b->d_t3;
         T.lat = b->d_lat3;
         T.maps = b->d_maps;
         T.arenaA = b->arena[0];
@@ -363,11 +363,7 @@ cudaError_t enqueue_steps(lbm_batch* b, int steps, int parity, bool even)
             const int k = mode2_pass(b, steps, count, p);
             if (k < 2) break;                  // single steps: below
             T.parity = parity;
-            T.tiles = b->d_t3;
-            cudaError_t e = b->ops->batch_tbp_step(T, k, false, b->nt3[0], b->s);
-            if (e != cudaSuccess) return e;
-            T.tiles = b->d_t3 + b->nt3[0];
-            e = b->ops->batch_tbp_step(T, k, true, b->nt3[1], b->s);
+            cudaError_t e = b->ops->batch_tbp_step(T, k, b->nt3, b->s);
             if (e != cudaSuccess) return e;
             parity ^= 1;
             i += k;

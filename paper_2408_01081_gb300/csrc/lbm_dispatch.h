@@ -109,9 +109,9 @@ struct KindOps {
     // cudaErrorNotSupported for other formats and for lattices that one launch per step serves better
     cudaError_t (*step_multi)(const lbmk::StepArgs&, int variant, int steps, unsigned int* flags, int max_flags,
                               int* timeout, cudaStream_t s);
-    // three fused steps over the tiles of a batch (FP32 / BF16 / FP16; others return
-    // cudaErrorNotSupported): `ntiles` blocks, all of periodic or all of Dirichlet lattices
-    cudaError_t (*batch_tbp_step)(const lbmk::BatchTbpArgs&, int steps, bool dirichlet, int ntiles, cudaStream_t s);
+    // several fused steps over the tiles of a batch (FP32 two to four, BF16 / FP16 three; others
+    // return cudaErrorNotSupported): `ntiles` blocks
+    cudaError_t (*batch_tbp_step)(const lbmk::BatchTbpArgs&, int steps, int ntiles, cudaStream_t s);
     int vec_split;                 // nodes per thread of the FP64 split-level step kernels
     int batch_vec;                 // nodes per thread of the batch kernel
 };

@@ -390,34 +390,33 @@ cudaError_t tbpms_step(const CUtensorMap* maps, const lbmk::TbpMsArgs& a, int st
 }
 
 template <int KK, int NL>
-cudaError_t batch_tbp_nl(const lbmk::BatchTbpArgs& a, bool dirichlet, int ntiles, cudaStream_t s)
+cudaError_t batch_tbp_nl(const lbmk::BatchTbpArgs& a, int ntiles, cudaStream_t s)
 {
-    using G = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>;
-    void (*kern)(lbmk::BatchTbpArgs) =
-        dirichlet ? lbmk::batch_tbp_kernel<KK, NL, true> : lbmk::batch_tbp_kernel<KK, NL, false>;
+    using G = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E), true>;
+    void (*kern)(lbmk::BatchTbpArgs) = lbmk::batch_tbp_kernel<KK, NL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
     if (e != cudaSuccess) return e;
     return lbmh::launch_dependent(kern, dim3(ntiles), dim3(G::THREADS), G::SMEM, s, a);
 }
 
 template <int KK>
-cudaError_t batch_tbp_t(const lbmk::BatchTbpArgs& a, int steps, bool dirichlet, int ntiles, cudaStream_t s)
+cudaError_t batch_tbp_t(const lbmk::BatchTbpArgs& a, int steps, int ntiles, cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
     if constexpr (KK == lbmk::K_F32 || KK == lbmk::K_BF16 || KK == lbmk::K_F16) {
         constexpr int MX = lbmk::TbpGeom<(int)sizeof(typename lbmk::Fmt<KK>::E)>::NLMAX;
         switch (steps) {
-        case 2: if constexpr (MX >= 4) return batch_tbp_nl<KK, 2>(a, dirichlet, ntiles, s); break;
-        case 3: return batch_tbp_nl<KK, 3>(a, dirichlet, ntiles, s);
-        case 4: if constexpr (MX >= 4) return batch_tbp_nl<KK, 4>(a, dirichlet, ntiles, s); break;
+        case 2: if constexpr (MX >= 4) return batch_tbp_nl<KK, 2>(a, ntiles, s); break;
+        case 3: return batch_tbp_nl<KK, 3>(a, ntiles, s);
+        case 4: if constexpr (MX >= 4) return batch_tbp_nl<KK, 4>(a, ntiles, s); break;
         }
     }
     return cudaErrorNotSupported;
 }
 
-cudaError_t batch_tbp_step(const lbmk::BatchTbpArgs& a, int steps, bool dirichlet, int ntiles, cudaStream_t s)
+cudaError_t batch_tbp_step(const lbmk::BatchTbpArgs& a, int steps, int ntiles, cudaStream_t s)
 {
-    return batch_tbp_t<K>(a, steps, dirichlet, ntiles, s);
+    return batch_tbp_t<K>(a, steps, ntiles, s);
 }
 
 cudaError_t batch_occupancy(int* n)

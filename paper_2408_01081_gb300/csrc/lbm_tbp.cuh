@@ -237,12 +237,18 @@ struct TbpArgs {
 #define LBM_TBP_MIN2 2
 #endif
 
-template <int ES>
+// BATCH: the 16-bit formats take FP32's tile there.  Most tiles of a batch of small lattices touch an
+// edge, and the Dirichlet edge code spills 200 bytes at the 168 registers of five warps (three registers
+// sets per scheduler for two blocks); at four warps it has 203 and none.  48 steps, before this tile
+// and with it: 64 Dirichlet lattices of 256 x 512 in BF16 5069 -> 3639 us, periodic ones 3791 -> 3032.
+// Single lattices keep the wider tile: 8192^2 periodic 312 us a step against 371.
+template <int ES, bool BATCH = false>
 struct TbpGeom {
+    static constexpr bool TALL = ES == 4 || BATCH;
     static constexpr int NLMAX = (ES == 4) ? LBM_TBP_NL4 : 3;          // steps per pass at most
-    static constexpr int NW = (ES == 4) ? LBM_TBP_NW4 : LBM_TBP_NW2;
-    static constexpr int MIN_BLOCKS = (ES == 4) ? LBM_TBP_MIN4 : LBM_TBP_MIN2;
-    static constexpr int LEAD = (ES == 4) ? LBM_TBP_LEAD4 : LBM_TBP_LEAD2;   // columns a warp computes left and right of
+    static constexpr int NW = TALL ? LBM_TBP_NW4 : LBM_TBP_NW2;
+    static constexpr int MIN_BLOCKS = TALL ? LBM_TBP_MIN4 : LBM_TBP_MIN2;
+    static constexpr int LEAD = TALL ? LBM_TBP_LEAD4 : LBM_TBP_LEAD2;        // columns a warp computes left and right of
                                                                        // its output (even, at least NLMAX - 1)
     static constexpr int OUTW = 64 - 2 * LEAD;                         // output columns per warp
     static constexpr int OUT = NW * OUTW;
@@ -255,7 +261,7 @@ struct TbpGeom {
     static constexpr int LOFF = (ROW_BYTES + 127) / 128 * 128;         // columns wrapped below x = 0
     static constexpr int ROFF = LOFF + WRAP_BYTES;                     // columns wrapped beyond x = nx - 1
     static constexpr int STAGE_BYTES = ROFF + WRAP_BYTES;
-    static constexpr int NST = (ES == 4) ? LBM_TBP_NST4 : LBM_TBP_NST2;
+    static constexpr int NST = TALL ? LBM_TBP_NST4 : LBM_TBP_NST2;
     static constexpr int SMEM = NST * STAGE_BYTES + 128;
     static_assert(LEAD % 2 == 0 && LEAD >= NLMAX - 1, "columns lost per level");
     static_assert((WIN * ES) % 16 == 0 && WIN <= 256, "staged row geometry");
@@ -294,17 +300,16 @@ inline int tbp_pass(long long n, long long count, long long i)
 }
 
 // first column of the copy that holds the columns nx - LEAD - 1 .. nx - 1
-template <int ES>
-__device__ __forceinline__ int tbp_wrap_x(int nx) { return (nx - TbpGeom<ES>::LEAD - 1) & ~(16 / ES - 1); }
+template <typename G>
+__device__ __forceinline__ int tbp_wrap_x(int nx) { return (nx - G::LEAD - 1) & ~(G::WRAP / 2 - 1); }
 
 // the compute warps' part of a block.  EDGE: the tile touches x = 0 or x = nx - 1.
-template <int K, int NL, bool DIRICHLET, bool EDGE>
+template <typename G, int K, int NL, bool DIRICHLET, bool EDGE>
 __device__ __forceinline__ void tbp_compute(const TbpArgs& A, int X0, int y0, int y1, uint32_t sbase,
                                             unsigned long long* full_bar, unsigned long long* empty_bar,
                                             volatile int* abort_flag)
 {
     using E = typename Fmt<K>::E;
-    using G = TbpGeom<(int)sizeof(E)>;
     constexpr int NST = G::NST, WIN = G::WIN, HL = G::HL;
     constexpr uint32_t ES = sizeof(E), PL = WIN * sizeof(E);
     constexpr bool NEGOUT = (NL & 1) != 0;
@@ -324,7 +329,7 @@ __device__ __forceinline__ void tbp_compute(const TbpArgs& A, int X0, int y0, in
         for (int q = 0; q < 4; ++q) {
             int c = (xs - 1 + q) % nx;
             c = c < 0 ? c + nx : c;
-            const int m = c - X0 + HL, xl = tbp_wrap_x<(int)ES>(nx);
+            const int m = c - X0 + HL, xl = tbp_wrap_x<G>(nx);
             if (m >= 0 && m < WIN) {
                 eo[q] = m * ES;
                 es[q] = PL;
@@ -489,12 +494,10 @@ __device__ __forceinline__ void tbp_compute(const TbpArgs& A, int X0, int y0, in
 
 // One block's work: output columns X0 .. and rows y0 .. of the lattice A describes; maps[0]: its
 // row map (box WIN), maps[1]: the wrap map (box WRAP), as kernel parameters or in global memory.
-template <int K, int NL, bool DIRICHLET>
+template <typename G, int K, int NL, bool DIRICHLET>
 __device__ __forceinline__ void tbp_body(const CUtensorMap* map, const CUtensorMap* wmap, const TbpArgs& A, int X0,
                                          int y0)
 {
-    using E = typename Fmt<K>::E;
-    using G = TbpGeom<(int)sizeof(E)>;
     constexpr int NST = G::NST;
     extern __shared__ __align__(128) unsigned char tbp_smem_raw[];
     __shared__ __align__(8) unsigned long long full_bar[NST], empty_bar[NST];
@@ -524,7 +527,7 @@ __device__ __forceinline__ void tbp_body(const CUtensorMap* map, const CUtensorM
             lbmt::prefetch_map(map);
             const bool wrap = !DIRICHLET && edge && nx > G::OUT;   // columns beyond the row's ends, copied apart
             const uint32_t bytes = G::ROW_BYTES + (wrap ? 2 * G::WRAP_BYTES : 0);
-            const int xl = tbp_wrap_x<(int)sizeof(E)>(nx);
+            const int xl = tbp_wrap_x<G>(nx);
             lbmt::grid_dependency_wait();
             int j = 0, s = 0, ph = 1;
             for (; j < nin; ++j) {
@@ -562,8 +565,8 @@ __device__ __forceinline__ void tbp_body(const CUtensorMap* map, const CUtensorM
     if (warp >= nact) return;
     // the stores of the previous launch's last blocks may still read what this one overwrites
     lbmt::grid_dependency_wait();
-    if (edge) tbp_compute<K, NL, DIRICHLET, true>(A, X0, y0, y1, sbase, full_bar, empty_bar, &abort_flag);
-    else tbp_compute<K, NL, DIRICHLET, false>(A, X0, y0, y1, sbase, full_bar, empty_bar, &abort_flag);
+    if (edge) tbp_compute<G, K, NL, DIRICHLET, true>(A, X0, y0, y1, sbase, full_bar, empty_bar, &abort_flag);
+    else tbp_compute<G, K, NL, DIRICHLET, false>(A, X0, y0, y1, sbase, full_bar, empty_bar, &abort_flag);
 }
 
 template <int K, int NL, bool DIRICHLET>
@@ -572,13 +575,15 @@ __global__ void __launch_bounds__(TbpGeom<(int)sizeof(typename Fmt<K>::E)>::THRE
     tbp_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap wmap, TbpArgs A)
 {
     using G = TbpGeom<(int)sizeof(typename Fmt<K>::E)>;
-    tbp_body<K, NL, DIRICHLET>(&map, &wmap, A, blockIdx.x * G::OUT, blockIdx.y * A.rows);
+    tbp_body<G, K, NL, DIRICHLET>(&map, &wmap, A, blockIdx.x * G::OUT, blockIdx.y * A.rows);
 }
 
 // ---------------------------------------------------------------------------
-// Batches of lattices, three steps per pass (lbm_batch.cu, mode 2): one block per tile
-// {lattice, X0, y0} of a flat list, each running tbp_body on its lattice with that lattice's row
-// and wrap maps of the source arena.  The maps live in global memory, written by the host before
+// Batches of lattices, several steps per pass (lbm_batch.cu, mode 2): one block per tile
+// {lattice, X0, y0, Dirichlet} of a flat list, each running tbp_body on its lattice with that
+// lattice's row and wrap maps of the source arena.  Periodic and Dirichlet tiles share the launch: a
+// launch for each, one behind the other, left half the chip idle where either kind fills it less than
+// once (128 lattices of 64^2 in FP32, 48 steps: 941 us, 556 so).  The maps live in global memory, written by the host before
 // the launch; a lattice's planes sit at its element offset in each arena.
 // ---------------------------------------------------------------------------
 struct BatchLatT3 {
@@ -590,7 +595,7 @@ struct BatchLatT3 {
 };
 
 struct BatchTbpArgs {
-    const int4* tiles;          // {lattice, X0, y0, 0} per block
+    const int4* tiles;          // {lattice, X0, y0, 1 if Dirichlet} per block
     const BatchLatT3* lat;
     const CUtensorMap* maps;    // [lattice][arena][2]: row map, wrap map
     void* arenaA;
@@ -600,9 +605,9 @@ struct BatchTbpArgs {
     int* timeout;               // set when a bounded wait ran out
 };
 
-template <int K, int NL, bool DIRICHLET>
-__global__ void __launch_bounds__(TbpGeom<(int)sizeof(typename Fmt<K>::E)>::THREADS,
-                                  TbpGeom<(int)sizeof(typename Fmt<K>::E)>::MIN_BLOCKS)
+template <int K, int NL>
+__global__ void __launch_bounds__(TbpGeom<(int)sizeof(typename Fmt<K>::E), true>::THREADS,
+                                  TbpGeom<(int)sizeof(typename Fmt<K>::E), true>::MIN_BLOCKS)
     batch_tbp_kernel(BatchTbpArgs B)
 {
     using E = typename Fmt<K>::E;
@@ -623,7 +628,9 @@ __global__ void __launch_bounds__(TbpGeom<(int)sizeof(typename Fmt<K>::E)>::THRE
     A.timeout = B.timeout;
     A.withhold = -1;
     const CUtensorMap* m = B.maps + 2 * (2 * t.x + B.parity);
-    tbp_body<K, NL, DIRICHLET>(m, m + 1, A, t.y, t.z);
+    using G = TbpGeom<(int)sizeof(E), true>;
+    if (t.w) tbp_body<G, K, NL, true>(m, m + 1, A, t.y, t.z);
+    else tbp_body<G, K, NL, false>(m, m + 1, A, t.y, t.z);
 }
 
 }  // namespace lbmk
