@@ -92,24 +92,6 @@ __device__ __forceinline__ void wall_links(const StepArgs& A, const double* g, i
     }
 }
 
-// dt/2 times the body load at node (x, y), called by the whole warp for one row: lane r * 2 + c
-// computes coefficient (r, c) (R <= 16) into the warp's buffer cf, so the products of the row cost
-// two FP64 instructions per warp and each node is left with 2R fused multiply-adds
-__device__ __forceinline__ void warp_body_load(const StepArgs& A, const double* T, double hdt, double* cf, int x, int y,
-                                               double& hx, double& hy)
-{
-    const int l = threadIdx.x & 31;
-    __syncwarp();                                      // the previous row's coefficients have been read
-    if (l < 2 * A.R) cf[l] = body_coef(A, T, hdt, l >> 1, l & 1, y);
-    __syncwarp();
-    hx = hy = 0.0;
-    for (int r = 0; r < A.R; ++r) {
-        const double X = A.X[(long long)r * A.nx + x];
-        hx = fma(X, cf[2 * r], hx);
-        hy = fma(X, cf[2 * r + 1], hy);
-    }
-}
-
 // grid: (ceil(nx / SA_THREADS), ceil(ny / rows)), block SA_THREADS; block (cb, r) computes
 // the rows r * rows ... of column block cb, one after the other
 template <bool DIRICHLET, bool TRACK, bool FORCE, unsigned long long SPLIT>

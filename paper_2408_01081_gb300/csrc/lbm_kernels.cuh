@@ -296,6 +296,24 @@ __device__ __forceinline__ double body_coef(const StepArgs& A, const double* T, 
     return __dmul_rn(__dmul_rn(hdt, T[c * A.R + r]), A.Y[(long long)r * A.ny + y]);
 }
 
+// dt/2 times the body load at node (x, y), called by the whole warp for one row: lane r * 2 + c
+// computes coefficient (r, c) (R <= 16) into the warp's buffer cf, so the products of the row cost
+// two FP64 instructions per warp and each node is left with 2R fused multiply-adds
+__device__ __forceinline__ void warp_body_load(const StepArgs& A, const double* T, double hdt, double* cf, int x, int y,
+                                               double& hx, double& hy)
+{
+    const int l = threadIdx.x & 31;
+    __syncwarp();                                      // the previous row's coefficients have been read
+    if (l < 2 * A.R) cf[l] = body_coef(A, T, hdt, l >> 1, l & 1, y);
+    __syncwarp();
+    hx = hy = 0.0;
+    for (int r = 0; r < A.R; ++r) {
+        const double X = A.X[(long long)r * A.nx + x];
+        hx = fma(X, cf[2 * r], hx);
+        hy = fma(X, cf[2 * r + 1], hy);
+    }
+}
+
 #ifndef LBM_FX_FORCED_NI
 #define LBM_FX_FORCED_NI 5      // conversions of a node with body load on the integer pipes (0 .. 12)
 #endif
@@ -576,15 +594,12 @@ step_kernel(StepArgs A)
         if constexpr (SPLIT > 0 && sizeof(M) == 8 && !FORCING && !OMEGA) {
             collide_split<SPLIT>(f, a, b, U, o);
         } else if constexpr ((SPLIT & kSplitFixed) != 0 && sizeof(M) == 8 && FORCING && !OMEGA) {
-            // dt/2 times the body load in FP64, then the fixed-point node update with it
-            double hx = 0.0, hy = 0.0;
-            if (x < nx) {
-                for (int r = 0; r < A.R; ++r) {
-                    const double X = A.X[(long long)r * nx + x];
-                    hx = fma(X, body_coef(A, A.T, 0.5 * A.dt, r, 0, y), hx);
-                    hy = fma(X, body_coef(A, A.T, 0.5 * A.dt, r, 1, y), hy);
-                }
-            }
+            // dt/2 times the body load in FP64, then the fixed-point node update with it.  The row's
+            // coefficients once per warp: computed per node (six FP64 operations a term against the two
+            // left here) 2000 x 1500 nodes with four terms took 251 us a step, 199 so.
+            __shared__ double coef[8][32];
+            double hx, hy;
+            warp_body_load(A, A.T, 0.5 * A.dt, coef[threadIdx.x >> 5], x < nx ? x : nx - 1, y, hx, hy);
             collide_fixed_forced(f, hx, hy, a, b, U, o);
         } else {
 #pragma unroll
