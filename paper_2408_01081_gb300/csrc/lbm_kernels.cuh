@@ -432,7 +432,8 @@ __device__ __forceinline__ void wall_source(int i, int j, double gx, double gy, 
 // tracking in FP32, once enough warps are in flight.  Four nodes per thread took 204 registers, so 8
 // warps per SM loaded, waited and stored in turn, and read the body load's factors once per node: 2048 x
 // 1024 92 us, 4096^2 732 us.  Two nodes, 80 registers, 24 warps: 66 and 528 us (0.9 of the copy
-// bandwidth), 1021 x 515 28.9 -> 17.6; one node: 69 and 536, 16.6.
+// bandwidth), 1021 x 515 28.9 -> 17.6; one node: 69 and 536, 16.6.  The 16-bit formats' plain step on
+// large lattices keeps four nodes (step_v), at up to 128 registers.
 #ifndef LBM_STEP_MIN_BLOCKS_F32
 #define LBM_STEP_MIN_BLOCKS_F32 3       // blocks of 256
 #endif
@@ -442,7 +443,7 @@ __device__ __forceinline__ void wall_source(int i, int j, double gx, double gy, 
 
 template <int K, int V, bool DIRICHLET, bool FORCING, bool TRACK, bool OMEGA = false, unsigned long long SPLIT = 0>
 __global__ void __launch_bounds__(256, SPLIT > 0 ? LBM_SPLIT_MIN_BLOCKS
-                                       : sizeof(typename Fmt<K>::M) == 4 ? LBM_STEP_MIN_BLOCKS_F32 : 1)
+                                       : sizeof(typename Fmt<K>::M) == 4 ? (V == 4 ? 2 : LBM_STEP_MIN_BLOCKS_F32) : 1)
 step_kernel(StepArgs A)
 {
     using E = typename Fmt<K>::E;
