@@ -123,6 +123,10 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
  * steps_per_pass = 1 always uses one kernel per step. */
 lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t rows_per_block);
 
+/* Step kernels launched by this context so far (host counts), counts: [3]: kernels of one
+ * step, of one pass of several steps, and cooperative launches of all steps of an lbm_step call. */
+lbm_status lbm_step_launches(const lbm_ctx* ctx, int64_t* counts);
+
 /* How the multi-step kernels of lbm_set_step_fusion and the LBM_F64 step at split
  * levels 1 and 12 read their input (no counterpart in the paper; results are identical
  * either way).  1 (the default): each multi-step block's input rows are copied into
@@ -134,7 +138,8 @@ lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t row
  * kernel prefetches the next row there).  A bounded wait of the staged
  * kernel that runs out (about 2 s) makes the next lbm_synchronize return
  * LBM_ERR_TIMEOUT.  Mode 2 is a test hook: staged, but the producer withholds one
- * input row of every block, so that the compute warps' waits run out and the
+ * input row of every block (in the one-launch LBM_F64 form: a block never reports
+ * its steps to its neighbours), so that the waits run out and the
  * bounded-wait path is exercised (the state is then undefined).  Other modes
  * return LBM_ERR_ARG. */
 lbm_status lbm_set_staging(lbm_ctx* ctx, int32_t mode);

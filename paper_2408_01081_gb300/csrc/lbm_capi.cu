@@ -233,6 +233,7 @@ struct lbm_ctx {
                                  // the fixed-point node update, the default where it applies)
     int echeck_every = 0;        // energy monitor (lbm_set_energy_check): steps between checks, 0 = off
     int echeck_since = 0;        // steps since the last check
+    int64_t launches[3] = {0, 0, 0};   // step kernels launched: single steps, passes, runs of steps
     int staging = 1;             // 1 = rows staged in shared memory (tensor copies for the fused kernels,
                                  // asynchronous copies for the FP64 step), 0 = register loads
     int nyi = 0;                 // rows of the lattice's own (a slab: without its halo rows)
@@ -655,7 +656,7 @@ lbm_status lbm_synchronize(lbm_ctx* ctx)
     if (h) {
         LBM_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), ctx->s));
         LBM_CUDA(ctx, cudaStreamSynchronize(ctx->s));
-        return fail(ctx, LBM_ERR_TIMEOUT, "a bounded wait of the staged two-step kernel ran out; the state is "
+        return fail(ctx, LBM_ERR_TIMEOUT, "a bounded wait of a step kernel ran out; the state is "
                                           "undefined until re-initialised");
     }
     if (ctx->echeck_every > 0) {
@@ -691,6 +692,13 @@ lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t row
         ctx->tb_rows = rows_per_block;
         ctx->rows_set = true;
     }
+    return LBM_OK;
+}
+
+lbm_status lbm_step_launches(const lbm_ctx* ctx, int64_t* counts)
+{
+    if (!ctx || !counts) return LBM_ERR_ARG;
+    std::copy(ctx->launches, ctx->launches + 3, counts);
     return LBM_OK;
 }
 
@@ -920,6 +928,7 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
                     P.dst = ctx->buf[ctx->cur ^ 1];
                     cudaError_t e = ops->tbp_step(ctx->map[ctx->cur], P, k, ctx->p.bc == LBM_DIRICHLET, ctx->s);
                     if (e != cudaSuccess) return cuda_fail(ctx, e, "staged multi-step kernel");
+                    ++ctx->launches[1];
                     ctx->cur ^= 1;
                     ctx->m += k;
                     return LBM_OK;
@@ -962,6 +971,7 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
                     Q.dst = ctx->buf[ctx->cur ^ 1];
                     cudaError_t e = ops->tbpms_step(ctx->map[ctx->cur], Q, k, ctx->p.bc == LBM_DIRICHLET, ctx->s);
                     if (e != cudaSuccess) return cuda_fail(ctx, e, "staged multi-step kernel");
+                    ++ctx->launches[1];
                     ctx->cur ^= 1;
                     ctx->m += k;
                     n -= k;
@@ -973,13 +983,14 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
             T.dst = ctx->buf[ctx->cur ^ 1];
             cudaError_t e = ops->tb2_step(T, ctx->p.bc == LBM_DIRICHLET, tgrid, tblock, ctx->s);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "fused two-step kernel");
+            ++ctx->launches[1];
             ctx->cur ^= 1;
             ctx->m += 2;
             n -= 2;
         }
     }
     // small FP64 lattices at the fixed-point level: the steps in one cooperative launch
-    if (split && ctx->split == lbmh::STEP_SPLIT_FIXED && ctx->staging == 1 && !ctx->slab && !ctx->one_step &&
+    if (split && ctx->split == lbmh::STEP_SPLIT_FIXED && ctx->staging >= 1 && !ctx->slab && !ctx->one_step &&
         !ctx->rows_set && n >= 2 && n <= (1 << 30)) {
         const long long m = ctx->m;
         A.src = ctx->buf[ctx->cur];
@@ -988,8 +999,10 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
         A.Tf = nullptr;
         A.g = ctx->g ? ctx->g + m * 2 * ctx->nwall : nullptr;
         cudaError_t e = ops->step_multi(A, variant, (int)n, reinterpret_cast<unsigned int*>(ctx->scratch),
-                                        kRedBlocks * 60, reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot), ctx->s);
+                                        kRedBlocks * 60, reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot),
+                                        ctx->staging == 2 ? 0 : -1, ctx->s);
         if (e == cudaSuccess) {
+            ++ctx->launches[2];
             ctx->cur ^= (int)(n & 1);
             ctx->m = m + n;
             return LBM_OK;
@@ -1016,6 +1029,7 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
         }
         if (e == cudaErrorNotSupported) e = ops->step(A, variant, grid, block, ctx->s);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "step kernel");
+        ++ctx->launches[0];
         ctx->cur ^= 1;
         ctx->m = m + 1;
     }

@@ -105,10 +105,11 @@ struct KindOps {
     // cudaErrorNotSupported)
     cudaError_t (*step_staged)(const lbmk::StepArgs&, int variant, int rows, cudaStream_t s);
     // `steps` FP64 steps of a small lattice in one cooperative launch (split level 12; the variant's
-    // boundary, body load and tracking bits); flags: max_flags words of device scratch.
+    // boundary, body load and tracking bits); flags: max_flags words of device scratch; withhold: test
+    // hook, a block that never reports its steps (-1: none).
     // cudaErrorNotSupported for other formats and for lattices that one launch per step serves better
     cudaError_t (*step_multi)(const lbmk::StepArgs&, int variant, int steps, unsigned int* flags, int max_flags,
-                              int* timeout, cudaStream_t s);
+                              int* timeout, int withhold, cudaStream_t s);
     // several fused steps over the tiles of a batch (FP32 two to four, BF16 / FP16 three; others
     // return cudaErrorNotSupported): `ntiles` blocks
     cudaError_t (*batch_tbp_step)(const lbmk::BatchTbpArgs&, int steps, int ntiles, cudaStream_t s);

@@ -202,6 +202,7 @@ struct MultiArgs {
     int nblk, reach;       // blocks; neighbours on each side whose flags a step waits for
     unsigned int* flags;   // [nblk * MULTI_FLAG], zero at launch
     int* timeout;
+    int withhold;          // test hook: the block whose flag never rises (-1: none)
 };
 constexpr int MULTI_WARPS = 4;
 constexpr int MULTI_FLAG = 8;        // 32 bytes apart
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(32 * MULTI_WARPS, LBM_SA_FX_MIN_BLOCKS) multi_
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && (int)blockIdx.x != Q.withhold) {
             __threadfence();
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(Q.flags + blockIdx.x * MULTI_FLAG),
                          "r"((unsigned)(s + 1))

@@ -127,7 +127,7 @@ cudaError_t step_staged(const lbmk::StepArgs& a, int variant, int rows, cudaStre
 // (multi_f64_kernel); cudaErrorNotSupported where one launch per step is the better form
 template <bool D, bool T, bool F>
 cudaError_t step_multi_dtf(const lbmk::StepArgs& a, int steps, unsigned int* flags, int max_flags, int* timeout,
-                           cudaStream_t s)
+                           int withhold, cudaStream_t s)
 {
     if constexpr (K != lbmk::K_F64) {
         return cudaErrorNotSupported;
@@ -156,6 +156,7 @@ cudaError_t step_multi_dtf(const lbmk::StepArgs& a, int steps, unsigned int* fla
         q.reach = std::min((q.nseg + W - 1) / W + 2, q.nblk - 1);
         q.flags = flags;
         q.timeout = timeout;
+        q.withhold = withhold;
         e = cudaMemsetAsync(flags, 0, (size_t)q.nblk * lbmk::MULTI_FLAG * sizeof(unsigned int), s);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
@@ -177,17 +178,17 @@ cudaError_t step_multi_dtf(const lbmk::StepArgs& a, int steps, unsigned int* fla
 }
 
 cudaError_t step_multi(const lbmk::StepArgs& a, int variant, int steps, unsigned int* flags, int max_flags,
-                       int* timeout, cudaStream_t s)
+                       int* timeout, int withhold, cudaStream_t s)
 {
     switch (variant & 7) {
-    case 0: return step_multi_dtf<false, false, false>(a, steps, flags, max_flags, timeout, s);
-    case 1: return step_multi_dtf<true, false, false>(a, steps, flags, max_flags, timeout, s);
-    case 2: return step_multi_dtf<false, false, true>(a, steps, flags, max_flags, timeout, s);
-    case 3: return step_multi_dtf<true, false, true>(a, steps, flags, max_flags, timeout, s);
-    case 4: return step_multi_dtf<false, true, false>(a, steps, flags, max_flags, timeout, s);
-    case 5: return step_multi_dtf<true, true, false>(a, steps, flags, max_flags, timeout, s);
-    case 6: return step_multi_dtf<false, true, true>(a, steps, flags, max_flags, timeout, s);
-    default: return step_multi_dtf<true, true, true>(a, steps, flags, max_flags, timeout, s);
+    case 0: return step_multi_dtf<false, false, false>(a, steps, flags, max_flags, timeout, withhold, s);
+    case 1: return step_multi_dtf<true, false, false>(a, steps, flags, max_flags, timeout, withhold, s);
+    case 2: return step_multi_dtf<false, false, true>(a, steps, flags, max_flags, timeout, withhold, s);
+    case 3: return step_multi_dtf<true, false, true>(a, steps, flags, max_flags, timeout, withhold, s);
+    case 4: return step_multi_dtf<false, true, false>(a, steps, flags, max_flags, timeout, withhold, s);
+    case 5: return step_multi_dtf<true, true, false>(a, steps, flags, max_flags, timeout, withhold, s);
+    case 6: return step_multi_dtf<false, true, true>(a, steps, flags, max_flags, timeout, withhold, s);
+    default: return step_multi_dtf<true, true, true>(a, steps, flags, max_flags, timeout, withhold, s);
     }
 }
 

@@ -25,7 +25,7 @@ STATUS_NAMES = ["LBM_OK", "LBM_ERR_ARG", "LBM_ERR_CFL", "LBM_ERR_OOM", "LBM_ERR_
                 "LBM_ERR_TIMEOUT", "LBM_ERR_STATE"]
 
 # every symbol declared in include/lbm.h
-EXPORTS = ["lbm_create", "lbm_init", "lbm_set_relaxation", "lbm_set_step_fusion", "lbm_set_staging", "lbm_set_fp64_split", "lbm_set_energy_check", "lbm_set_forcing", "lbm_set_dirichlet", "lbm_set_dirichlet_separable", "lbm_step", "lbm_moments",
+EXPORTS = ["lbm_create", "lbm_init", "lbm_set_relaxation", "lbm_set_step_fusion", "lbm_step_launches", "lbm_set_staging", "lbm_set_fp64_split", "lbm_set_energy_check", "lbm_set_forcing", "lbm_set_dirichlet", "lbm_set_dirichlet_separable", "lbm_step", "lbm_moments",
            "lbm_energy", "lbm_error_sums", "lbm_get_populations", "lbm_set_populations", "lbm_check_finite",
            "lbm_time_step", "lbm_synchronize", "lbm_destroy", "lbm_last_error", "lbm_state_bytes",
            "lbm_save_state", "lbm_load_state", "lbm_energy_noalloc", "lbm_create_slab", "lbm_halo_bytes",
@@ -78,6 +78,7 @@ def load(path: Optional[str] = None):
         "lbm_set_forcing": ([vp, i32, dp, dp, dp, i64, i32], i32),
         "lbm_set_relaxation": ([vp, ctypes.c_double], i32),
         "lbm_set_step_fusion": ([vp, i32, i32], i32),
+        "lbm_step_launches": ([vp, ctypes.POINTER(i64)], i32),
         "lbm_set_staging": ([vp, i32], i32),
         "lbm_set_fp64_split": ([vp, i32], i32),
         "lbm_set_energy_check": ([vp, i32, ctypes.c_double], i32),
@@ -210,6 +211,13 @@ def lbm_init(ctx, U0, dU0dx, dU0dy, B0=None, u0=None):
 
 def lbm_set_step_fusion(ctx, steps_per_pass=2, rows_per_block=0):
     _check(ctx, load().lbm_set_step_fusion(ctx, int(steps_per_pass), int(rows_per_block)))
+
+
+def lbm_step_launches(ctx):
+    """Step kernels launched so far: (of one step, of one pass of several, of all steps of a call)."""
+    c = (ctypes.c_int64 * 3)()
+    _check(ctx, load().lbm_step_launches(ctx, c))
+    return tuple(c)
 
 
 def lbm_set_staging(ctx, mode=1):
@@ -476,6 +484,9 @@ class Lattice:
 
     def set_step_fusion(self, steps_per_pass=2, rows_per_block=0):
         lbm_set_step_fusion(self.ctx, steps_per_pass, rows_per_block)
+
+    def step_launches(self):
+        return lbm_step_launches(self.ctx)
 
     def set_staging(self, mode=1):
         lbm_set_staging(self.ctx, mode)

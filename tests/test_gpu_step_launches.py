@@ -1,0 +1,69 @@
+"""Which step kernels a call launches, and the bounded wait of the launch that takes all its steps."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _lattice(lbm, nx, ny, storage="f64", dirichlet=False, load=False):
+    lat = lbm.Lattice(nx, ny, 0.1, 0.1 / 3.2, 1.0, 0.6, dirichlet=dirichlet, storage=storage, track_displacement=load)
+    rng = np.random.default_rng(nx + ny)
+    if load:
+        lat.set_forcing(rng.standard_normal((2, nx)), rng.standard_normal((2, ny)), rng.standard_normal((60, 2, 2)) * 1e-3)
+    lat.set_populations(rng.standard_normal((4, 5, ny, nx)) * 1e-3, None)
+    return lat
+
+
+# the sizes of test_fp64_steps_in_one_launch_equal_single_launches
+@pytest.mark.parametrize("load", [False, True])
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 7), (31, 4), (32, 3), (33, 65), (64, 64), (100, 300), (700, 40),
+                                   (2049, 2), (9000, 3)])
+def test_small_fp64_lattices_take_one_launch(lbm, nx, ny, dirichlet, load):
+    lat = _lattice(lbm, nx, ny, dirichlet=dirichlet, load=load)
+    assert lat.step_launches() == (0, 0, 0)
+    lat.step(2)
+    lat.step(17)
+    assert lat.step_launches() == (0, 0, 2)
+    lat.step(1)                                  # a single step is one launch as it is
+    lat.set_step_fusion(1)
+    lat.step(4)
+    assert lat.step_launches() == (5, 0, 2)
+    lat.synchronize()
+    lat.close()
+
+
+def test_larger_lattices_take_a_launch_per_step_or_pass(lbm):
+    for nx, ny, storage, want in ((512, 256, "f64", (9, 0, 0)), (64, 64, "f32", (0, 3, 0)), (64, 64, "bf16", (0, 3, 0)),
+                                  (64, 64, "ms_bfp", (0, 3, 0))):
+        lat = _lattice(lbm, nx, ny, storage)
+        lat.step(9)
+        assert lat.step_launches() == want, (nx, ny, storage)
+        lat.synchronize()
+        lat.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(20, 3), (64, 64)])
+def test_one_launch_reports_a_wait_that_runs_out(lbm, nx, ny):
+    """Test hook: one block never reports its steps, so its neighbours' bounded waits run out (about
+    2 s), theirs with them; lbm_synchronize reports it once and the context stays usable."""
+    lat = _lattice(lbm, nx, ny)
+    lat.set_staging(2)
+    lat.step(5)
+    with pytest.raises(lbm.LbmError) as e:
+        lat.synchronize()
+    assert e.value.status == lbm.LBM_ERR_TIMEOUT
+    lat.synchronize()                            # the flag was cleared
+    lat.set_staging(1)
+    f = np.random.default_rng(1).standard_normal((4, 5, ny, nx)) * 1e-3
+    got = []
+    for one in (False, True):
+        if one:
+            lat.set_step_fusion(1)
+        lat.set_populations(f, None)
+        lat.step(6)
+        lat.synchronize()
+        got.append(lat.populations()[0])
+    assert lat.step_launches() == (6, 0, 2)
+    np.testing.assert_array_equal(got[0], got[1])
+    lat.close()
