@@ -117,8 +117,9 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
  * default: from the lattice's size, 2 to 96; for the staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
  * level 1, fewer on small lattices).  By default (this call not made, staging 1)
  * the steps of one lbm_step call on a small LBM_F64 lattice at split level 12 (up to
- * about 1800 segments of 32 columns of a row) run in one cooperative launch, with
- * the same results; a bounded wait of it that runs out (about 2 s) makes the next
+ * 1216 segments of 32 columns of a row) run in one cooperative launch, with
+ * the same results; it holds up to half of the chip until its last step, so a third
+ * lattice of that size on a stream of its own waits for one of the first two's call; a bounded wait of it that runs out (about 2 s) makes the next
  * lbm_synchronize return LBM_ERR_TIMEOUT.
  * steps_per_pass = 1 always uses one kernel per step. */
 lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t rows_per_block);

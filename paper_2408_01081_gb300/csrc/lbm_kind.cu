@@ -144,10 +144,13 @@ cudaError_t step_multi_dtf(const lbmk::StepArgs& a, int steps, unsigned int* fla
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lbmk::multi_f64_kernel<D, T, F>, 32 * W, 0);
         if (e != cudaSuccess) return e;
-        // up to three blocks per SM: beyond that a launch per step is as fast (us per step, this
-        // kernel / launches: 64^2 3.3 / 5.0, 128^2 3.4 / 5.2, 256^2 5.9 / 5.6; with body load and
+        // up to half of the blocks that fit on the chip (two per SM), so that two such lattices on streams
+        // of their own run side by side: one that takes more makes the others wait for its whole call (200
+        // steps, us, this kernel / a launch per step before: two of 208^2 2057 / 2645, but four 4112 / 3418,
+        // sixteen 16829 / 8671).  Alone, beyond three blocks per SM a launch per step is as fast (us per step,
+        // this kernel / launches: 64^2 3.3 / 5.0, 128^2 3.4 / 5.2, 256^2 5.9 / 5.6; with body load and
         // tracking 4.1 / 5.1, 4.3 / 6.3, 6.6 / 6.6)
-        const long long cap = std::min((long long)std::min(occ, 3) * sms, (long long)max_flags / lbmk::MULTI_FLAG) * W;
+        const long long cap = std::min((long long)std::min(occ, 4) * sms / 2, (long long)max_flags / lbmk::MULTI_FLAG) * W;
         if (cap < W || ntask > cap) return cudaErrorNotSupported;
         q.ntask = (int)ntask;
         q.nblk = (q.ntask + W - 1) / W;

@@ -34,7 +34,9 @@ def test_small_fp64_lattices_take_one_launch(lbm, nx, ny, dirichlet, load):
 
 
 def test_larger_lattices_take_a_launch_per_step_or_pass(lbm):
-    for nx, ny, storage, want in ((512, 256, "f64", (9, 0, 0)), (64, 64, "f32", (0, 3, 0)), (64, 64, "bf16", (0, 3, 0)),
+    # FP64: one launch where two such lattices fit on the chip together, 4 x 152 / 2 blocks of 4 segments
+    for nx, ny, storage, want in ((32, 1216, "f64", (0, 0, 1)), (32, 1217, "f64", (9, 0, 0)), (208, 208, "f64", (9, 0, 0)),
+                                  (512, 256, "f64", (9, 0, 0)), (64, 64, "f32", (0, 3, 0)), (64, 64, "bf16", (0, 3, 0)),
                                   (64, 64, "ms_bfp", (0, 3, 0))):
         lat = _lattice(lbm, nx, ny, storage)
         lat.step(9)
