@@ -99,10 +99,10 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out);
 lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const double* dU0dy,
                     const double* B0, const double* u0, int32_t on_device);
 
-/* Steps per pass over memory: 1, 2 or 3.  Without this call LBM_F32 takes up to four
- * steps per pass (results do not depend on the grouping), the other reduced formats
- * three and LBM_F64, whose step is bound by arithmetic as well as by memory, one.
- * With 2 lbm_step advances
+/* Steps per pass over memory: 1, 2 or 3; 0 (and a context without this call) is the
+ * default: up to four for LBM_F32 (results do not depend on the grouping), three for the
+ * other reduced formats, one for LBM_F64, whose step is bound by arithmetic as well as by
+ * memory.  With 2 lbm_step advances
  * pairs of steps with one kernel that keeps the intermediate state on chip (halving
  * the memory traffic per step), with 3 triples, whenever the lattice stores FP32 / BF16 / FP16
  * populations (or moment-space deviations, with staged rows: lbm_set_staging),
@@ -110,16 +110,18 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* U0, const double* dU0dx, const d
  * boundary is periodic or homogeneous Dirichlet; otherwise, and for an odd last
  * step, one kernel per step runs.  FP32 results are bit-identical to single
  * steps; 16-bit and moment-space results skip one rounding per pair and are more
- * accurate.  Three steps per kernel need staged rows (lbm_set_staging 1; with 0 pairs
+ * accurate.  More than two steps per kernel need staged rows (lbm_set_staging 1; with 0 pairs
  * run instead); a remainder of one or two steps runs as a single step or a pair
  * (LBM_F32: passes of equal length instead).
- * rows_per_block sets the rows each thread block streams through (0 keeps the
- * default: from the lattice's size, 2 to 96; for the staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
- * level 1, fewer on small lattices).  By default (this call not made, staging 1)
+ * rows_per_block sets the rows each thread block streams through until it is set again
+ * or steps_per_pass = 0 is (0 leaves it; the default is chosen from the lattice's size: 2 to
+ * 96, for the staged LBM_F64 step of lbm_set_staging up to 4 at split level 12 and up to 2 at
+ * level 1).  Unless steps_per_pass is 1 or rows_per_block set, and with staging 1,
  * the steps of one lbm_step call on a small LBM_F64 lattice at split level 12 (up to
  * 1216 segments of 32 columns of a row) run in one cooperative launch, with
  * the same results; it holds up to half of the chip until its last step, so a third
- * lattice of that size on a stream of its own waits for one of the first two's call; a bounded wait of it that runs out (about 2 s) makes the next
+ * lattice of that size on a stream of its own waits for one of the first two's call;
+ * a bounded wait of it that runs out (about 2 s) makes the next
  * lbm_synchronize return LBM_ERR_TIMEOUT.
  * steps_per_pass = 1 always uses one kernel per step. */
 lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t rows_per_block);

@@ -402,6 +402,18 @@ lbm_status choose_neq_scale(lbm_ctx* ctx, Launch launch)
     return LBM_OK;
 }
 
+// Steps per pass and rows per block of a context that was not told otherwise (lbm_set_step_fusion):
+// four steps in FP32, three in the other reduced formats (8192^2: each faster than fewer steps, and
+// fewer roundings to the storage format), one in FP64 and in slabs.  tb_rows serves the register
+// kernels; the staged ones size their blocks from the lattice (tbp_rows) unless rows_set.
+static void default_step_fusion(lbm_ctx* ctx)
+{
+    const int st = ctx->p.storage;
+    ctx->fuse = (st == LBM_F64 || ctx->slab) ? 1 : (st == LBM_F32) ? lbmk::TbpGeom<4>::NLMAX : 3;
+    ctx->tb_rows = (st == LBM_F64) ? 2 : (st == LBM_F32) ? 12 : 64;
+    ctx->one_step = ctx->rows_set = false;
+}
+
 extern "C" {
 
 lbm_status lbm_create(const lbm_params* p, lbm_ctx** out)
@@ -457,11 +469,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out)
     ctx->a = p->cK / c;
     ctx->b = p->cmu / c;
     ctx->nwall = 2 * (p->nx + p->ny);
-    // three steps per pass for every reduced format (measured faster than one or two steps for each
-    // of them at 8192^2, and fewer roundings to the storage format); rows per block measured best
-    // per format
-    ctx->fuse = (p->storage == LBM_F64) ? 1 : (p->storage == LBM_F32) ? lbmk::TbpGeom<4>::NLMAX : 3;
-    ctx->tb_rows = (p->storage == LBM_F64) ? 2 : (p->storage == LBM_F32) ? 12 : 64;
+    default_step_fusion(ctx);
     // FP64: the fixed-point node update by default (within FP64 accuracy, bound by memory
     // instead of the FP64 pipe); the exact integer-pipe sums where its multipliers do not fit
     ctx->split = (lbmfx::mul_ok(ctx->a) && lbmfx::mul_ok(ctx->b)) ? lbmh::STEP_SPLIT_FIXED : 1;
@@ -568,7 +576,7 @@ lbm_status lbm_create_slab(const lbm_params* p, int32_t y_begin, int32_t rows, l
     ctx->yo = lo;
     ctx->halo_lo = lo;
     ctx->halo_hi = hi;
-    ctx->fuse = 1;
+    default_step_fusion(ctx);
     return LBM_OK;
 }
 
@@ -684,10 +692,14 @@ lbm_status lbm_set_staging(lbm_ctx* ctx, int32_t mode)
 lbm_status lbm_set_step_fusion(lbm_ctx* ctx, int32_t steps_per_pass, int32_t rows_per_block)
 {
     LBM_CHECK_CTX(ctx);
-    if (steps_per_pass < 1 || steps_per_pass > 3 || rows_per_block < 0 || rows_per_block > 65535)
-        return fail(ctx, LBM_ERR_ARG, "steps_per_pass must be 1, 2 or 3 and rows_per_block in [0, 65535]");
-    ctx->fuse = steps_per_pass;
-    ctx->one_step = steps_per_pass == 1;
+    if (steps_per_pass < 0 || steps_per_pass > 3 || rows_per_block < 0 || rows_per_block > 65535)
+        return fail(ctx, LBM_ERR_ARG, "steps_per_pass must be 0, 1, 2 or 3 and rows_per_block in [0, 65535]");
+    if (steps_per_pass == 0) {
+        default_step_fusion(ctx);
+    } else {
+        ctx->fuse = steps_per_pass;
+        ctx->one_step = steps_per_pass == 1;
+    }
     if (rows_per_block > 0) {
         ctx->tb_rows = rows_per_block;
         ctx->rows_set = true;

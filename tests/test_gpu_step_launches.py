@@ -69,3 +69,40 @@ def test_one_launch_reports_a_wait_that_runs_out(lbm, nx, ny):
     assert lat.step_launches() == (6, 0, 2)
     np.testing.assert_array_equal(got[0], got[1])
     lat.close()
+
+
+@pytest.mark.parametrize("storage,nx,ny,default", [("f32", 300, 40, (0, 3, 0)), ("bf16", 300, 40, (0, 4, 0)),
+                                                   ("f64", 64, 64, (0, 0, 1)), ("f64", 512, 256, (12, 0, 0))])
+def test_zero_steps_per_pass_restores_the_default(lbm, storage, nx, ny, default):
+    lat = _lattice(lbm, nx, ny, storage)
+    lat.step(12)
+    assert lat.step_launches() == default
+    lat.set_step_fusion(1, 7)
+    lat.step(12)
+    before = lat.step_launches()
+    assert before == (default[0] + 12, default[1], default[2])
+    lat.set_step_fusion(0)
+    lat.step(12)
+    assert tuple(b - a for a, b in zip(before, lat.step_launches())) == default
+    for bad in (-1, 4):
+        with pytest.raises(lbm.LbmError):
+            lat.set_step_fusion(bad)
+    lat.synchronize()
+    lat.close()
+
+
+@pytest.mark.parametrize("rows", [2, 5, 64])
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+def test_default_passes_with_rows_given(lbm, storage, dirichlet, rows):
+    """FP32's four steps per pass (FP16's three) with the rows of a block given."""
+    got = []
+    for r in (0, rows):
+        lat = _lattice(lbm, 173, 131, storage, dirichlet)
+        lat.set_step_fusion(0, r)
+        lat.step(12)
+        assert lat.step_launches() == (0, {"f32": 3, "f16": 4}[storage], 0)
+        lat.synchronize()
+        got.append(lat.populations()[0])
+        lat.close()
+    np.testing.assert_array_equal(got[0], got[1])
