@@ -615,10 +615,10 @@ __global__ void __launch_bounds__(256) conv_wgrad_kernel(WgradArgs a)
         }
 }
 
-// Sum the split partials into dW (FP32) in a fixed order.  A block takes 32 consecutive elements;
-// its warps take every 8th split each (a 128-byte line per load) and their sums are added in warp
-// order.  One thread per element walked all splits before: 32 -> 32 channels has 9216 elements and
-// up to 600 splits, 36 blocks of dependent loads, 55 us for 19 MB; 9 us so.
+// Sum the split partials into dW (FP32) in a fixed order: launch_sum_splits chooses between two forms.
+// Few elements and many splits (32 -> 32 channels: 9216 and up to 600): a block takes 32 consecutive
+// elements; its warps take every 8th split each (a 128-byte line per load) and their sums are added in
+// warp order.  One thread per element would be 36 blocks of dependent loads (608 splits: 19 us, 6 so).
 __global__ void __launch_bounds__(256) sum_splits_kernel(const float* __restrict__ partial, int splits, long long n,
                                                          float* __restrict__ out, int beta)
 {
@@ -638,6 +638,28 @@ __global__ void __launch_bounds__(256) sum_splits_kernel(const float* __restrict
         for (int w = 1; w < 8; ++w) t += red[w][lane];
         out[i] = beta ? out[i] + t : t;
     }
+}
+
+// Up to 64 splits, or elements enough for the chip: a thread per element, in the order of the splits.  A
+// block per 32 elements is bound by the number of blocks there (589824 elements, us, by warps / so: 1 split
+// 12.4 / 4.2, 16 16.4 / 6.2, 152 72 / 57; 147456 elements, 64 splits 8.2 / 6.2; 27648, 64: 4.1 / 4.6).
+__global__ void __launch_bounds__(256) sum_splits_flat_kernel(const float* __restrict__ partial, int splits,
+                                                              long long n, float* __restrict__ out, int beta)
+{
+    const long long i = blockIdx.x * 256LL + threadIdx.x;
+    if (i >= n) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < splits; ++k) s += partial[(long long)k * n + i];
+    out[i] = beta ? out[i] + s : s;
+}
+
+void launch_sum_splits(const float* partial, int splits, long long n, float* out, int beta, cudaStream_t s)
+{
+    if (splits <= 64 || n >= 1 << 17)
+        sum_splits_flat_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(partial, splits, n, out, beta);
+    else
+        sum_splits_kernel<<<(unsigned)((n + 31) / 32), 256, 0, s>>>(partial, splits, n, out, beta);
 }
 
 // db[c] = sum_p dY[p][c] in two fixed-order passes.  Pass 1: block b sums the
@@ -1248,7 +1270,7 @@ lbm_status lbm_nn_conv_backward_weight(const float* dy, int32_t Cout, const floa
             return LBM_ERR_CUDA;
         const int splits = conv3_wgrad_tc_split(Cin, Cout, B, H, W).partials();
         const long long n = (long long)Cout * 9 * Cin;
-        sum_splits_kernel<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(static_cast<const float*>(workspace), splits, n, dw, beta);
+        launch_sum_splits(static_cast<const float*>(workspace), splits, n, dw, beta, st);
         g_conv_launches[2].fetch_add(1, std::memory_order_relaxed);
         return launch_status();
     }
@@ -1262,7 +1284,7 @@ lbm_status lbm_nn_conv_backward_weight(const float* dy, int32_t Cout, const floa
     dim3 grid((unsigned)((Cout + 63) / 64), (unsigned)(KS * KS * ((Cin + 63) / 64)), (unsigned)splits);
     conv_wgrad_kernel<<<grid, 256, 0, s>>>(a);
     const long long n = (long long)Cout * KS * KS * Cin;
-    sum_splits_kernel<<<(unsigned)((n + 31) / 32), 256, 0, s>>>(static_cast<const float*>(workspace), splits, n, dw, beta);
+    launch_sum_splits(static_cast<const float*>(workspace), (int)splits, n, dw, beta, s);
     return launch_status();
 }
 
