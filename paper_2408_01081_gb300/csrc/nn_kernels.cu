@@ -704,6 +704,9 @@ __global__ void bias_grad_partial_kernel(const float* __restrict__ dy, long long
 // the block's partial sum of the masked dy per channel (pass 1 of the bias gradient).  Bound by memory:
 // the mask alone is 12 bytes per element, the sums came in a second pass of 4 (29 + 28 us for 8 x 256 x
 // 256 x 32, 30 us so).  A thread keeps four adjacent channels (C a multiple of 4, at most 1024).
+// SUMS: sums a thread keeps.  One up to 256 channels; four beyond, where its chain of additions would be
+// two to four times as long (in one kernel with the other: 44 us there for its registers, 38 so).
+template <int SUMS>
 __global__ void __launch_bounds__(256) relu_bias_partial_kernel(float4* __restrict__ dy, const float4* __restrict__ y,
                                                                 long long P, int C4, long long ppb,
                                                                 float4* __restrict__ partial)
@@ -731,11 +734,11 @@ __global__ void __launch_bounds__(256) relu_bias_partial_kernel(float4* __restri
         add(u, v);
     };
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < rows && rows >= 4) {
+    if (SUMS == 1 && r < rows) {
 #pragma unroll 4
         for (long long p = p0 + r; p < p1; p += rows) take(p, s);
-    } else if (r < rows) {                        // more than 256 channels: four sums a thread, or its chain of
-        float4 s1 = s, s2 = s, s3 = s;            // additions would be two to four times as long
+    } else if (r < rows) {
+        float4 s1 = s, s2 = s, s3 = s;
         long long p = p0 + r;
         for (; p + 3 * rows < p1; p += 4 * rows) {
             take(p, s);
@@ -1319,8 +1322,9 @@ lbm_status lbm_nn_relu_bias_backward(float* dy, const float* y, int64_t P, int32
     }
     const int nblk = bias_grad_blocks(P, C);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    relu_bias_partial_kernel<<<nblk, 256, 0, s>>>(reinterpret_cast<float4*>(dy), reinterpret_cast<const float4*>(y), P,
-                                                  C / 4, bias_grad_ppb(P, C), static_cast<float4*>(workspace));
+    const auto kern = C <= 256 ? relu_bias_partial_kernel<1> : relu_bias_partial_kernel<4>;
+    kern<<<nblk, 256, 0, s>>>(reinterpret_cast<float4*>(dy), reinterpret_cast<const float4*>(y), P,
+                              C / 4, bias_grad_ppb(P, C), static_cast<float4*>(workspace));
     bias_grad_finish_kernel<<<C, 256, 0, s>>>(static_cast<const float*>(workspace), nblk, C, db);
     return launch_status();
 }
