@@ -108,7 +108,7 @@ struct lbm_batch {
     unsigned long long timeout_ns = 2000000000ull;
     unsigned int extra_arrivals = 0;
     bool own_stream = false;              // created here because the caller gave the legacy stream
-    // mode 2: three steps per pass with staged rows (FP32 / BF16 / FP16)
+    // mode 2: several steps per pass with staged rows (FP32 / BF16 / FP16)
     bool t3_ok = false;                   // row maps encoded and tile lists built
     int t3_rows = 0;                      // output rows per tile
     lbmk::BatchLatT3* d_lat3 = nullptr;
@@ -222,7 +222,6 @@ lbm_status setup_t3(lbm_batch* b)
         q.pitch = L.pitch;
         q.af = (float)L.a;
         q.bf = (float)L.b;
-        q.pad_ = 0;
         for (int y = 0; y < L.ny; y += b->t3_rows)
             for (int x = 0; x < L.nx; x += out) tiles[L.bc ? 1 : 0].push_back(make_int4(i, x, y, L.bc ? 1 : 0));
     }
@@ -855,7 +854,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, const char* cache_path)
         b->graph_steps = 2;
         tpr_mode[mode] = b->tpr_of_class;
     }
-    // mode 2 (three steps per pass, FP32 / 16 bits) and mode 3 (FP64 on staged rows) run over
+    // mode 2 (several steps per pass, FP32 / 16 bits) and mode 3 (FP64 on staged rows) run over
     // fixed tiles; mode 2's remainder steps use mode 0's widths
     for (int m = 2; m < 4; ++m) {
         if (!(m == 2 ? b->t3_ok : b->f64s_ok)) continue;

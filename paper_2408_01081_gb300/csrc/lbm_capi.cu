@@ -936,7 +936,6 @@ static lbm_status step_n(lbm_ctx* ctx, int64_t n)
                 P.timeout = reinterpret_cast<int*>(ctx->scratch + kTimeoutSlot);
                 P.withhold = ctx->staging == 2 ? 2 : -1;
                 auto pass = [&](int k) {
-                    P.src = ctx->buf[ctx->cur];
                     P.dst = ctx->buf[ctx->cur ^ 1];
                     cudaError_t e = ops->tbp_step(ctx->map[ctx->cur], P, k, ctx->p.bc == LBM_DIRICHLET, ctx->s);
                     if (e != cudaSuccess) return cuda_fail(ctx, e, "staged multi-step kernel");

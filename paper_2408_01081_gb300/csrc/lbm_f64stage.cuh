@@ -6,8 +6,8 @@
 // with 80 registers and three 256-thread blocks per SM, about a sixth of its warp
 // cycles go to that wait (long scoreboard) while the integer pipe, which shares the
 // bound of the split collision with the FP64 pipe, idles.  Here a block of 128 threads
-// owns 128 consecutive columns and walks down `rows` rows (the library passes 2 at level 1
-// and 4 at level 12), thread t computing column t of each row.  The copies of the next row are issued as soon as
+// owns 128 consecutive columns and walks down `rows` rows (the library passes up to 2 at level 1
+// and up to 4 at level 12, fewer on small lattices), thread t computing column t of each row.  The copies of the next row are issued as soon as
 // the current row has been read out of shared memory, so they are in flight during its
 // whole collision and occupy no registers.  Each thread copies exactly the 20 values its
 // own node pulls (f*_(1,0) from x - 1, f*_(-1,0) from x + 1, f*_(0,1) from y - 1,

@@ -3,21 +3,26 @@
 // adjacent columns per thread in packed FP32 arithmetic (fma.rn.f32x2 / add.rn.f32x2).  Every
 // packed operation rounds each half as the scalar one does and the operations are those of
 // collide() (lbm_kernels.cuh) up to exact sign changes, so FP32 results equal single steps.
+// (Packed products that are added are merged into one packed multiply-add; the update has none.)
 //
-// Block = NW compute warps + 1 producer warp over a tile of 60 NW output columns and `rows`
-// output rows.  The producer's elected lane streams the input rows y0 - NL .. y1 + NL - 1 of
-// all 20 planes, columns [X0 - HL, X0 + 60 NW + HL), into a ring of shared-memory stages, one
-// tensor copy per row (lbm_tma.cuh).  A lane of warp w owns the columns X0 - 2 + 60 w + 2 lane
+// Block = NW compute warps + 1 producer warp over a tile of OUT = NW OUTW output columns and `rows`
+// output rows (TbpGeom: a warp's 64 columns are OUTW = 64 - 2 LEAD stored ones and LEAD on each side
+// that feed them; 56 and 4 in FP32, 60 and 2 in the 16-bit formats' single lattices).  The producer's
+// elected lane streams the input rows y0 - NL .. y1 + NL - 1 of
+// all 20 planes, columns [X0 - HL, X0 + OUT + HL), into a ring of shared-memory stages, one
+// tensor copy per row (lbm_tma.cuh).  A lane of warp w owns the columns X0 - LEAD + OUTW w + 2 lane
 // and the next one.  Level 1, S1 = f*(t+dt) of row r, is pulled from the staged rows r-1, r,
 // r+1; level l + 1 of row r - l is pulled from level l's rows r-l-1 .. r-l+1, which stay in
 // registers (x-neighbours: one shuffle per component and direction for both columns); level NL
-// of row r - NL + 1 is stored by lanes 1..30.  Per level and node only what later rows still
+// of row r - NL + 1 is stored by lanes LEAD / 2 .. 31 - LEAD / 2.  Per level and node only what later rows still
 // read is kept: the shifted (1,0) and (-1,0) populations of the last row and the (0,1)
 // populations of the last two.
 //
-// What bounds it: instruction issue before, memory now.  One column per thread took 164 thread
+// What bounds it: instruction issue before, memory and latency now (FP32: DRAM 74 % busy, 40 % of the
+// issue slots, two warps per scheduler; BF16: 61 %, 56 %).  One column per thread took 164 thread
 // instructions per node and step in the three-step kernel it replaces (scalar arithmetic, a shuffle
-// per component and column, register copies of the kept rows); two columns take about 50.
+// per component and column, register copies of the kept rows); here it is 97 in FP32 and 106 in BF16,
+// the columns and rows around a tile included.
 // Measured at 8192^2 periodic: FP32 110k -> 154k MLUPS at four steps per pass (three: 117k, bound by
 // HBM at 53 B per node and step; five spill), 0.91 of the copy bandwidth at 40 B; BF16 158k -> 215k at
 // three, 0.85 of it at 26.7 B.  FP32: 3 compute warps, 2 blocks per SM, 232 registers (168 spill: 17k);
@@ -43,8 +48,8 @@
 
 namespace lbmk {
 
-// r modulo ny in [0, ny) for r within three rows of the lattice (the staged rows of the
-// three-step kernels): one wrap suffices unless ny = 2, where the remainder is taken
+// r modulo ny in [0, ny) for r within four rows of the lattice (the rows staged for up to four
+// steps): one wrap suffices unless ny is 2 or 3, where the remainder is taken
 __device__ __forceinline__ int wrap_row(int r, int ny)
 {
     if (r < 0) r += ny;
@@ -197,8 +202,7 @@ __device__ __forceinline__ void tbp_update(const TbpConst& C, const f32x2 (&x0)[
 }
 
 struct TbpArgs {
-    const void* src;       // f*(t) planes (only the row maps read them)
-    void* dst;             // f*(t + NL dt) planes
+    void* dst;             // f*(t + NL dt) planes; f*(t) is read through the row maps
     int nx, ny, pitch;
     long long plane;
     float af, bf;          // cK/c, cmu/c in FP32
@@ -563,7 +567,7 @@ __device__ __forceinline__ void tbp_body(const CUtensorMap* map, const CUtensorM
         return;
     }
     if (warp >= nact) return;
-    // the stores of the previous launch's last blocks may still read what this one overwrites
+    // the previous launch's last blocks may still read what this one overwrites
     lbmt::grid_dependency_wait();
     if (edge) tbp_compute<G, K, NL, DIRICHLET, true>(A, X0, y0, y1, sbase, full_bar, empty_bar, &abort_flag);
     else tbp_compute<G, K, NL, DIRICHLET, false>(A, X0, y0, y1, sbase, full_bar, empty_bar, &abort_flag);
@@ -591,7 +595,6 @@ struct BatchLatT3 {
     long long plane;       // elements per plane = ny * pitch
     int nx, ny, pitch;
     float af, bf;          // cK / c, cmu / c in FP32
-    int pad_;
 };
 
 struct BatchTbpArgs {
@@ -616,7 +619,6 @@ __global__ void __launch_bounds__(TbpGeom<(int)sizeof(typename Fmt<K>::E), true>
     E* a = static_cast<E*>(B.arenaA) + L.off;
     E* b = static_cast<E*>(B.arenaB) + L.off;
     TbpArgs A;
-    A.src = B.parity ? b : a;
     A.dst = B.parity ? a : b;
     A.nx = L.nx;
     A.ny = L.ny;

@@ -17,11 +17,13 @@
 // seams.  Without them the 16-bit roundings part from there on within a few hundred steps: the fields
 // of a run differ by as much as the format's own error (1e-5).  About a tenth more instructions.
 //
-// What bounds it: instruction issue (decoding, rebuilding, encoding).  One column per thread took
-// about 470 thread instructions per node and step in block floating point at 3 blocks per SM.
-// Measured, block floating point, 300 steps on 4095 x 4001 from the initial fields to the moments:
-// 104.7 ms before (three steps per pass, one column per thread), 67.4 ms now; the floor at 33.3 bytes
-// per node and step is 24 ms.
+// What bounds it: latency, with at most two compute warps per scheduler (236 to 255 registers): 47 % of
+// the issue slots and 32 % of DRAM in block floating point.  One column per thread took about 470 thread
+// instructions per node and step there at 3 blocks per SM, two columns take 217.  Measured, block
+// floating point, 300 steps on 4095 x 4001 from the initial fields to the moments: 104.7 ms before
+// (three steps per pass, one column per thread), 67.5 ms now; the floor at 33.3 bytes per node and step
+// is 24 ms.  30 steps of 4095 x 4001, one column per thread / now: BF16 and FP16 deviations 6.47 / 4.97 ms,
+// Dirichlet 6.97 / 5.53, Dirichlet block floating point 9.57 / 7.17.
 #pragma once
 
 #include "lbm_ms.cuh"

@@ -417,7 +417,7 @@ def evaluate(sur, chunk, batch=16, act_bf16=False):
 
 
 def _solver_mode(storage):
-    """The fastest batch mode of a storage format: three steps per pass (mode 2) for the
+    """The fastest batch mode of a storage format: several steps per pass (mode 2) for the
     population formats in FP32 / 16 bits (bit-identical to single steps in FP32), one step per
     launch on staged rows (mode 3) for FP64."""
     return 2 if storage in ("f32", "bf16", "f16") else 3 if storage == "f64" else 0
