@@ -242,8 +242,8 @@ struct TbpArgs {
 #endif
 
 // BATCH: the 16-bit formats take FP32's tile there.  Most tiles of a batch of small lattices touch an
-// edge, and the Dirichlet edge code spills 200 bytes at the 168 registers of five warps (three registers
-// sets per scheduler for two blocks); at four warps it has 203 and none.  48 steps, before this tile
+// edge, and the Dirichlet edge code spills 180 bytes at the 168 registers of five warps (two blocks put
+// three warps on a scheduler); at four warps it has 203 and none.  48 steps, before this tile
 // and with it: 64 Dirichlet lattices of 256 x 512 in BF16 5069 -> 3639 us, periodic ones 3791 -> 3032.
 // Single lattices keep the wider tile: 8192^2 periodic 312 us a step against 371.
 template <int ES, bool BATCH = false>
@@ -349,6 +349,15 @@ __device__ __forceinline__ void tbp_compute(const TbpArgs& A, int X0, int y0, in
     const bool wl = EDGE && DIRICHLET && xs == 0;                        // lower column on the left wall
     const bool wr0 = EDGE && DIRICHLET && xs == nx - 1, wr1 = EDGE && DIRICHLET && xs + 1 == nx - 1;
 
+    // where this lane's pulled (1,0) population of the lower column and its two (-1,0) ones sit in the
+    // staged row, from its own column on; on a Dirichlet wall, with BYADDR, the node's own opposite
+    // populations (a missing link is D f* of the opposite direction, D = (-1, -1, 1, 1, 1)).  In the
+    // 16-bit formats that saves the second loads (BF16 Dirichlet, us a step: 2048^2 33.4 -> 31.1, 2500 x
+    // 5000 93 -> 80, 8192^2 334 -> 316); in FP32 the offsets spill at four steps (4095 x 4001: 114 -> 120).
+    constexpr bool BYADDR = EDGE && DIRICHLET && ES == 2;
+    const uint32_t wo0 = BYADDR && wl ? 10 * PL : 0u - ES, wo2 = BYADDR && wr0 ? 0u : 10 * PL + ES;
+    const uint32_t wo3 = BYADDR && wr1 ? ES : 10 * PL + 2 * ES;
+
     // level l + 1 reads: s0 / s2 the pulled (1,0) / (-1,0) populations of its row, k1 the (0,1)
     // populations of the row below, c1 those of its own row (the next row's k1)
     f32x2 s0[NL - 1][5], s2[NL - 1][5], k1[NL - 1][5], c1[NL - 1][5];
@@ -386,15 +395,26 @@ __device__ __forceinline__ void tbp_compute(const TbpArgs& A, int X0, int y0, in
                 }
             } else {
                 const uint32_t c = st_c + own;
+                uint32_t a1 = st_m + own + 5 * PL, a3 = st_p + own + 15 * PL;
+                if (BYADDR && r == 0) a1 = c + 15 * PL;
+                if (BYADDR && r == ny - 1) a3 = c + 5 * PL;
 #pragma unroll
                 for (int k = 0; k < 5; ++k) {
-                    x0[k] = pk(Fmt<K>::ld(lbmt::lds<E>(c + k * PL - ES)), Fmt<K>::ld(lbmt::lds<E>(c + k * PL)));
-                    x2[k] = pk(Fmt<K>::ld(lbmt::lds<E>(c + (10 + k) * PL + ES)),
-                               Fmt<K>::ld(lbmt::lds<E>(c + (10 + k) * PL + 2 * ES)));
-                    x1[k] = Pair<K>::lds(st_m + own + (5 + k) * PL);
-                    x3[k] = Pair<K>::lds(st_p + own + (15 + k) * PL);
+                    float l0 = Fmt<K>::ld(lbmt::lds<E>(c + wo0 + k * PL)), l2 = Fmt<K>::ld(lbmt::lds<E>(c + wo2 + k * PL));
+                    float h2 = Fmt<K>::ld(lbmt::lds<E>(c + wo3 + k * PL));
+                    x1[k] = Pair<K>::lds(a1 + k * PL);
+                    x3[k] = Pair<K>::lds(a3 + k * PL);
+                    if (BYADDR && k < 2) {
+                        if (wl) l0 = -l0;
+                        if (wr0) l2 = -l2;
+                        if (wr1) h2 = -h2;
+                        if (r == 0) x1[k] = neg2(x1[k]);
+                        if (r == ny - 1) x3[k] = neg2(x3[k]);
+                    }
+                    x0[k] = pk(l0, Fmt<K>::ld(lbmt::lds<E>(c + k * PL)));
+                    x2[k] = pk(l2, h2);
                 }
-                if (EDGE && DIRICHLET) {
+                if (EDGE && DIRICHLET && !BYADDR) {
                     // missing links: D f* of the opposite direction at the node, D = (-1, -1, 1, 1, 1)
 #pragma unroll
                     for (int k = 0; k < 5; ++k) {
