@@ -51,7 +51,7 @@ STEPS_PER_PASS = {"f64": 1, "f32": 4, "bf16": 3, "f16": 3, "ms_bf16": 3, "ms_f16
 # from one ncu capture of this benchmark's own 8192^2 workload, averaged over its launches; no
 # scaling), valid only while the kernel sources hash to "sha256".  "<fmt>_fused<k>" is one launch
 # of k steps, "f64_pipe" the FP64 step with every operation on the FP64 pipe.
-TRAFFIC_CAPTURE = {"sha256": "4c4e1cbe92af584ddb16528bc5746b82cf1a4f63640e43faedf7d9ba19f24793",
+TRAFFIC_CAPTURE = {"sha256": "e99ccb988c3b8cccf4bd3a16bf5cc5fd12a56f8def5e3071775e3291fb28396a",
                    "nodes": 8192 * 8192,
                    "bytes_per_node": {"f64": 319.23, "f64_ieee": 322.73, "f64_pipe": 319.26, "f32_fused4": 172.90,
                                       "bf16_fused3": 82.60, "f16_fused3": 82.62, "ms_bf16_fused3": 103.93,
@@ -67,7 +67,7 @@ KERNEL_SOURCES = ["paper_2408_01081_gb300/csrc/lbm_kernels.cuh", "paper_2408_010
 # valid only while the kernel sources hash to "sha256".  Each SM issues 64 ALU-pipe and 2
 # FP64-pipe thread instructions per clock, so one node needs at least
 # max(alu / 64, fp64 / 2) SM clocks: the arithmetic roof of this kernel.
-PIPE_CAPTURE = {"sha256": "4c4e1cbe92af584ddb16528bc5746b82cf1a4f63640e43faedf7d9ba19f24793",
+PIPE_CAPTURE = {"sha256": "e99ccb988c3b8cccf4bd3a16bf5cc5fd12a56f8def5e3071775e3291fb28396a",
                 "alu_per_node": 586.8, "fp64_per_node": 20.0, "fma_per_node": 189.3}
 ALU_LANES_PER_SM, FP64_LANES_PER_SM, N_SM = 64, 2, 152
 
